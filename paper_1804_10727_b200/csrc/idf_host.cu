@@ -45,14 +45,12 @@ struct LayerPlan {
     TcPlan tc_pool;                         // plan of the launches that also emit the following max-pool's rows
     alignas(64) unsigned char w_map_pool[128];
     long long tc_launches = 0;
-    // thin layers (the whole receptive field of an output position in one shared-memory row): a kernel of its own for
-    // the rows a block determines completely
     std::vector<unsigned char> wq_packed;      // int nets, Cin % 4 == 0: [Kh][Kw][Cin/4][Cout] words of four int8 (all-layers launch)
     size_t wq_off = 0;
-    ThinPlan thin;
-    std::vector<unsigned char> wthin_packed;   // [Cout][row bytes] in the activation type, zero padded
-    size_t wthin_off = 0;
-    alignas(64) unsigned char w_map_thin[128];
+    WinPlan win;                               // thin layers: the window kernel (win.ok)
+    std::vector<unsigned char> wwin_packed;    // its banded weight matrix
+    size_t wwin_off = 0;
+    alignas(64) unsigned char w_map_win[128];
     // x-unfold in front of the tensor-core kernel (thin or x-strided layers): the Kw taps of every
     // output position are laid side by side as kpad channels, the conv then has Kw = 1, stride_x = 1
     int unfold = 0, kpad = 0, in_cap_rows = 0;
@@ -224,20 +222,9 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
         a.ring_rows = P.ring_rows; a.in_elem = P.in_elem; a.out_elem = P.out_elem;
         a.r0 = r0; a.r1 = r1; a.o_begin = o_begin; a.o_end = o_end; a.done_end = done_end;
         ce = cudaErrorNotSupported;
-        if (P.thin.ok && !P.use_sparse && n_in > 0) {
-            // rows not begun by an earlier block (first tap row o*stride - pad >= r0) and completed by this one: the
-            // thin-layer kernel computes them from the block's rows alone; the others exchange state with the ring
-            long long int_begin = r0 > 0 ? (r0 + P.l.pad + P.l.stride - 1) / P.l.stride : o_begin;
-            if (int_begin < o_begin) int_begin = o_begin;
-            const long long int_end = done_end;
-            if (int_end - int_begin >= 4) {
-                ce = launch_conv_thin(a, P.thin, net->dtype, P.w_map_thin, int_begin, int_end, status, net->stream);
-                if (ce == cudaSuccess) {
-                    net->launches += 1;
-                    P.tc_launches += 1;
-                    ce = launch_conv_edges(a, net->dtype, int_begin, int_end, net->stream);
-                }
-            }
+        if (P.win.ok && n_in > 0) {
+            ce = launch_conv_win(a, P.win, net->dtype, P.w_map_win, P.use_sparse, net->stream);
+            if (ce == cudaSuccess) P.tc_launches += 1;
         }
         if (ce == cudaErrorNotSupported && P.tc.ok && !P.use_sparse && n_in > 0) {
             ConvArgs t = a;
@@ -831,7 +818,18 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
             const size_t es = spec->dtype == IDF_I8_I32 ? 1 : 2;
             const int taps = l.kh * l.kw;
             const bool pool_next = i + 1 < spec->n_layers && spec->layers[i + 1].kind == IDF_MAXPOOL2;
-            if (tc_allowed && tc_make_plan(spec->dtype, net->n_streams, w, P.out_w, l.cin, l.cout, l.kh, l.kw,
+            // A thin layer (at most 128 bytes of receptive field) takes the window kernel, also where it reports its input
+            // events, unless its events are to be scattered one by one (IDF_PATH_SPARSE) or the max-pool behind it is better
+            // folded into the row-ring kernel's launch.
+            const bool win_allowed = !(debug_flags() & IDF_DEBUG_NO_TENSOR_CORES) && spec->dtype != IDF_F32 && !net->eager &&
+                                     l.path != IDF_PATH_SPARSE && (size_t)taps * l.cin * es <= 128 &&
+                                     (!P.use_sparse || (w > 1 && l.stride == 1));
+            const bool prefer_thin = (debug_flags() & IDF_DEBUG_PREFER_THIN) != 0;
+            if (win_allowed && (!pool_next || P.use_sparse || prefer_thin) &&
+                win_make_plan(spec->dtype, net->n_streams, P.out_w, l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, w == 1, &P.win)) {
+                P.wwin_packed.resize(P.win.w_bytes);
+                win_pack_weights(P.win, spec->dtype, weights[i], l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, P.wwin_packed.data());
+            } else if (tc_allowed && tc_make_plan(spec->dtype, net->n_streams, w, P.out_w, l.cin, l.cout, l.kh, l.kw,
                                            w == 1 ? 1 : l.stride, P.ring_rows, (int)elem_size(P.out_elem), 0, &P.tc)) {
                 if (pool_next)
                     tc_make_plan(spec->dtype, net->n_streams, w, P.out_w, l.cin, l.cout, l.kh, l.kw, w == 1 ? 1 : l.stride,
@@ -862,20 +860,6 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                                    (const unsigned char*)weights[i] + (((size_t)co * l.kh + ky) * l.kw * l.cin) * es,
                                    (size_t)l.kw * l.cin * es);
                 }
-            }
-            // A layer whose whole receptive field fits one 128-byte row gets the thin-layer kernel where the row-ring kernel
-            // has no good form for it: 1D nets (behind an x-unfold pass every tap row would carry Cin values padded to a
-            // K step: audio1d's first layer 1.68 -> 0.84 ms) and shapes it cannot take at all.  2D layers with kx taps stay
-            // with x-unfold + row ring (vgg2d conv1: 0.19 ms against 0.52 ms: building 27-value rows element by element
-            // costs more than the unfold pass saves).
-            const bool prefer_thin = (debug_flags() & IDF_DEBUG_PREFER_THIN) != 0;
-            if (tc_allowed && ((P.unfold && (w == 1 || prefer_thin)) || !P.tc.ok) && !(pool_next && P.tc_pool.ok) &&
-                thin_make_plan(spec->dtype, net->n_streams, P.out_w, l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride,
-                               (int)elem_size(P.out_elem), &P.thin)) {
-                P.wthin_packed.assign((size_t)l.cout * P.thin.swb, 0);
-                for (int co = 0; co < l.cout; ++co)
-                    memcpy(P.wthin_packed.data() + (size_t)co * P.thin.swb, (const unsigned char*)weights[i] + (size_t)co * taps * l.cin * es,
-                           (size_t)taps * l.cin * es);
             }
             if (spec->dtype == IDF_I8_I32 && l.cin % 4 == 0) {
                 P.wq_packed.resize((size_t)taps * l.cin * l.cout);
@@ -997,7 +981,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
         P.w_off = off; off = align_up(off + P.w_packed.size());
         P.b_off = off; off = align_up(off + P.b_packed.size());
         P.wtc_off = off; off = align_up(off + P.wtc_packed.size(), 1024);
-        P.wthin_off = off; off = align_up(off + P.wthin_packed.size(), 1024);
+        P.wwin_off = off; off = align_up(off + P.wwin_packed.size(), 1024);
         P.wq_off = off; off = align_up(off + P.wq_packed.size());
     }
     net->state_region_off = off;
@@ -1103,9 +1087,9 @@ int idf_stream_open(idf_net* net, void* d_workspace, size_t workspace_bytes, voi
         }
         if (!P.wq_packed.empty() && e == cudaSuccess)
             e = cudaMemcpyAsync(net->ws + P.wq_off, P.wq_packed.data(), P.wq_packed.size(), cudaMemcpyHostToDevice, net->stream);
-        if (!P.wthin_packed.empty() && e == cudaSuccess) {
-            e = cudaMemcpyAsync(net->ws + P.wthin_off, P.wthin_packed.data(), P.wthin_packed.size(), cudaMemcpyHostToDevice, net->stream);
-            if (thin_encode_weights(P.thin, net->dtype, net->ws + P.wthin_off, P.l.cout, P.w_map_thin) != 0) P.thin.ok = 0;
+        if (!P.wwin_packed.empty() && e == cudaSuccess) {
+            e = cudaMemcpyAsync(net->ws + P.wwin_off, P.wwin_packed.data(), P.wwin_packed.size(), cudaMemcpyHostToDevice, net->stream);
+            if (win_encode_weights(P.win, net->dtype, net->ws + P.wwin_off, P.w_map_win) != 0) P.win.ok = 0;
         }
     }
     if (e != cudaSuccess) { net->phase = CREATED; return fail(IDF_ERR_CUDA, "stream_open: %s", cudaGetErrorString(e)); }

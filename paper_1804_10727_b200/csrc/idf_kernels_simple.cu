@@ -217,28 +217,6 @@ static cudaError_t launch_rows(const ConvArgs& a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <typename TI, typename TW, typename TS, typename TO>
-static cudaError_t launch_edges_t(const ConvArgs& a, long long skip_begin, long long skip_end, cudaStream_t st)
-{
-    const long long total = (long long)a.ring_rows * a.S * a.Wout * a.Cout;
-    if (total == 0 || a.o_end <= a.o_begin) return cudaSuccess;
-    long long blocks = (total + 255) / 256;
-    if (blocks > 148LL * 64) blocks = 148LL * 64;
-    conv_rows_kernel<TI, TW, TS, TO><<<(unsigned)blocks, 256, 0, st>>>(a, skip_begin, skip_end, (unsigned)blocks);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_conv_edges(const ConvArgs& a, int dtype, long long skip_begin, long long skip_end, cudaStream_t st)
-{
-    if (dtype == 0) return launch_edges_t<float, float, float, float>(a, skip_begin, skip_end, st);
-    if (dtype == 1) {
-        if (a.in_elem != E_BF16) return cudaErrorInvalidValue;
-        if (a.out_elem == E_BF16) return launch_edges_t<__nv_bfloat16, float, float, __nv_bfloat16>(a, skip_begin, skip_end, st);
-        return launch_edges_t<__nv_bfloat16, float, float, float>(a, skip_begin, skip_end, st);
-    }
-    return launch_edges_t<int8_t, int8_t, int, int8_t>(a, skip_begin, skip_end, st);
-}
-
 cudaError_t launch_conv_simple(const ConvArgs& a, int dtype, cudaStream_t st)
 {
     if (dtype == 0) return launch_rows<float, float, float, float>(a, st);
