@@ -113,23 +113,15 @@ __device__ __forceinline__ void finalise_chunk(const uint32_t (&v)[W], bool emit
                                                const TS* bias_c, const StageSink& sink, uint32_t col_byte, int out_elem,
                                                int relu, int shift, const PoolCtx& pc, bool state_ok)
 {
-    TS acc[W];
-#pragma unroll
-    for (int j = 0; j < W; ++j) acc[j] = DT == 1 ? (TS)__uint_as_float(v[j]) : (TS)(int)v[j];
     if (!emit) {
 #pragma unroll
-        for (int j8 = 0; j8 < W / 8; ++j8) {
-            uint32_t t[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) t[j] = DT == 1 ? __float_as_uint((float)acc[8 * j8 + j]) : (uint32_t)(int)acc[8 * j8 + j];
-            st_global_v8(rp + 8 * j8, t);
-        }
+        for (int j8 = 0; j8 < W / 8; ++j8) st_global_v8(rp + 8 * j8, *(const uint32_t(*)[8])(v + 8 * j8));
         return;
     }
     if (DT == 1) {
         float f[W];
 #pragma unroll
-        for (int j = 0; j < W; ++j) f[j] = (float)acc[j];
+        for (int j = 0; j < W; ++j) f[j] = __uint_as_float(v[j]);
         if (bias_c) {
 #pragma unroll
             for (int j4 = 0; j4 < W / 4; ++j4) {
@@ -161,35 +153,8 @@ __device__ __forceinline__ void finalise_chunk(const uint32_t (&v)[W], bool emit
             deliver<W, 1>(fw, sink, col_byte, pc, state_ok);
         }
     } else {
-        // Requantisation through the saturating packs (two values per instruction): the shift, then ReLU and clamp as the
-        // pack's bounds.  A negative sum gives (t + rnd) >> shift <= 0, so the unsigned pack's lower bound is the ReLU; the
-        // upper bound 127 and the symmetric lower bound -127 are one byte-wise min / max per four values.  The kernel's int8
-        // layers are bound by this arithmetic, not by the tensor pipe (a scalar clamp and shift-or packing cost eight
-        // instructions per value instead of two).
         uint32_t pk[W / 4];
-        const int rnd = shift > 0 ? 1 << (shift - 1) : 0;
-#pragma unroll
-        for (int j = 0; j < W / 4; ++j) {
-            int t[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[u] = (int)acc[4 * j + u] + rnd;
-            if (bias_c) {
-                const int4 b4 = ((const int4*)bias_c)[j];
-                t[0] += b4.x; t[1] += b4.y; t[2] += b4.z; t[3] += b4.w;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[u] >>= shift;
-            uint32_t hi2;
-            if (relu) {
-                asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
-                asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(pk[j]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
-                pk[j] = __vminu4(pk[j], 0x7f7f7f7fu);
-            } else {
-                asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
-                asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(pk[j]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
-                pk[j] = __vmaxs4(pk[j], 0x81818181u);
-            }
-        }
+        pack_i8<W>(v, (const int*)bias_c, relu, shift, pk);
         deliver<W / 4, 2>(pk, sink, col_byte, pc, state_ok);
     }
 }

@@ -23,8 +23,8 @@
 // CTA per SM.  Layers that report their input events (Eq. 3: non-zero components) count them while the runs pass by.
 //
 // Measured on B200, against the kernels that served these layers before (event scatter on CUDA cores; one im2col row per
-// output; x-unfold pass + row ring): 2 -> 32 channels int8, 2048 streams of 256-wide rows, 256 rows 5.46 -> 2.35 ms;
-// 1 -> 16 int8, 4096 28x28 images 0.287 -> 0.040 ms; 1 -> 32 bf16 1D, 1024 streams of 16000 samples 0.54 -> 0.16 ms;
+// output; x-unfold pass + row ring): 2 -> 32 channels int8, 2048 streams of 256-wide rows, 256 rows 5.46 -> 1.75 ms;
+// 1 -> 16 int8, 4096 28x28 images 0.287 -> 0.033 ms; 1 -> 32 bf16 1D, 1024 streams of 16000 samples 0.54 -> 0.16 ms;
 // 3 -> 64 bf16, 64 streams of 224-wide rows, 112 rows 0.094 -> 0.071 ms.
 #include "../../include/idf.h"
 #include "idf_ptx.h"
@@ -156,36 +156,6 @@ __device__ __forceinline__ void win_emit16f(const uint32_t* v, const float* bias
         }
     }
 }
-// 16 int32 sums -> 4 words of four int8 (see finalise_chunk of the row-ring kernel for the saturating packs)
-__device__ __forceinline__ void win_pack16(const uint32_t* v, const int* bias_c, int relu, int shift, uint32_t* pk)
-{
-    const int rnd = shift > 0 ? 1 << (shift - 1) : 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        int t[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) t[u] = (int)v[4 * j + u];
-        if (bias_c) {
-            const int4 b4 = ((const int4*)bias_c)[j];
-            t[0] += b4.x; t[1] += b4.y; t[2] += b4.z; t[3] += b4.w;
-        }
-        if (shift > 0) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[u] = (t[u] + rnd) >> shift;
-        }
-        uint32_t hi2;
-        if (relu) {
-            asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
-            asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(pk[j]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
-            pk[j] = __vminu4(pk[j], 0x7f7f7f7fu);
-        } else {
-            asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
-            asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(pk[j]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
-            pk[j] = __vmaxs4(pk[j], 0x81818181u);
-        }
-    }
-}
-
 // AX 0: a window runs along x; 1: along the rows (1D nets).  RWT: words of a run of a 3-row layer, known at compile time
 // (the whole window is then fetched one step ahead and leaves in 16-byte stores), or 0.
 template <int DT, int AX, int RWT>
@@ -500,8 +470,12 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                     else tmem_ld<16>(trow + c, v);
                     if (DT == 2) {
                         uint32_t pk[8];
-                        win_pack16(v, (const int*)b_lo, a.relu, a.shift, pk);
-                        win_pack16(v + 16, (const int*)b_hi, a.relu, a.shift, pk + 4);
+                        if (!a.bias) {
+                            pack_i8<32>(v, nullptr, a.relu, a.shift, pk);
+                        } else {
+                            pack_i8<16>(v, (const int*)b_lo, a.relu, a.shift, pk);
+                            pack_i8<16>(v + 16, (const int*)b_hi, a.relu, a.shift, pk + 4);
+                        }
                         if (a.out_wide) {
                             if (lo) st_global_v8(d0, pk);
                         } else {
@@ -560,7 +534,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                     const uint32_t* b = a.bias ? (const uint32_t*)a.bias + co : nullptr;
                     if (DT == 2) {
                         uint32_t pk[4];
-                        win_pack16(v, (const int*)b, a.relu, a.shift, pk);
+                        pack_i8<16>(v, (const int*)b, a.relu, a.shift, pk);
                         st_global_v4(out + e, pk);
                     } else if (a.out_elem == E_BF16) {
                         win_emit16f<E_BF16>(v, (const float*)b, a.relu, out + 2 * e, a.out_wide);

@@ -260,6 +260,51 @@ __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&v)[8])
                  :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "l"(p) : "memory");
 }
 
+// W int32 sums -> W / 4 words of four int8: shift with rounding, ReLU and clamp.  The layers that end here are bound by this
+// arithmetic, so it is kept to (two for the shift and) one instruction per value: the saturating pack of two values clamps to
+// [-128, 127], and ReLU is the sign bytes (one byte permute) masked out of four values at once.  (A byte-wise minimum on top of an
+// unsigned pack costs three times as much: it has no instruction of its own.)
+template <int W, bool SHIFT, bool BIAS>
+__device__ __forceinline__ void pack_i8_as(const uint32_t* v, const int* bias_c, int relu, int rnd, int shift, uint32_t* pk)
+{
+#pragma unroll
+    for (int j = 0; j < W / 4; ++j) {
+        int t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = (int)v[4 * j + u];
+        if (BIAS) {
+            const int4 b4 = ((const int4*)bias_c)[j];
+            t[0] += b4.x; t[1] += b4.y; t[2] += b4.z; t[3] += b4.w;
+        }
+        if (SHIFT) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[u] = (t[u] + rnd) >> shift;
+        }
+        uint32_t hi2;
+        asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
+        asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(pk[j]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
+    }
+    if (relu) {
+#pragma unroll
+        for (int j = 0; j < W / 4; ++j) {
+            uint32_t neg;
+            asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(neg) : "r"(pk[j]));         // 0xff where a byte is negative
+            pk[j] &= ~neg;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < W / 4; ++j) pk[j] = __vmaxs4(pk[j], 0x81818181u);    // symmetric: not below -127
+    }
+}
+template <int W>
+__device__ __forceinline__ void pack_i8(const uint32_t* v, const int* bias_c, int relu, int shift, uint32_t* pk)
+{
+    const int rnd = shift > 0 ? 1 << (shift - 1) : 0;
+    if (bias_c) pack_i8_as<W, true, true>(v, bias_c, relu, rnd, shift, pk);
+    else if (shift > 0) pack_i8_as<W, true, false>(v, bias_c, relu, rnd, shift, pk);
+    else pack_i8_as<W, false, false>(v, bias_c, relu, rnd, shift, pk);
+}
+
 template <int DT> struct Acc;
 template <> struct Acc<1> { typedef float S; };
 template <> struct Acc<2> { typedef int S; };
