@@ -51,8 +51,10 @@ struct LayerPlan {
     std::vector<unsigned char> wwin_packed;    // its banded weight matrix
     size_t wwin_off = 0;
     alignas(64) unsigned char w_map_win[128];
-    // x-unfold in front of the tensor-core kernel (thin or x-strided layers): the Kw taps of every
-    // output position are laid side by side as kpad channels, the conv then has Kw = 1, stride_x = 1
+    // How the tensor-core kernel sees the x axis of the layer's input: as it is; in groups of g positions as one position of
+    // g*Cin channels (x-strided layers: the stride is then 1; 16-byte positions: `pair`); or x-unfolded by a pass in front
+    // (thin layers without another form): the Kw taps of every output position side by side as kpad channels, Kw = 1.
+    int x_win = 0, x_cin = 0, x_kw = 0, x_stride = 1, x_pad = 0;
     int unfold = 0, kpad = 0, in_cap_rows = 0;
     size_t unf_off = 0;
     // host copies of the packed parameters
@@ -142,6 +144,13 @@ long long layer_rows_at_flush(const LayerPlan& P, long long rows_in)
     return P.l.kind == IDF_CONV ? conv_rows_at_flush(P.l, rows_in) : P.l.kind == IDF_MAXPOOL2 ? rows_in / 2 : (rows_in > 0 ? 1 : 0);
 }
 
+// The x axis as the tensor-core plan sees it.
+void as_planned(const LayerPlan& P, ConvArgs* t)
+{
+    if (!P.unfold) t->in_stream_elems = (long long)P.in_w * P.in_c;
+    t->Win = P.x_win; t->Cin = P.x_cin; t->Kw = P.x_kw; t->stride_x = P.x_stride; t->pad_x = P.x_pad;
+}
+
 // Enqueue one layer on n_in input rows found at in_ptr (slots 0..n_in-1).  With `flush` (n_in == 0)
 // the layer learns that its input has ended and completes the rows that wait only for bottom padding.
 // Rows it emits go to the next layer's buffer starting at slot `out_slot` (or to the caller's output
@@ -228,17 +237,15 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
         }
         if (ce == cudaErrorNotSupported && P.tc.ok && !P.use_sparse && n_in > 0) {
             ConvArgs t = a;
-            if (P.unfold && n_in <= P.in_cap_rows) {
-                ce = launch_unfold(a, (int)n_in, P.kpad, net->ws + P.unf_off, net->stream);
+            as_planned(P, &t);
+            ce = cudaSuccess;
+            if (P.unfold) {
+                ce = n_in <= P.in_cap_rows ? launch_unfold(a, (int)n_in, P.kpad, net->ws + P.unf_off, net->stream) : cudaErrorNotSupported;
                 t.in = net->ws + P.unf_off;
-                t.Win = a.Wout; t.Cin = P.kpad; t.Kw = 1; t.stride_x = 1; t.pad_x = 0;
-                if (ce == cudaSuccess) {
-                    net->launches += 1;
-                    ce = launch_conv_tc(t, P.tc, net->dtype, P.w_map, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
-                }
-            } else if (!P.unfold) {
-                ce = launch_conv_tc(t, P.tc, net->dtype, P.w_map, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
+                if (ce == cudaSuccess) net->launches += 1;
             }
+            if (ce == cudaSuccess)
+                ce = launch_conv_tc(t, P.tc, net->dtype, P.w_map, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
         if (ce == cudaErrorNotSupported)
@@ -341,13 +348,13 @@ int launch_conv_pool(idf_net* net, size_t i, const void* in_ptr, long long n_in,
     }
     cudaError_t ce;
     ConvArgs t = a;
+    as_planned(P, &t);
     if (P.unfold) {
         // (if the conv launch below declines, this pass has only filled its own buffer: harmless)
         ce = launch_unfold(a, (int)n_in, P.kpad, net->ws + P.unf_off, net->stream);
         if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed at layer %zu: %s", i, cudaGetErrorString(ce));
         net->launches += 1;
         t.in = net->ws + P.unf_off;
-        t.Win = a.Wout; t.Cin = P.kpad; t.Kw = 1; t.stride_x = 1; t.pad_x = 0;
     }
     ce = launch_conv_tc(t, P.tc_pool, net->dtype, P.w_map_pool, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
     if (net->timing) {
@@ -829,36 +836,59 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                 win_make_plan(spec->dtype, net->n_streams, P.out_w, l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, w == 1, &P.win)) {
                 P.wwin_packed.resize(P.win.w_bytes);
                 win_pack_weights(P.win, spec->dtype, weights[i], l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, P.wwin_packed.data());
-            } else if (tc_allowed && tc_make_plan(spec->dtype, net->n_streams, w, P.out_w, l.cin, l.cout, l.kh, l.kw,
-                                           w == 1 ? 1 : l.stride, P.ring_rows, (int)elem_size(P.out_elem), 0, &P.tc)) {
-                if (pool_next)
-                    tc_make_plan(spec->dtype, net->n_streams, w, P.out_w, l.cin, l.cout, l.kh, l.kw, w == 1 ? 1 : l.stride,
-                                 P.ring_rows, (int)elem_size(P.out_elem), 1, &P.tc_pool);
-                P.wtc_packed.resize(nw * es);
-                for (int co = 0; co < l.cout; ++co)
-                    for (int k = 0; k < taps; ++k)
-                        memcpy(P.wtc_packed.data() + (((size_t)tc_weight_slot(k / l.kw, k % l.kw, l.kh, l.stride) * l.cout + co) * l.cin) * es,
-                               (const unsigned char*)weights[i] + (((size_t)co * taps + k) * l.cin) * es, (size_t)l.cin * es);
             } else if (tc_allowed) {
-                // thin (Cin*Kw below a tensor-core K step) or x-strided layer: unfold x first
-                const size_t kbytes = (size_t)l.kw * l.cin * es;
-                const size_t padded = kbytes <= 32 ? 32 : (kbytes <= 64 ? 64 : (kbytes + 127) / 128 * 128);
-                const int kpad = (int)(padded / es);
-                if (padded <= 1024 &&
-                    tc_make_plan(spec->dtype, net->n_streams, P.out_w, P.out_w, kpad, l.cout, l.kh, 1, 1, P.ring_rows,
-                                 (int)elem_size(P.out_elem), 0, &P.tc)) {
+                const int sx = w == 1 ? 1 : l.stride, px = w == 1 ? 0 : l.pad;
+                // one plan for launches that emit the layer's rows, one for launches that emit pooled rows
+                auto plan_as = [&](int x_win, int x_cin, int x_kw, int x_stride, int x_pad, int pair) {
+                    if (!tc_make_plan(spec->dtype, net->n_streams, x_win, P.out_w, x_cin, l.cout, l.kh, x_kw, x_stride, P.ring_rows,
+                                      (int)elem_size(P.out_elem), 0, pair, &P.tc)) return false;
                     if (pool_next)
-                        tc_make_plan(spec->dtype, net->n_streams, P.out_w, P.out_w, kpad, l.cout, l.kh, 1, 1, P.ring_rows,
-                                     (int)elem_size(P.out_elem), 1, &P.tc_pool);
-                    P.unfold = 1;
-                    P.kpad = kpad;
-                    P.in_cap_rows = in_cap;
-                    P.wtc_packed.assign((size_t)l.kh * l.cout * kpad * es, 0);      // [ky][Cout][kx*Cin + ci], zero padded
+                        tc_make_plan(spec->dtype, net->n_streams, x_win, P.out_w, x_cin, l.cout, l.kh, x_kw, x_stride, P.ring_rows,
+                                     (int)elem_size(P.out_elem), 1, pair, &P.tc_pool);
+                    P.x_win = x_win; P.x_cin = x_cin; P.x_kw = x_kw; P.x_stride = x_stride; P.x_pad = x_pad;
+                    return true;
+                };
+                // Groups of g positions: tap kx lies at position (kx + shift) of a run of groups that starts x_pad groups to the
+                // left.  The last group of a row may reach into the next stream's row, or past the buffer: only where no output
+                // reads there (its weights are zero), the buffer is the library's own and any bits are a number (int8).
+                int g = sx > 1 ? sx : ((size_t)l.cin * es == 16 ? 2 : 1), shift = 0;
+                bool planned = false;
+                if (g > 1 && w > 1 && ((size_t)w * l.cin * es) % 16 == 0) {
+                    const bool pair = sx == 1;
+                    const int x_pad = pair ? px : (px + g - 1) / g, need = (P.out_w - 1) * sx - px + l.kw;
+                    shift = pair ? 0 : g * x_pad - px;
+                    const int x_kw = (l.kw + shift + g - 1) / g;
+                    const int whole = w / g, x_win = pair ? w : (need <= whole * g ? whole : (w + g - 1) / g);
+                    const bool spill = !pair && x_win * g > w;
+                    if (!spill || (need <= w && i > 0 && spec->dtype == IDF_I8_I32))
+                        planned = plan_as(x_win, g * l.cin, x_kw, 1, x_pad, pair);
+                }
+                if (!planned) { g = 1; shift = 0; planned = plan_as(w, l.cin, l.kw, sx, px, 0); }
+                if (planned) {
+                    const size_t tap_elems = (size_t)l.cout * P.x_cin;
+                    P.wtc_packed.assign((size_t)l.kh * P.x_kw * tap_elems * es, 0);
                     for (int co = 0; co < l.cout; ++co)
-                        for (int ky = 0; ky < l.kh; ++ky)
-                            memcpy(P.wtc_packed.data() + (((size_t)tc_weight_slot(ky, 0, l.kh, l.stride) * l.cout + co) * kpad) * es,
-                                   (const unsigned char*)weights[i] + (((size_t)co * l.kh + ky) * l.kw * l.cin) * es,
-                                   (size_t)l.kw * l.cin * es);
+                        for (int k = 0; k < taps; ++k) {
+                            const int ky = k / l.kw, t = k % l.kw + shift;
+                            memcpy(P.wtc_packed.data() + ((size_t)tc_weight_slot(ky, t / g, l.kh, l.stride) * tap_elems + (size_t)co * P.x_cin + (size_t)(t % g) * l.cin) * es,
+                                   (const unsigned char*)weights[i] + (((size_t)co * taps + k) * l.cin) * es, (size_t)l.cin * es);
+                        }
+                } else {
+                    // thin (Cin*Kw below a tensor-core K step) or x-strided layer without another form: unfold x first
+                    const size_t kbytes = (size_t)l.kw * l.cin * es;
+                    const size_t padded = kbytes <= 32 ? 32 : (kbytes <= 64 ? 64 : (kbytes + 127) / 128 * 128);
+                    const int kpad = (int)(padded / es);
+                    if (padded <= 1024 && plan_as(P.out_w, kpad, 1, 1, 0, 0)) {
+                        P.unfold = 1;
+                        P.kpad = kpad;
+                        P.in_cap_rows = in_cap;
+                        P.wtc_packed.assign((size_t)l.kh * l.cout * kpad * es, 0);      // [ky][Cout][kx*Cin + ci], zero padded
+                        for (int co = 0; co < l.cout; ++co)
+                            for (int ky = 0; ky < l.kh; ++ky)
+                                memcpy(P.wtc_packed.data() + (((size_t)tc_weight_slot(ky, 0, l.kh, l.stride) * l.cout + co) * kpad) * es,
+                                       (const unsigned char*)weights[i] + (((size_t)co * l.kh + ky) * l.kw * l.cin) * es,
+                                       (size_t)l.kw * l.cin * es);
+                    }
                 }
             }
             if (spec->dtype == IDF_I8_I32 && l.cin % 4 == 0) {
@@ -924,13 +954,14 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
             net->state_bytes_stream += P.state_bytes_stream;
         }
     }
-    // a dense tensor-core conv layer directly followed by a 2x2 max-pool emits the pooled rows itself
+    // a dense tensor-core conv layer directly followed by a 2x2 max-pool emits the pooled rows itself (the x neighbours of a
+    // pooled pair are neighbouring lanes: every stream of a tile must start on an even one)
     {
         const bool no_fuse = (debug_flags() & IDF_DEBUG_NO_POOL_FUSION) != 0;
         for (size_t i = 0; i + 1 < net->L.size(); ++i) {
             LayerPlan& P = net->L[i];
             P.fuse_pool = P.l.kind == IDF_CONV && net->L[i + 1].l.kind == IDF_MAXPOOL2 && P.tc.ok && P.tc_pool.ok && !P.use_sparse &&
-                          P.out_w >= 2 && (P.tc_pool.BX % 2) == 0 && !no_fuse && !net->eager;
+                          P.out_w >= 2 && (P.tc_pool.BX % 2) == 0 && (P.tc_pool.BXP % 2 == 0 || P.tc_pool.BS == 1) && !no_fuse && !net->eager;
         }
     }
     // one launch for all layers, state in shared memory: possible when a stream's rings, pooling rows and one row per
@@ -1078,11 +1109,9 @@ int idf_stream_open(idf_net* net, void* d_workspace, size_t workspace_bytes, voi
             e = cudaMemcpyAsync(net->ws + P.b_off, P.b_packed.data(), P.b_packed.size(), cudaMemcpyHostToDevice, net->stream);
         if (!P.wtc_packed.empty() && e == cudaSuccess) {
             e = cudaMemcpyAsync(net->ws + P.wtc_off, P.wtc_packed.data(), P.wtc_packed.size(), cudaMemcpyHostToDevice, net->stream);
-            if (tc_encode_weights(P.tc, net->dtype, net->ws + P.wtc_off, P.unfold ? P.l.kh : P.l.kh * P.l.kw,
-                                  P.unfold ? P.kpad : P.l.cin, P.l.cout, P.w_map) != 0)
+            if (tc_encode_weights(P.tc, net->dtype, net->ws + P.wtc_off, P.l.kh * P.x_kw, P.x_cin, P.l.cout, P.w_map) != 0)
                 P.tc.ok = 0;               // no TMA descriptor: this layer stays on the CUDA-core kernel
-            if (P.tc_pool.ok && tc_encode_weights(P.tc_pool, net->dtype, net->ws + P.wtc_off, P.unfold ? P.l.kh : P.l.kh * P.l.kw,
-                                                  P.unfold ? P.kpad : P.l.cin, P.l.cout, P.w_map_pool) != 0)
+            if (P.tc_pool.ok && tc_encode_weights(P.tc_pool, net->dtype, net->ws + P.wtc_off, P.l.kh * P.x_kw, P.x_cin, P.l.cout, P.w_map_pool) != 0)
                 P.tc_pool.ok = 0;
         }
         if (!P.wq_packed.empty() && e == cudaSuccess)

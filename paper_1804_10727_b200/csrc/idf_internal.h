@@ -42,6 +42,7 @@ inline size_t elem_size(int e) { return e == E_F32 || e == E_I32 ? 4 : (e == E_B
 // A free ring slot holds zeros; the state excludes the bias, which joins at emission.
 struct ConvArgs {
     const void* in;        // input rows of this block: [r - r0][S][Win][Cin]
+    long long in_stream_elems;   // elements from one stream's row to the next (0: Win*Cin)
     const void* w;         // packed weights (layout depends on the kernel)
     const void* bias;      // [Cout] in the state type, or nullptr
     void* ring;            // [ring_rows][S][Wout][Cout] state words
@@ -156,6 +157,7 @@ struct TcPlan {
     int BX = 0, BS = 0;      // a 128-row M tile = BS streams x BX consecutive x positions
     int BXP = 0;             // positions per stream held in the shared-memory tile (BX + kx halo)
     int shift_mode = 0;      // kx taps read one haloed tile at row offsets instead of one box per kx
+    int pair = 0;            // positions of 16 bytes, two to a K step
     int sx = 1;              // x stride (> 1 only without shift_mode: the tensor map walks the input row in steps of sx)
     int a_stage_bytes = 0;
     int n_box = 1, a_box_pitch = 0;   // TMA boxes per stage (one per kx tap where the taps cannot share a haloed box), their distance
@@ -174,7 +176,7 @@ struct TcPlan {
     size_t w_bytes = 0;      // device weights for this path: [tap slot][Cout][Cin] in the activation type
 };
 bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, int Kw, int stride_x, int ring_rows,
-                  int out_esize, int pooled, TcPlan* p);
+                  int out_esize, int pooled, int pair, TcPlan* p);
 int tc_weight_slot(int ky, int kx, int Kh, int stride);
 int tc_encode_weights(const TcPlan& p, int dtype, const void* d_w, int taps, int Cin, int Cout, void* map_out);
 cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const void* w_map, int n_in_rows,

@@ -179,6 +179,7 @@ struct TcArgs {
     int S, Wout, Cout, Kh, Kw, stride, pad_x, relu, shift, ring_rows, out_elem;
     int BX, BXP, BS, n_xt, Ntile, n_nt, KB, n_kb, swb, nslot, nstage, tmem_cols;
     int shift_mode;              // 1: one box per (row, K block) holds the kx halo, taps address it at row offsets
+    int pair;                    // 1: A rows are single 16-byte positions, a K step reads two neighbouring ones (see tc_make_plan)
     int sx;                      // x stride of the conv (1, or more when every kx tap has a box of its own: the tensor map then
                                  // walks the input row in steps of sx, so a box still holds BXP consecutive OUTPUT positions)
     int n_chunks, chunk_rows, chunk_shift;   // the block's output rows are cut into n_chunks runs of chunk_rows rows (the first one
@@ -224,7 +225,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int taps = a.Kh * a.Kw;
     const uint32_t w_tile_bytes = (uint32_t)a.Ntile * a.swb;
     const uint32_t a_stage_bytes = (uint32_t)a.a_stage_bytes;
-    const uint32_t a_box_bytes = (uint32_t)a.BXP * a.BS * a.swb;
+    const uint32_t a_box_bytes = (uint32_t)a.BXP * a.BS * (a.pair ? 16u : (uint32_t)a.swb);
     // (rows of 128 bytes always share one haloed box: for that instantiation the compiler sees the constant)
     const int n_box = KSTEPS == 4 ? 1 : a.n_box;
 
@@ -369,7 +370,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         mbar_expect_tx(bar_full + 8u * stage, (uint32_t)n_box * a_box_bytes);
                         for (int xl = 0; xl < n_box; ++xl)
                             tma_load_4d(sA + (uint32_t)stage * a_stage_bytes + (uint32_t)xl * a.a_box_pitch, &tmA, bar_full + 8u * stage,
-                                        kb * a.KB, x0 * a.sx - a.pad_x + xl, s0, c_ra + ri);
+                                        a.pair ? 2 * (x0 - a.pad_x) : kb * a.KB, a.pair ? 0 : x0 * a.sx - a.pad_x + xl, s0, c_ra + ri);
                         ++t;
                         if (++stage == a.nstage) { stage = 0; phase ^= 1u; }
                     }
@@ -392,7 +393,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint64_t desc_hi = make_smem_desc(0, a.swb);
             const int n_kx = KX3 ? 3 : (a.shift_mode ? a.Kw : n_box);   // kx taps of a stage: row-shifted reads of one box, or one box each
             const int nslot = a.nslot;
-            const uint32_t kx_bytes = (KSTEPS == 4 || a.shift_mode) ? (uint32_t)a.swb >> 4 : (uint32_t)a.a_box_pitch >> 4;
+            const uint32_t kx_bytes = a.pair ? 2u : ((KSTEPS == 4 || a.shift_mode) ? (uint32_t)a.swb >> 4 : (uint32_t)a.a_box_pitch >> 4);
             // weight tiles in shared memory: [K block][kx][stacked ky block]
             const uint32_t wtile_kx = ((uint32_t)a.Kh * w_tile_bytes) >> 4;              // descriptor units per kx
             const uint32_t wtile_kb = ((uint32_t)taps * w_tile_bytes) >> 4;
@@ -403,7 +404,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int slot = 0; slot < (c_n_orows < nslot ? c_n_orows : nslot) && ok; ++slot)
                 ok = mbar_wait(bar_free + 8u * slot, 0, abort_flag);
             ok = ok && mbar_wait(bar_w, 0, abort_flag);          // the CTA's weight slice has landed
-            const uint64_t adesc_base = desc_hi | (uint64_t)((sA & 0x3FFFFu) >> 4);
+            // (paired positions: no swizzle, 8 rows of 16 bytes are 128 bytes, and the second half of a K step is the next position)
+            const uint64_t adesc_base = (a.pair ? ((uint64_t)1 << 16) | ((uint64_t)8 << 32) | ((uint64_t)1 << 46) : desc_hi) | (uint64_t)((sA & 0x3FFFFu) >> 4);
             const uint64_t bdesc_base = desc_hi | (uint64_t)((sW & 0x3FFFFu) >> 4);
             const int n_st = n_kb;                               // tiles (stages) per input row
             const bool issuer = elect_one();                     // the lane that issues (the warp stays converged)
@@ -731,7 +733,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }  // namespace
 
 bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, int Kw, int stride_x, int ring_rows,
-                  int out_esize, int pooled, TcPlan* p)
+                  int out_esize, int pooled, int pair, TcPlan* p)
 {
     *p = TcPlan{};
     if (dtype != 1 && dtype != 2) return false;
@@ -743,12 +745,22 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     p->swb = row_bytes >= 128 ? 128 : row_bytes;
     p->KB = p->swb / esize;
     p->n_kb = Cin / p->KB;
-    // With 128-byte rows one box per (input row, K block) carries the Kw-1 halo positions of every
-    // stream in the tile and the kx taps read it at row offsets; narrower rows take one box per kx.
-    p->shift_mode = (p->swb == 128 && Kw > 1) ? 1 : 0;
-    const int halo = p->shift_mode ? Kw - 1 : 0;
-    if (Wout >= 128) {
-        p->n_xt = (Wout + 127) / 128;
+    // One box per (input row, K block) carries the Kw-1 halo positions of every stream in the tile and the kx taps read it at
+    // row offsets (the swizzle is a function of the absolute shared-memory address, whatever its span).  A box per kx tap, as
+    // x-strided layers whose positions cannot be taken in groups need, moves Kw times the rows through the copy engine
+    // (32 -> 64 channels int8, stride 2, 2048 streams of 254-wide rows: 2.15 ms with three strided boxes, 1.93 ms as groups of
+    // two positions).
+    // `pair`: a position is 16 bytes, half a K step.  The input row then lies in shared memory as it is (no swizzle, rows of 16
+    // bytes) and a K step is two neighbouring positions: the leading-dimension offset of the A descriptor is one row.  Cin and Kw
+    // are those of the pairs: 32 bytes, half the taps (rounded up; the odd one has zero weights).  No x-unfold pass is needed
+    // (16 -> 32 channels int8, 4096 streams of 26-wide rows with pool: 0.183 -> 0.149 ms).
+    p->pair = pair;
+    if (pair && (row_bytes != 32 || stride_x != 1)) return false;
+    p->shift_mode = Kw > 1 && stride_x == 1;
+    const int halo = pair ? 2 * Kw : (p->shift_mode ? Kw - 1 : 0);      // (paired: one position more than the taps read, an even number)
+    const int max_bx = pair ? 128 - halo : 128;          // (a paired box is counted in half positions, at most 256)
+    if (Wout >= max_bx) {
+        p->n_xt = (Wout + max_bx - 1) / max_bx;
         p->BX = (Wout + p->n_xt - 1) / p->n_xt;
         p->BS = 1;
     } else {
@@ -760,16 +772,16 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     p->BXP = p->BX + halo;
     // An x-strided layer needs one box per kx tap (the tap's positions x' * stride + kx - pad are then one strided
     // walk of the input row, which the tensor map does); the haloed tile of the row-shift mode has no such form.
-    if (stride_x != 1 && (p->shift_mode || Kw == 1)) return false;
+    if (stride_x != 1 && (p->swb == 128 || Kw == 1)) return false;
     p->sx = stride_x;
     if (p->BXP * stride_x > 256) return false;          // the box is given in input positions
     // A stage holds exactly the TMA box (BS streams x BXP positions).  The MMAs read 128 rows from row kx on,
     // so for the last positions they run past the box into whatever follows in shared memory: those are
     // lanes outside the tile, whose accumulators nobody reads.
-    // kx taps that cannot share a haloed box (rows of 32 or 64 bytes, x-strided layers) get a box each, side by side in
-    // the stage, under one barrier
-    const int n_box = (!p->shift_mode && Kw > 1) ? Kw : 1;
-    const size_t box_pitch = ((size_t)p->BS * p->BXP * p->swb + 1023) / 1024 * 1024;
+    // (the boxes of an x-strided layer lie side by side in the stage, under one barrier)
+    const int n_box = stride_x != 1 ? Kw : 1;
+    const size_t pos_bytes = pair ? 16 : p->swb;
+    const size_t box_pitch = ((size_t)p->BS * p->BXP * pos_bytes + 1023) / 1024 * 1024;
     const size_t a_stage = (size_t)n_box * box_pitch;
     p->a_stage_bytes = (int)a_stage;
     p->n_box = n_box;
@@ -822,7 +834,7 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     if (wb + (want_stages + 1) * a_stage + 2 * (size_t)p->out_groups * p->out_stage_bytes + 10240 <= SMEM_LIMIT) p->out_bufs = 2;
     // the MMAs' run past a small box (see a_stage) must end inside this CTA's shared memory: what follows the
     // last stage (the staging tiles) covers it, or padding is added behind them
-    const size_t overrun = (size_t)(128 + halo) * p->swb > box_pitch ? (size_t)(128 + halo) * p->swb - box_pitch : 0;
+    const size_t overrun = (size_t)(128 + halo) * pos_bytes > box_pitch ? (size_t)(128 + halo) * pos_bytes - box_pitch : 0;
     const size_t tail_have = (size_t)p->out_groups * p->out_bufs * p->out_stage_bytes;
     const size_t tail_pad = overrun > tail_have ? (overrun - tail_have + 1023) / 1024 * 1024 : 0;
     if (SMEM_LIMIT < 8192 + wb + 1024 + tail_have + tail_pad + 2 * a_stage) return false;
@@ -868,16 +880,22 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const 
     if (((uintptr_t)a.in & 15) != 0 || n_in_rows < 1) return cudaErrorNotSupported;
     const int esize = dtype == 1 ? 2 : 1;
     CUtensorMap tmA;
+    const long long stream_elems = a.in_stream_elems ? a.in_stream_elems : (long long)a.Win * a.Cin;
     cuuint64_t dims[4] = {(cuuint64_t)a.Cin, (cuuint64_t)a.Win, (cuuint64_t)a.S, (cuuint64_t)n_in_rows};
-    cuuint64_t strides[3] = {(cuuint64_t)a.Cin * esize, (cuuint64_t)a.Win * a.Cin * esize,
-                             (cuuint64_t)a.S * a.Win * a.Cin * esize};
+    cuuint64_t strides[3] = {(cuuint64_t)a.Cin * esize, (cuuint64_t)stream_elems * esize, (cuuint64_t)a.S * stream_elems * esize};
     // (with a traversal stride the box is counted in input positions and delivers every sx-th of them)
     cuuint32_t box[4] = {(cuuint32_t)p.KB, (cuuint32_t)(p.BXP * p.sx), (cuuint32_t)p.BS, 1};
     cuuint32_t es[4] = {1, 1, 1, 1}, es_in[4] = {1, (cuuint32_t)p.sx, 1, 1};
     if (a.stride_x != p.sx) return cudaErrorNotSupported;
-    CUresult r = enc(&tmA, dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 4,
-                     const_cast<void*>(a.in), dims, strides, box, es_in, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(p.swb),
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (p.pair) {
+        // (a stream's row in 8-byte units, two to a position; a.Win counts positions)
+        dims[0] = (cuuint64_t)a.Win * 2; dims[1] = 1;
+        strides[0] = (cuuint64_t)a.Win * 16;
+        box[0] = (cuuint32_t)p.BXP * 2; box[1] = 1;
+    }
+    CUresult r = enc(&tmA, p.pair ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 4,
+                     const_cast<void*>(a.in), dims, strides, box, es_in, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     p.pair ? CU_TENSOR_MAP_SWIZZLE_NONE : swizzle_of(p.swb), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorNotSupported;
 
     // emitted rows leave through a TMA store: [channel][x][stream][row] or [channel][x][row][stream]
@@ -924,7 +942,7 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const 
     t.pad_x = a.pad_x; t.relu = a.relu; t.shift = a.shift; t.ring_rows = a.ring_rows; t.out_elem = a.out_elem;
     t.BX = p.BX; t.BS = p.BS; t.n_xt = p.n_xt; t.Ntile = p.Ntile; t.n_nt = p.n_nt; t.KB = p.KB; t.n_kb = p.n_kb;
     t.swb = p.swb; t.nslot = p.nslot; t.nstage = p.nstage; t.tmem_cols = p.tmem_cols;
-    t.BXP = p.BXP; t.shift_mode = p.shift_mode; t.sx = p.sx; t.a_stage_bytes = p.a_stage_bytes; t.n_box = p.n_box; t.a_box_pitch = p.a_box_pitch;
+    t.BXP = p.BXP; t.shift_mode = p.shift_mode; t.pair = p.pair; t.sx = p.sx; t.a_stage_bytes = p.a_stage_bytes; t.n_box = p.n_box; t.a_box_pitch = p.a_box_pitch;
     t.out_esize = p.out_esize; t.out_pwb = p.out_pwb; t.out_panels = p.out_panels; t.out_stage_bytes = p.out_stage_bytes; t.out_stage_rows = p.out_stage_rows; t.out_groups = p.out_groups; t.out_bufs = p.out_bufs;
     t.out_row_dim = row_dim; t.out_row_first = (int)(a.o_begin - a.out_row_base);
     t.pool = a.pool_fused; t.pool_keep = a.pool_keep; t.pool_state = a.pool_state; t.pool_row_base = a.out_row_base;
