@@ -323,8 +323,8 @@ int idf_conv_rows_noalloc(const float* d_in, int n_rows, int n_streams, int in_w
 /* Debug only.  Process-wide switches that route work away from the default kernels so that tests can compare
  * the paths with one another; results are the same with any combination (bit-exact for int nets), only the
  * kernels and launch counts differ.  Not for production use; the paper has no counterpart.  flags is a
- * combination of the bits below (0 = defaults); IDF_DEBUG_NO_TENSOR_CORES, IDF_DEBUG_NO_POOL_FUSION and
- * IDF_DEBUG_PREFER_THIN are read by idf_net_create (they affect nets created afterwards), the others at every push or launch.
+ * combination of the bits below (0 = defaults); IDF_DEBUG_NO_TENSOR_CORES, IDF_DEBUG_NO_POOL_FUSION,
+ * IDF_DEBUG_PREFER_THIN and IDF_DEBUG_NO_TILED_EAGER are read by idf_net_create (they affect nets created afterwards), the others at every push or launch.
  * IDF_ERR_ARG for an unknown bit (nothing changes). */
 typedef enum {
     IDF_DEBUG_NO_TENSOR_CORES = 1,  /* dense layers stay on the CUDA-core kernel                              */
@@ -334,7 +334,8 @@ typedef enum {
     IDF_DEBUG_PREFER_THIN = 16,     /* thin layers (receptive field of at most 128 bytes) take the thin-layer */
                                     /* kernel also where x-unfold + row ring is the default (2D nets)          */
     IDF_DEBUG_NO_FUSED = 32,        /* never the single launch over all layers (state in shared memory)       */
-    IDF_DEBUG_FORCE_FUSED = 64      /* ... always, where a stream's state fits (by default: small pushes only) */
+    IDF_DEBUG_FORCE_FUSED = 64,     /* ... always, where a stream's state fits (by default: small pushes only) */
+    IDF_DEBUG_NO_TILED_EAGER = 128  /* eager emission: the plain kernels for every shape               */
 } idf_debug_flag;
 int idf_set_debug_flags(unsigned int flags);
 

@@ -71,6 +71,8 @@ struct LayerPlan {
     int fire_rows = 0;                     // the layer runs once this many rows wait (or when a push ends)
     int fuse_pool = 0;                     // conv layer whose tensor-core launch may emit the following 2x2 max-pool's rows
     // eager emission: rings of e_cap rows for the state, the announced activation and the change of the current step
+    int e_d_elem = 0;                      // element type of the announced changes
+    size_t e_w_words = 0, e_d_words = 0;   // tiled kernel: shared memory for the weights and a stream's changed rows below
     int e_cap = 0, e_window = 0;           // ring capacity in rows; most rows one segment can touch (the input cone)
     size_t e_c_off = 0, e_h_off = 0, e_d_off = 0;
     long long e_hi = -1;                   // last row touched so far
@@ -88,6 +90,8 @@ struct idf_net {
     std::vector<int> fused_state_soff, fused_rowbuf_soff;
     double macs_per_row = 0;               // multiply-accumulates one segment of one stream costs (all layers, steady state)
     int eager = 0;                         // emission policy: 0 = once per unit (deferred), 1 = after every segment (eager)
+    int eager_tiled = 0, eager_G = 0;      // every layer fits the tiled kernel; streams per block if all fit one launch, else 0
+    size_t eager_w_words = 0, eager_d_words = 0;   // shared memory: weights of all layers, most changed rows of a stream
     size_t eager_in_off = 0;               // the pushed segment as words (the input layer's announcement)
     std::vector<LayerPlan> L;
     size_t workspace_bytes = 0, state_region_off = 0, state_region_bytes = 0, counters_off = 0, status_off = 0;
@@ -503,6 +507,47 @@ void reach(const LayerPlan& P, long long lo, long long hi, long long* o_lo, long
     }
 }
 
+// One layer of an eager step: launched at once by the plain kernels; the tiled kernel takes all layers of a step together where
+// they fit (`batch`: launch_eager_batch does it after the last one).
+cudaError_t launch_eager(idf_net* net, size_t i, EagerArgs& a, EagerNetArgs* batch)
+{
+    const LayerPlan& P = net->L[i];
+    const bool int_net = net->dtype == IDF_I8_I32, pool = P.l.kind == IDF_MAXPOOL2;
+    if (!net->eager_tiled) { net->launches += 1; return launch_eager_layer(a, pool, int_net, net->stream); }
+    a.din_elem = i == 0 ? P.in_elem : net->L[i - 1].e_d_elem;
+    a.d_elem = P.e_d_elem;
+    a.wq = P.wq_packed.empty() ? nullptr : net->ws + P.wq_off;
+    if (pool && net->L[i - 1].l.kind == IDF_CONV) {
+        const LayerPlan& B = net->L[i - 1];
+        a.pool_of_conv = 1;
+        a.hin = net->ws + B.e_c_off;
+        a.below_bias = B.b_packed.empty() ? nullptr : net->ws + B.b_off;
+        a.below_relu = B.l.relu; a.below_shift = B.l.shift; a.below_round_bf16 = B.out_elem == E_BF16;
+    }
+    if (a.o_hi < a.o_lo) return cudaSuccess;
+    if (batch && net->eager_G) {
+        batch->layer[batch->n] = a;
+        batch->pool[batch->n] = pool;
+        batch->w_at[batch->n] = batch->d_at;
+        batch->d_at += (int)(P.e_w_words + 3) / 4 * 4;
+        batch->n += 1;
+        return cudaSuccess;
+    }
+    EagerNetArgs one{};
+    one.layer[0] = a; one.pool[0] = pool; one.n = 1;
+    one.G = eager_tiled_group(net->n_streams, P.e_w_words, P.e_d_words, EAGER_SMEM_WORDS);
+    one.d_at = (int)P.e_w_words;
+    net->launches += 1;
+    return launch_eager_tiled(one, int_net, P.e_w_words + one.G * P.e_d_words, net->stream);
+}
+cudaError_t launch_eager_batch(idf_net* net, EagerNetArgs* batch)
+{
+    if (batch->n == 0) return cudaSuccess;
+    batch->G = net->eager_G;
+    net->launches += 1;
+    return launch_eager_tiled(*batch, net->dtype == IDF_I8_I32, (size_t)batch->d_at + net->eager_G * net->eager_d_words, net->stream);
+}
+
 // Eager emission, one segment at a time: the segment is the input layer's announcement; every layer in turn takes up
 // the changes of the rows below that moved, re-evaluates the rows of its cone and announces their changes.
 int eager_step(idf_net* net, const void* seg, long long r, void* d_out, long long out_cap)
@@ -510,10 +555,14 @@ int eager_step(idf_net* net, const void* seg, long long r, void* d_out, long lon
     const long long S = net->n_streams;
     const bool int_net = net->dtype == IDF_I8_I32;
     unsigned long long* counters = (unsigned long long*)(net->ws + net->counters_off);
-    cudaError_t ce = launch_eager_input(seg, net->L[0].in_elem, net->ws + net->eager_in_off, S * net->in_w * net->in_c,
-                                        counters, net->stream);
-    if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed (eager input): %s", cudaGetErrorString(ce));
-    net->launches += 1;
+    cudaError_t ce = cudaSuccess;
+    if (!net->eager_tiled) {
+        ce = launch_eager_input(seg, net->L[0].in_elem, net->ws + net->eager_in_off, S * net->in_w * net->in_c, counters, net->stream);
+        if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed (eager input): %s", cudaGetErrorString(ce));
+        net->launches += 1;
+    }
+    EagerNetArgs batch;                    // (filled layer by layer; only the first n entries are read)
+    batch.n = 0; batch.d_at = 0;
     long long lo = r, hi = r;
     for (size_t i = 0; i < net->L.size(); ++i) {
         LayerPlan& P = net->L[i];
@@ -542,12 +591,14 @@ int eager_step(idf_net* net, const void* seg, long long r, void* d_out, long lon
         a.out_elems = S * out_cap * P.out_w * P.out_c;
         a.status = (unsigned int*)(net->ws + net->status_off);
         if (o_hi - o_lo + 1 > P.e_window) return fail(IDF_ERR_CAPACITY, "internal: layer %zu cone of %lld rows exceeds %d", i, o_hi - o_lo + 1, P.e_window);
-        ce = launch_eager_layer(a, P.l.kind == IDF_MAXPOOL2, int_net, net->stream);
+        if (net->eager_tiled && i == 0) { a.din = seg; a.in_events = counters; }
+        ce = launch_eager(net, i, a, &batch);
         if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed at layer %zu: %s", i, cudaGetErrorString(ce));
-        net->launches += 1;
         if (o_hi > P.e_hi) P.e_hi = o_hi;
         lo = o_lo; hi = o_hi;
     }
+    ce = launch_eager_batch(net, &batch);
+    if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed (eager step): %s", cudaGetErrorString(ce));
     return IDF_OK;
 }
 
@@ -572,6 +623,7 @@ int eager_finish(idf_net* net, void* d_out, long long out_cap)
     for (size_t i = 0; i < net->L.size(); ++i) {
         LayerPlan& P = net->L[i];
         const bool last = i + 1 == net->L.size();
+        const long long below_rows = h;
         h = layer_rows_at_flush(P, h);                       // rows this layer's map really has
         long long p_lo = (1LL << 62), p_hi = -1;
         if (changed) reach(P, lo, hi, &p_lo, &p_hi);
@@ -602,9 +654,10 @@ int eager_finish(idf_net* net, void* d_out, long long out_cap)
         a.status = (unsigned int*)(net->ws + net->status_off);
         // (rows beyond the caller's buffer are not written: they hold nothing the caller will read)
         if (last && a.o_hi >= out_cap) a.o_hi = out_cap - 1;
-        cudaError_t ce = launch_eager_layer(a, P.l.kind == IDF_MAXPOOL2, int_net, net->stream);
+        // (conv rows beyond the end of the input stand at 0; the plain kernels have written that into their h ring)
+        if (net->eager_tiled && P.l.kind == IDF_MAXPOOL2) a.in_hi = std::min(a.in_hi, below_rows - 1);
+        cudaError_t ce = launch_eager(net, i, a, nullptr);
         if (ce != cudaSuccess) return fail(IDF_ERR_CUDA, "kernel launch failed at layer %zu: %s", i, cudaGetErrorString(ce));
-        net->launches += 1;
         changed = true; lo = p_lo; hi = p_hi;
     }
     return IDF_OK;
@@ -727,7 +780,7 @@ const char* idf_last_error(void) { return g_err.c_str(); }
 
 int idf_set_debug_flags(unsigned int flags)
 {
-    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED))
+    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED | IDF_DEBUG_NO_TILED_EAGER))
         return fail(IDF_ERR_ARG, "unknown debug flag in 0x%x", flags);
     g_debug_flags.store(flags, std::memory_order_relaxed);
     return IDF_OK;
@@ -945,6 +998,20 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                 P.e_window = std::max<long long>(P.e_window, hi - lo + 1);
             }
         }
+        // The tiled kernels pass changes of int nets on as int8: a unit behind a ReLU stands at 0..127 and moves by at most that.
+        net->eager_tiled = !(debug_flags() & IDF_DEBUG_NO_TILED_EAGER);
+        const bool int_net = net->dtype == IDF_I8_I32;
+        for (size_t i = 0; i < net->L.size(); ++i) {
+            LayerPlan& P = net->L[i];
+            P.e_d_elem = int_net ? E_I8 : E_F32;
+            if (int_net && P.l.kind == IDF_CONV && !P.l.relu) net->eager_tiled = 0;
+            if (!eager_tiled_words(P.l.kind == IDF_MAXPOOL2, int_net, P.in_w, P.in_c, P.out_c, P.l.kh, P.l.kw,
+                                   (int)(i ? net->L[i - 1].e_window : 1), &P.e_w_words, &P.e_d_words))
+                net->eager_tiled = 0;
+            net->eager_w_words += P.e_w_words;
+            net->eager_d_words = std::max(net->eager_d_words, P.e_d_words);
+        }
+        net->eager_G = net->L.size() <= EAGER_MAX_LAYERS ? eager_tiled_group(net->n_streams, net->eager_w_words, net->eager_d_words, EAGER_SMEM_WORDS) : 0;
         net->state_bytes_stream = 0;
         for (auto& P : net->L) {
             P.e_cap = P.e_window + 2;      // (a pooling layer above still reads the two rows below its oldest open pair)

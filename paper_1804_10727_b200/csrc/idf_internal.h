@@ -114,7 +114,29 @@ struct EagerArgs {
     long long o_cut;          // rows >= o_cut turn out not to exist (end of input): their activation goes back to 0
     long long in_elems, ring_elems, out_elems;    // extents of din/hin, of each of c/h/d, of out (range-checked build)
     unsigned int* status;
+    // Tiled kernels only: changes travel in the activation type where they fit (din_elem, d_elem: Elem), the first layer reads the
+    // pushed segment itself and counts its events, conv layers keep no ring of announced activations (h = f(c + b) of the old state).
+    int din_elem, d_elem;
+    const void* wq;                // int nets, Cin % 4 == 0: four input channels to a word [Kh][Kw][Cin/4][Cout], else nullptr
+    unsigned long long* in_events; // first layer: count of non-zero input components, else nullptr
+    int pool_of_conv;              // pool layer on a conv layer: the inputs are f(c + b) of that layer's states `hin`
+    const void* below_bias;
+    int below_relu, below_shift, below_round_bf16;
 };
+// Tiled eager kernel: n consecutive layers of one segment in one launch, a block per group of G streams.
+constexpr int EAGER_MAX_LAYERS = 12;
+struct EagerNetArgs {
+    EagerArgs layer[EAGER_MAX_LAYERS];
+    int pool[EAGER_MAX_LAYERS];    // 1: max-pool layer
+    int w_at[EAGER_MAX_LAYERS];    // conv: first word of its weights in shared memory
+    int n, G, d_at;                // layers, streams per block, first word of the changed rows in shared memory
+};
+// Shared-memory words one layer needs for its weights and for at most rows_in changed rows of one stream; false: not a shape for the
+// tiled kernel.
+bool eager_tiled_words(int is_pool, int int_net, int Win, int Cin, int Cout, int Kh, int Kw, int rows_in, size_t* w, size_t* d);
+int eager_tiled_group(int S, size_t w, size_t d, size_t limit_words);   // streams per block, 0: one stream does not fit
+constexpr size_t EAGER_SMEM_WORDS = 24 * 1024;    // 96 KB: two blocks per SM
+cudaError_t launch_eager_tiled(const EagerNetArgs& a, int int_net, size_t smem_words, cudaStream_t st);
 cudaError_t launch_eager_input(const void* in, int in_elem, void* d, long long n, unsigned long long* events, cudaStream_t st);
 cudaError_t launch_eager_layer(const EagerArgs& a, int is_pool, int int_net, cudaStream_t st);
 
