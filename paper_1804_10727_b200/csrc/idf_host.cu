@@ -528,15 +528,16 @@ cudaError_t launch_eager(idf_net* net, size_t i, EagerArgs& a, EagerNetArgs* bat
     if (batch && net->eager_G) {
         batch->layer[batch->n] = a;
         batch->pool[batch->n] = pool;
-        batch->w_at[batch->n] = batch->d_at;
-        batch->d_at += (int)(P.e_w_words + 3) / 4 * 4;
+        batch->w_at[batch->n] = batch->d_at[0];
+        batch->d_at[0] += (int)(P.e_w_words + 3) / 4 * 4;
         batch->n += 1;
         return cudaSuccess;
     }
     EagerNetArgs one{};
     one.layer[0] = a; one.pool[0] = pool; one.n = 1;
     one.G = eager_tiled_group(net->n_streams, P.e_w_words, P.e_d_words, EAGER_SMEM_WORDS);
-    one.d_at = (int)P.e_w_words;
+    one.d_at[0] = one.d_at[1] = (int)P.e_w_words;
+    one.d_ring = 1;
     net->launches += 1;
     return launch_eager_tiled(one, int_net, P.e_w_words + one.G * P.e_d_words, net->stream);
 }
@@ -545,7 +546,9 @@ cudaError_t launch_eager_batch(idf_net* net, EagerNetArgs* batch)
     if (batch->n == 0) return cudaSuccess;
     batch->G = net->eager_G;
     net->launches += 1;
-    return launch_eager_tiled(*batch, net->dtype == IDF_I8_I32, (size_t)batch->d_at + net->eager_G * net->eager_d_words, net->stream);
+    const size_t rows = (size_t)net->eager_G * net->eager_d_words;
+    batch->d_at[1] = batch->d_at[0] + (int)rows;
+    return launch_eager_tiled(*batch, net->dtype == IDF_I8_I32, (size_t)batch->d_at[1] + rows, net->stream);
 }
 
 // Eager emission, one segment at a time: the segment is the input layer's announcement; every layer in turn takes up
@@ -562,7 +565,7 @@ int eager_step(idf_net* net, const void* seg, long long r, void* d_out, long lon
         net->launches += 1;
     }
     EagerNetArgs batch;                    // (filled layer by layer; only the first n entries are read)
-    batch.n = 0; batch.d_at = 0;
+    batch.n = 0; batch.d_at[0] = 0; batch.d_ring = 0;
     long long lo = r, hi = r;
     for (size_t i = 0; i < net->L.size(); ++i) {
         LayerPlan& P = net->L[i];

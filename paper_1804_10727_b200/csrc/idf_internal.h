@@ -129,13 +129,15 @@ struct EagerNetArgs {
     EagerArgs layer[EAGER_MAX_LAYERS];
     int pool[EAGER_MAX_LAYERS];    // 1: max-pool layer
     int w_at[EAGER_MAX_LAYERS];    // conv: first word of its weights in shared memory
-    int n, G, d_at;                // layers, streams per block, first word of the changed rows in shared memory
+    int n, G, d_at[2];             // layers, streams per block; changed rows in shared memory: layer l reads at d_at[l & 1], leaves its own at the other
+    int d_ring;                    // 1: one layer at a time, changes travel through the d rings in global memory
 };
 // Shared-memory words one layer needs for its weights and for at most rows_in changed rows of one stream; false: not a shape for the
 // tiled kernel.
 bool eager_tiled_words(int is_pool, int int_net, int Win, int Cin, int Cout, int Kh, int Kw, int rows_in, size_t* w, size_t* d);
 int eager_tiled_group(int S, size_t w, size_t d, size_t limit_words);   // streams per block, 0: one stream does not fit
 constexpr size_t EAGER_SMEM_WORDS = 24 * 1024;    // 96 KB: two blocks per SM
+enum EagerOut : int { EO_NONE = 0, EO_RING = 1, EO_QUADS = 2, EO_WORDS = 3 };   // where a layer's changes go
 cudaError_t launch_eager_tiled(const EagerNetArgs& a, int int_net, size_t smem_words, cudaStream_t st);
 cudaError_t launch_eager_input(const void* in, int in_elem, void* d, long long n, unsigned long long* events, cudaStream_t st);
 cudaError_t launch_eager_layer(const EagerArgs& a, int is_pool, int int_net, cudaStream_t st);

@@ -186,7 +186,9 @@ __global__ void __launch_bounds__(256) eager_pool_kernel(EagerArgs a)
 // broadcast load of NC weights, NC multiply-adds (dp4a on four channels for int nets).  A unit's old activation is f(c + b) of the
 // state it reads anyway.  Bound by shared-memory and multiply-add instructions.  Measured, 512 streams of 28x28 int8 (conv 1->16->32,
 // pool, 32->32), one row per push: 195 us per push with a thread per unit (global loads and a zero test per multiply-add, an atomic
-// per warp for the event counts, a launch per layer), 64 us tiled with a launch per layer, XX us in one launch.
+// per warp for the event counts, a launch per layer), 64 us tiled with a launch per layer, 48 us in one launch,
+// 39 us with the changes handed on in shared memory and int activations compared as bytes.  (Warp-level int8 matrix products instead of
+// dp4a: slower, 51 us.)
 constexpr int EAGER_THREADS = 512;
 constexpr int EAGER_NC = 8;
 
@@ -203,9 +205,8 @@ template <int NC> __device__ __forceinline__ void st_words(void* p, const uint32
 #pragma unroll
     for (int j = 0; j < NC / 4; ++j) ((uint4*)p)[j] = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
 }
-template <int NC> __device__ __forceinline__ void st_values(void* base, long long at, int elem, const float* v)
+template <int NC> __device__ __forceinline__ void st_values(void* base, long long at, const float* v)
 {
-    (void)elem;
     float* p = (float*)base + at;
     if (((uintptr_t)p & 15) == 0) st_words<NC>(p, (const uint32_t*)v);
     else {
@@ -213,55 +214,130 @@ template <int NC> __device__ __forceinline__ void st_values(void* base, long lon
         for (int j = 0; j < NC; ++j) p[j] = v[j];
     }
 }
-template <int NC> __device__ __forceinline__ void st_values(void* base, long long at, int elem, const int* v)
+template <int NC> __device__ __forceinline__ void st_bytes(int8_t* p, const uint32_t* v)
 {
-    if (elem != E_I8) { st_words<NC>((int*)base + at, (const uint32_t*)v); return; }
-    int8_t* p = (int8_t*)base + at;
     if (((uintptr_t)p & 3) == 0) {
 #pragma unroll
-        for (int j = 0; j < NC / 4; ++j)
-            ((uint32_t*)p)[j] = __byte_perm(__byte_perm(v[4 * j], v[4 * j + 1], 0x0040), __byte_perm(v[4 * j + 2], v[4 * j + 3], 0x0040), 0x5410);
+        for (int j = 0; j < NC / 4; ++j) ((uint32_t*)p)[j] = v[j];
     } else {
 #pragma unroll
-        for (int j = 0; j < NC; ++j) p[j] = (int8_t)v[j];
+        for (int j = 0; j < NC; ++j) p[j] = (int8_t)(v[j >> 2] >> (8 * (j & 3)));
     }
 }
 __device__ __forceinline__ float as_ts(float, uint32_t v) { return __uint_as_float(v); }
 __device__ __forceinline__ int as_ts(int, uint32_t v) { return (int)v; }
 
-template <typename TS, int NC, bool QUADS>
-__device__ __forceinline__ void eager_conv_units(const EagerArgs& a, const uint32_t* sw, const uint32_t* sd, int G, int s0, int Gn, unsigned int& n_out)
+// n / d by one multiplication (n below 2^16, d below 2^16: 0xffffffff / d + 1 is exact there)
+struct FastDiv {
+    uint32_t m;
+    int d;
+    __device__ __forceinline__ explicit FastDiv(int div) : m(0xffffffffu / (uint32_t)div + 1u), d(div) {}
+    __device__ __forceinline__ int div(int n, int& rem) const
+    {
+        const int q = d == 1 ? n : (int)__umulhi((uint32_t)n, m);
+        rem = n - q * d;
+        return q;
+    }
+};
+// A unit's NC changes (int nets: as words of four int8) on their way to the layer above: its d ring, or its changed rows in
+// shared memory, word (row_g * groups + group) * W + x.
+template <int NC>
+__device__ __forceinline__ void pass_changes(int mode, uint32_t* dn, int row_g, int C, int co, int W, int x, void* dring, long long e, const float* d)
 {
+    if (mode == EO_WORDS) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) dn[(row_g * C + co + j) * W + x] = __float_as_uint(d[j]);
+    } else if (mode == EO_RING) {
+        st_values<NC>(dring, e, d);
+    }
+}
+template <int NC>
+__device__ __forceinline__ void pass_changes(int mode, uint32_t* dn, int row_g, int C, int co, int W, int x, void* dring, long long e, const uint32_t* d)
+{
+    if (mode == EO_QUADS) {
+#pragma unroll
+        for (int j = 0; j < NC / 4; ++j) dn[(row_g * (C >> 2) + (co >> 2) + j) * W + x] = d[j];
+    } else if (mode == EO_WORDS) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) dn[(row_g * C + co + j) * W + x] = (uint32_t)(int)(int8_t)(d[j >> 2] >> (8 * (j & 3)));
+    } else if (mode == EO_RING) {
+        st_bytes<NC>((int8_t*)dring + e, d);
+    }
+}
+// h = f(c + b) of NC int units as bytes, and the bytes of h_new - h_old (both in 0..127: with bit 7 set first, and put right after,
+// no borrow crosses a byte)
+template <int NC>
+__device__ __forceinline__ void act_bytes(const uint32_t* c, const int* bias, int rnd, int shift, uint32_t* h)
+{
+#pragma unroll
+    for (int q = 0; q < NC / 4; ++q) {
+        int t[4];
+        uint32_t hi2, neg;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = ((int)c[4 * q + j] + (bias ? bias[4 * q + j] : 0) + rnd) >> shift;
+        asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi2) : "r"(t[3]), "r"(t[2]));
+        asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(h[q]) : "r"(t[1]), "r"(t[0]), "r"(hi2));
+        asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(neg) : "r"(h[q]));              // ReLU: 0xff where a byte is negative
+        h[q] &= ~neg;
+    }
+}
+__device__ __forceinline__ uint32_t sub_bytes(uint32_t x, uint32_t y) { return ((x | 0x80808080u) - y) ^ 0x80808080u; }
+__device__ __forceinline__ unsigned int count_bytes(uint32_t x) { return __popc((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) & 0x80808080u); }
+
+// (What the loops need of the arguments is copied out first: they lie in parameter space behind a runtime layer index, where every
+// use would be a load of its own.)
+template <typename TS, int NC, bool QUADS>
+__device__ __forceinline__ void eager_conv_units(const EagerArgs& a, const uint32_t* sw, const uint32_t* sd, int G, int s0, int Gn, int mode, uint32_t* dn, unsigned int& n_out)
+{
+    constexpr bool INT = (TS)0.5f == (TS)0;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int CQ = QUADS ? a.Cin >> 2 : a.Cin;
-    const int n_pw = (Gn * a.Wout + 31) >> 5, n_oct = a.Cout / NC;
-    const int n_units = (int)(a.o_hi - a.o_lo + 1) * n_pw * n_oct;
+    const int CQ = QUADS ? a.Cin >> 2 : a.Cin, Win = a.Win, Wout = a.Wout, Cout = a.Cout, Kw = a.Kw, stride = a.stride, stride_x = a.stride_x, pad_x = a.pad_x;
+    const int relu = a.relu, shift = a.shift, round_bf16 = a.round_bf16, rnd = shift > 0 ? 1 << (shift - 1) : 0;
+    const int n_pos = Gn * Wout, n_rows = (int)(a.o_hi - a.o_lo + 1);
+    const FastDiv by_oct(Cout / NC), by_run((n_pos + 31) >> 5), by_w(Wout);
+    const int n_units = n_rows * by_run.d * by_oct.d;
+    const int tap0 = (int)(a.in_lo - (a.o_lo * stride - a.pad)), n_in = (int)(a.in_hi - a.in_lo + 1), Kh = a.Kh;    // row o_lo reaches changed row 0 through tap tap0
+    const int slot0 = (int)(a.o_lo % a.cap), cap = a.cap;
+    const int new_rel = (int)min(a.o_new - a.o_lo, (long long)n_rows), cut_rel = (int)min(a.o_cut - a.o_lo, (long long)n_rows);
+    const long long row_elems = (long long)a.S * Wout * Cout;
+    uint32_t* cring = (uint32_t*)a.c + (long long)s0 * Wout * Cout;
+    void* dring = a.d;
     const TS* __restrict__ bias = (const TS*)a.bias;
+    const bool last = a.out != nullptr;
     for (int u = tid >> 5; u < n_units; u += blockDim.x >> 5) {
-        const int oct = u % n_oct, t = u / n_oct, pw = t % n_pw;
-        const long long o = a.o_lo + t / n_pw;
-        const int pos = pw * 32 + lane, co = oct * NC;
-        const bool live = pos < Gn * a.Wout;
-        const int g = live ? pos / a.Wout : 0, x = live ? pos - g * a.Wout : 0;
+        int oct, run, x;
+        const int orel = by_run.div(by_oct.div(u, oct), run);
+        const int pos = run * 32 + lane, co = oct * NC;
+        const bool live = pos < n_pos;
+        const int g = by_w.div(live ? pos : 0, x);
+        int slot = slot0 + orel;                                                // (a cone has at most `cap` rows)
+        if (slot >= cap) slot -= cap;
+        const long long e = slot * row_elems + pos * Cout + co;                 // from the block's first stream
+        const bool ok = live && IDF_OK_AT(a.status, e + (long long)s0 * Wout * Cout, a.ring_elems - (NC - 1));
+        const bool fresh = orel >= new_rel;                                     // first touch: the slot still holds an older row
+        uint32_t cw[NC];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) cw[j] = 0u;
+        if (ok && !fresh) ld_words<NC>(cring + e, cw);                          // (in flight during the sum)
         TS acc[NC];
 #pragma unroll
         for (int j = 0; j < NC; ++j) acc[j] = 0;
-        // changed rows below that row o reaches: taps ky0 ... ky1
-        const int first = (int)(a.in_lo - (o * a.stride - a.pad)), last = (int)(a.in_hi - (o * a.stride - a.pad));
-        const int ky0 = max(0, first), ky1 = min(a.Kh - 1, last);
-        for (int ky = ky0; ky <= ky1; ++ky) {
-            const uint32_t* drow = sd + ((ky - first) * G + g) * CQ * a.Win;
-            for (int kx = 0; kx < a.Kw; ++kx) {
-                const int ix = x * a.stride_x - a.pad_x + kx;
-                const bool in = (unsigned)ix < (unsigned)a.Win;
-                const uint32_t* wp = sw + (ky * a.Kw + kx) * CQ * a.Cout + co;
-                const uint32_t* dp = drow + (in ? ix : 0);
+        // changed rows below that this row reaches: taps first ... first + n_in - 1, as far as they are taps
+        const int first = tap0 - orel * stride;
+        const int ky0 = max(0, first), ky1 = min(Kh, first + n_in);
+        const int ix0 = x * stride_x - pad_x;
+        for (int ky = ky0; ky < ky1; ++ky) {
+            const uint32_t* drow = sd + ((ky - first) * G + g) * CQ * Win;
+            const uint32_t* wp = sw + ky * Kw * CQ * Cout + co;
+            for (int kx = 0; kx < Kw; ++kx) {
+                const bool in = (unsigned)(ix0 + kx) < (unsigned)Win;
+                const uint32_t* dp = drow + (in ? ix0 + kx : 0);
 #pragma unroll 4
-                for (int c = 0; c < CQ; ++c) {
-                    uint32_t v = dp[c * a.Win];
+                for (int c = 0; c < CQ; ++c, dp += Win, wp += Cout) {
+                    uint32_t v = *dp;
                     if (!in) v = 0u;
                     uint32_t wv[NC];
-                    ld_words<NC>(wp + c * a.Cout, wv);
+                    ld_words<NC>(wp, wv);
 #pragma unroll
                     for (int j = 0; j < NC; ++j) {
                         if constexpr (QUADS) acc[j] = __dp4a((int)v, (int)wv[j], acc[j]);
@@ -270,76 +346,123 @@ __device__ __forceinline__ void eager_conv_units(const EagerArgs& a, const uint3
                 }
             }
         }
-        const long long e = (((o % a.cap) * a.S + s0 + g) * a.Wout + x) * (long long)a.Cout + co;
-        if (!live || !IDF_OK_AT(a.status, e, a.ring_elems - (NC - 1))) continue;
-        const bool fresh = o >= a.o_new;                                        // first touch: the slot still holds an older row
-        uint32_t cw[NC];
+        if (!ok) continue;
+        const long long ring_at = e + (long long)s0 * Wout * Cout;
+        const long long out_at = last ? (long long)(s0 + g) * a.out_stream_stride + (a.o_lo + orel) * a.out_row_stride + (long long)x * Cout + co : 0;
+        const bool emit = last && IDF_OK_AT(a.status, out_at, a.out_elems - (NC - 1));
+        if constexpr (INT) {
+            const int* b = bias ? (const int*)bias + co : nullptr;
+            uint32_t h_old[NC / 4], h_new[NC / 4], d[NC / 4];
+            act_bytes<NC>(cw, b, rnd, shift, h_old);
 #pragma unroll
-        for (int j = 0; j < NC; ++j) cw[j] = 0u;
-        if (!fresh) ld_words<NC>((const uint32_t*)a.c + e, cw);
-        TS d[NC], h[NC];
+            for (int j = 0; j < NC; ++j) cw[j] += (uint32_t)acc[j];
+            act_bytes<NC>(cw, b, rnd, shift, h_new);
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            const TS b = bias ? bias[co + j] : (TS)0, c_old = as_ts(TS(0), cw[j]), c_new = c_old + acc[j];
-            const TS h_old = fresh ? (TS)0 : eager_act(c_old, b, a.relu, a.shift, a.round_bf16);
-            h[j] = o >= a.o_cut ? (TS)0 : eager_act(c_new, b, a.relu, a.shift, a.round_bf16);
-            d[j] = h[j] - h_old;
-            n_out += d[j] != (TS)0;
-            cw[j] = *(const uint32_t*)&c_new;
-        }
-        st_words<NC>((uint32_t*)a.c + e, cw);
-        st_values<NC>(a.d, e, a.d_elem, d);
-        if (a.out) {
-            const long long i = (long long)(s0 + g) * a.out_stream_stride + o * a.out_row_stride + (long long)x * a.Cout + co;
-            if (IDF_OK_AT(a.status, i, a.out_elems - (NC - 1))) st_values<NC>(a.out, i, E_I8, h);
+            for (int j = 0; j < NC / 4; ++j) {
+                if (orel >= cut_rel) h_new[j] = 0u;
+                d[j] = sub_bytes(h_new[j], fresh ? 0u : h_old[j]);
+                n_out += count_bytes(d[j]);
+            }
+            st_words<NC>(cring + e, cw);
+            pass_changes<NC>(mode, dn, orel * G + g, Cout, co, Wout, x, dring, ring_at, d);
+            if (emit) st_bytes<NC>((int8_t*)a.out + out_at, h_new);
+        } else {
+            float d[NC], h[NC];
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const float b = bias ? (float)bias[co + j] : 0.f, c_old = __uint_as_float(cw[j]), c_new = c_old + (float)acc[j];
+                const float h_old = fresh ? 0.f : eager_act(c_old, b, relu, shift, round_bf16);
+                h[j] = orel >= cut_rel ? 0.f : eager_act(c_new, b, relu, shift, round_bf16);
+                d[j] = h[j] - h_old;
+                n_out += d[j] != 0.f;
+                cw[j] = __float_as_uint(c_new);
+            }
+            st_words<NC>(cring + e, cw);
+            pass_changes<NC>(mode, dn, orel * G + g, Cout, co, Wout, x, dring, ring_at, d);
+            if (emit) st_values<NC>(a.out, out_at, h);
         }
     }
 }
 
 template <typename TS, int NC>
-__device__ __forceinline__ void eager_pool_units(const EagerArgs& a, int s0, int Gn, unsigned int& n_out)
+__device__ __forceinline__ void eager_pool_units(const EagerArgs& a, int G, int s0, int Gn, int mode, uint32_t* dn, unsigned int& n_out)
 {
-    const int px = a.Win == 1 ? 1 : 2, n_oct = a.Cout / NC;
-    const int n = (int)(a.o_hi - a.o_lo + 1) * Gn * a.Wout * n_oct;
+    constexpr bool INT = (TS)0.5f == (TS)0;
+    const int px = a.Win == 1 ? 1 : 2, Win = a.Win, C = a.Cout, Wout = a.Wout, S = a.S;
+    const FastDiv by_oct(C / NC), by_w(Wout), by_g(Gn);
+    const int n_rows = (int)(a.o_hi - a.o_lo + 1), n = n_rows * Gn * Wout * by_oct.d;
     const TS* __restrict__ bias = (const TS*)a.below_bias;
+    const int of_conv = a.pool_of_conv, relu = a.below_relu, shift = a.below_shift, round_bf16 = a.below_round_bf16, rnd = shift > 0 ? 1 << (shift - 1) : 0;
+    const int slot0 = (int)(a.o_lo % a.cap), cap = a.cap, slot_in0 = (int)((2 * a.o_lo) % a.cap_in), cap_in = a.cap_in;
+    const int new_rel = (int)min(a.o_new - a.o_lo, (long long)n_rows), cut_rel = (int)min(a.o_cut - a.o_lo, (long long)n_rows);
+    const int have_in = (int)min(a.in_hi + 1 - 2 * a.o_lo, 2LL * n_rows);        // rows below, from 2 * o_lo on, that have announced anything
+    const uint32_t* hin = (const uint32_t*)a.hin;
     for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int co = (idx % n_oct) * NC, t = idx / n_oct, x = t % a.Wout, t2 = t / a.Wout, s = s0 + t2 % Gn;
-        const long long o = a.o_lo + t2 / Gn;
+        // (more than 2^16 items where rows are wide and channels many: by division there)
+        int oct, x, sg;
+        int t, t2, orel;
+        if (n <= 65536) { t = by_oct.div(idx, oct); t2 = by_w.div(t, x); orel = by_g.div(t2, sg); }
+        else { t = idx / by_oct.d; oct = idx - t * by_oct.d; t2 = t / Wout; x = t - t2 * Wout; orel = t2 / Gn; sg = t2 - orel * Gn; }
+        const int co = oct * NC, s = s0 + sg;
         TS m[NC];
-        for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+            int slot = slot_in0 + 2 * orel + dy;
+            while (slot >= cap_in) slot -= cap_in;
             for (int dx = 0; dx < px; ++dx) {
-                const long long i = 2 * o + dy;
-                const long long at = (((i % a.cap_in) * a.S + s) * a.Win + (px * x + dx)) * (long long)a.Cin + co;
+                const long long at = (((long long)slot * S + s) * Win + (px * x + dx)) * C + co;
                 uint32_t w[NC];
 #pragma unroll
-                for (int j = 0; j < NC; ++j) w[j] = 0u;
-                const bool have = i <= a.in_hi && IDF_OK_AT(a.status, at, a.in_elems - (NC - 1));
-                if (have) ld_words<NC>((const uint32_t*)a.hin + at, w);
+                for (int j = 0; j < NC; ++j) w[j] = 0u;                         // a unit that has announced nothing stands at 0
+                const bool have = 2 * orel + dy < have_in && IDF_OK_AT(a.status, at, a.in_elems - (NC - 1));
+                if (have) ld_words<NC>(hin + at, w);
+                // (int nets: f never falls when c rises, so the maximum is taken of the states and f applied to it once)
 #pragma unroll
                 for (int j = 0; j < NC; ++j) {
-                    TS v = as_ts(TS(0), w[j]);                                  // a unit that has announced nothing stands at 0
-                    if (have && a.pool_of_conv) v = eager_act(v, bias ? bias[co + j] : (TS)0, a.below_relu, a.below_shift, a.below_round_bf16);
+                    TS v = as_ts(TS(0), w[j]);
+                    if (!INT && of_conv && have) v = eager_act(v, bias ? bias[co + j] : (TS)0, relu, shift, round_bf16);
+                    if (INT && of_conv && !have) v = (TS)(-0x40000000);          // f of it is 0, whatever the bias
                     m[j] = dy + dx == 0 ? v : (v > m[j] ? v : m[j]);
                 }
             }
-        const long long e = (((o % a.cap) * a.S + s) * a.Wout + x) * (long long)a.Cout + co;
+        }
+        int slot = slot0 + orel;
+        if (slot >= cap) slot -= cap;
+        const long long e = (((long long)slot * S + s) * Wout + x) * C + co;
         if (!IDF_OK_AT(a.status, e, a.ring_elems - (NC - 1))) continue;
         uint32_t hw[NC];
 #pragma unroll
         for (int j = 0; j < NC; ++j) hw[j] = 0u;
-        if (o < a.o_new) ld_words<NC>((const uint32_t*)a.h + e, hw);
-        TS d[NC];
+        if (orel < new_rel) ld_words<NC>((const uint32_t*)a.h + e, hw);
+        const long long out_at = a.out ? (long long)s * a.out_stream_stride + (a.o_lo + orel) * a.out_row_stride + (long long)x * C + co : 0;
+        const bool emit = a.out && IDF_OK_AT(a.status, out_at, a.out_elems - (NC - 1));
+        if constexpr (INT) {
+            uint32_t h[NC / 4], h_old[NC / 4], d[NC / 4];
+            act_bytes<NC>((const uint32_t*)m, of_conv && bias ? (const int*)bias + co : nullptr, of_conv ? rnd : 0, of_conv ? shift : 0, h);
+            act_bytes<NC>(hw, nullptr, 0, 0, h_old);
+            uint32_t hn[NC];
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            if (o >= a.o_cut) m[j] = 0;
-            d[j] = m[j] - as_ts(TS(0), hw[j]);
-            n_out += d[j] != (TS)0;
-        }
-        st_words<NC>((uint32_t*)a.h + e, (const uint32_t*)m);
-        st_values<NC>(a.d, e, a.d_elem, d);
-        if (a.out) {
-            const long long i = (long long)s * a.out_stream_stride + o * a.out_row_stride + (long long)x * a.Cout + co;
-            if (IDF_OK_AT(a.status, i, a.out_elems - (NC - 1))) st_values<NC>(a.out, i, E_I8, m);
+            for (int j = 0; j < NC / 4; ++j) {
+                if (orel >= cut_rel) h[j] = 0u;
+                d[j] = sub_bytes(h[j], h_old[j]);
+                n_out += count_bytes(d[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < NC; ++j) hn[j] = (h[j >> 2] >> (8 * (j & 3))) & 0xffu;
+            st_words<NC>((uint32_t*)a.h + e, hn);
+            pass_changes<NC>(mode, dn, orel * G + sg, C, co, Wout, x, a.d, e, d);
+            if (emit) st_bytes<NC>((int8_t*)a.out + out_at, h);
+        } else {
+            float d[NC], h[NC];
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                h[j] = orel >= cut_rel ? 0.f : (float)m[j];
+                d[j] = h[j] - __uint_as_float(hw[j]);
+                n_out += d[j] != 0.f;
+            }
+            st_words<NC>((uint32_t*)a.h + e, (const uint32_t*)h);
+            pass_changes<NC>(mode, dn, orel * G + sg, C, co, Wout, x, a.d, e, d);
+            if (emit) st_values<NC>(a.out, out_at, h);
         }
     }
 }
@@ -360,52 +483,60 @@ __global__ void __launch_bounds__(EAGER_THREADS, 2) eager_tiled_kernel(const __g
         const bool quads = INT && a.wq != nullptr;
         const int n_w = a.Kh * a.Kw * (quads ? a.Cin >> 2 : a.Cin) * a.Cout;
         uint32_t* sw = esm + net.w_at[l];
-        for (int i = tid; i < n_w; i += blockDim.x)
-            sw[i] = quads ? ((const uint32_t*)a.wq)[i] : (INT ? (uint32_t)(int)((const int8_t*)a.w)[i] : ((const uint32_t*)a.w)[i]);
+        const void* src = quads ? a.wq : a.w;
+        for (int i = tid; i < n_w; i += blockDim.x) sw[i] = INT && !quads ? (uint32_t)(int)((const int8_t*)src)[i] : ((const uint32_t*)src)[i];
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int s0 = blockIdx.x * G, Gn = min(G, net.layer[0].S - s0);
-    uint32_t* sd = esm + net.d_at;
     for (int l = 0; l < net.n; ++l) {
         const EagerArgs& a = net.layer[l];
         unsigned int n_in = 0, n_out = 0;
         const bool wide = a.Cout % EAGER_NC == 0;
-        __syncthreads();                                  // the layer below is done (and its changed rows in shared memory are used up)
+        uint32_t *sd = esm + net.d_at[l & 1], *dn = esm + net.d_at[(l + 1) & 1];
+        const int mode = net.d_ring ? EO_RING : (l + 1 == net.n || net.pool[l + 1] ? EO_NONE : (INT && net.layer[l + 1].wq ? EO_QUADS : EO_WORDS));
+        __syncthreads();                                  // the layer below is done
         if (net.pool[l]) {
-            if (wide) eager_pool_units<TS, EAGER_NC>(a, s0, Gn, n_out);
-            else eager_pool_units<TS, 4>(a, s0, Gn, n_out);
+            if (wide) eager_pool_units<TS, EAGER_NC>(a, G, s0, Gn, mode, dn, n_out);
+            else eager_pool_units<TS, 4>(a, G, s0, Gn, mode, dn, n_out);
         } else {
             const bool quads = INT && a.wq != nullptr;
             const int CQ = quads ? a.Cin >> 2 : a.Cin, row_elems = a.Win * a.Cin;
-            const int rows = (int)(a.in_hi - a.in_lo + 1);                      // changed rows below (may be none)
-            for (int r = 0; r < rows; ++r) {
+            const int rows = (int)(a.in_hi - a.in_lo + 1), Win = a.Win, elem = a.din_elem;      // changed rows below (may be none)
+            const bool count = a.in_events != nullptr;
+            const FastDiv by_c(CQ), by_w(Win);
+            const int n = Gn * Win * CQ;
+            // (within a launch the layer below has left its changes in place)
+            for (int r = 0; r < (l == 0 ? rows : 0); ++r) {
                 const long long first = (((a.in_lo + r) % a.cap_in) * a.S + s0) * (long long)row_elems;
                 if (!IDF_OK_AT(a.status, first + (long long)Gn * row_elems - 1, a.in_elems)) continue;
-                uint32_t* dst = sd + r * G * CQ * a.Win;
-                for (int i = tid; i < Gn * a.Win * CQ; i += blockDim.x) {
-                    const int c = i % CQ, t = i / CQ, x = t % a.Win, g = t / a.Win;
+                uint32_t* dst = sd + r * G * CQ * Win;
+                const unsigned char* src = (const unsigned char*)a.din + first * (elem == E_I8 ? 1 : (elem == E_BF16 ? 2 : 4));
+                const bool aligned = ((uintptr_t)src & 3) == 0;
+                for (int i = tid; i < n; i += blockDim.x) {
+                    int c, x;
+                    const int g = by_w.div(by_c.div(i, c), x);
                     uint32_t v;
                     if (quads) {
-                        const unsigned char* p = (const unsigned char*)a.din + first + 4LL * i;
-                        v = ((uintptr_t)p & 3) == 0 ? *(const uint32_t*)p : (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) | ((uint32_t)p[3] << 24);
-                        if (a.in_events) n_in += __popc((((v & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v) & 0x80808080u);
+                        const unsigned char* p = src + 4 * i;
+                        v = aligned ? *(const uint32_t*)p : (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) | ((uint32_t)p[3] << 24);
+                        if (count) n_in += __popc((((v & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v) & 0x80808080u);
                     } else {
-                        if (a.din_elem == E_I8) v = (uint32_t)(int)((const int8_t*)a.din)[first + i];
-                        else if (a.din_elem == E_BF16) v = __float_as_uint(__bfloat162float(((const __nv_bfloat16*)a.din)[first + i]));
-                        else v = ((const uint32_t*)a.din)[first + i];
-                        if (a.in_events) n_in += as_ts(TS(0), v) != TS(0);
+                        if (elem == E_I8) v = (uint32_t)(int)((const int8_t*)src)[i];
+                        else if (elem == E_BF16) v = __float_as_uint(__bfloat162float(((const __nv_bfloat16*)src)[i]));
+                        else v = ((const uint32_t*)src)[i];
+                        if (count) n_in += as_ts(TS(0), v) != TS(0);
                     }
-                    dst[(g * CQ + c) * a.Win + x] = v;
+                    dst[(g * CQ + c) * Win + x] = v;
                 }
             }
-            __syncthreads();
+            if (l == 0) __syncthreads();
             const uint32_t* sw = esm + net.w_at[l];
             if (quads) {
-                if (wide) eager_conv_units<TS, EAGER_NC, INT>(a, sw, sd, G, s0, Gn, n_out);
-                else eager_conv_units<TS, 4, INT>(a, sw, sd, G, s0, Gn, n_out);
+                if (wide) eager_conv_units<TS, EAGER_NC, INT>(a, sw, sd, G, s0, Gn, mode, dn, n_out);
+                else eager_conv_units<TS, 4, INT>(a, sw, sd, G, s0, Gn, mode, dn, n_out);
             } else {
-                if (wide) eager_conv_units<TS, EAGER_NC, false>(a, sw, sd, G, s0, Gn, n_out);
-                else eager_conv_units<TS, 4, false>(a, sw, sd, G, s0, Gn, n_out);
+                if (wide) eager_conv_units<TS, EAGER_NC, false>(a, sw, sd, G, s0, Gn, mode, dn, n_out);
+                else eager_conv_units<TS, 4, false>(a, sw, sd, G, s0, Gn, mode, dn, n_out);
             }
         }
         n_in = __reduce_add_sync(0xffffffffu, n_in);
@@ -460,15 +591,15 @@ bool eager_tiled_words(int is_pool, int int_net, int Win, int Cin, int Cout, int
     const size_t cq = int_net && Cin % 4 == 0 ? Cin / 4 : Cin;
     *w = (size_t)Kh * Kw * cq * Cout;
     *d = (size_t)rows_in * cq * Win;
-    return *w + *d <= EAGER_SMEM_WORDS;
+    return *w + 2 * *d <= EAGER_SMEM_WORDS;
 }
 // As few streams per block as still give every SM its two blocks (a narrow row fills a warp's lanes better with several streams).
 int eager_tiled_group(int S, size_t w, size_t d, size_t limit_words)
 {
-    if (w + d > limit_words) return 0;
+    if (w + 2 * d > limit_words) return 0;               // (two sets of changed rows: a layer's and the next one's)
     int G = (S + 295) / 296;
     if (G > 8) G = 8;
-    while (G > 1 && w + (size_t)G * d > limit_words) --G;
+    while (G > 1 && w + 2 * (size_t)G * d > limit_words) --G;
     return G;
 }
 
