@@ -87,14 +87,14 @@ struct idf_net {
     // depth-first over all layers in one launch (nets whose per-stream state is small): plan made at create
     int fused_ok = 0, fused_G = 0, fused_threads = 0, fused_in_soff = 0;
     size_t fused_smem = 0;
-    std::vector<int> fused_state_soff, fused_rowbuf_soff;
+    std::vector<int> fused_state_soff, fused_rowbuf_soff, fused_w_soff, fused_b_soff;
     double macs_per_row = 0;               // multiply-accumulates one segment of one stream costs (all layers, steady state)
     int eager = 0;                         // emission policy: 0 = once per unit (deferred), 1 = after every segment (eager)
     int eager_tiled = 0, eager_G = 0;      // every layer fits the tiled kernel; streams per block if all fit one launch, else 0
     size_t eager_w_words = 0, eager_d_words = 0;   // shared memory: weights of all layers, most changed rows of a stream
     size_t eager_in_off = 0;               // the pushed segment as words (the input layer's announcement)
     std::vector<LayerPlan> L;
-    size_t workspace_bytes = 0, state_region_off = 0, state_region_bytes = 0, counters_off = 0, status_off = 0;
+    size_t workspace_bytes = 0, state_region_off = 0, state_region_bytes = 0, reset_bytes = 0, counters_off = 0, status_off = 0;
     size_t ring_scratch_off = 0;           // room for a copy of the largest tensor-core layer's ring (row-chunked launches)
     size_t state_bytes_stream = 0;
     unsigned char* ws = nullptr;
@@ -710,7 +710,7 @@ int run_segments_fused(idf_net* net, const void* d_segments, long long n_seg, bo
 {
     const size_t nl = net->L.size();
     // rows complete after this call, layer by layer (the schedule inside the kernel follows the same closed forms)
-    std::vector<long long> in_after(nl), done_after(nl);
+    long long in_after[FUSED_MAX_LAYERS], done_after[FUSED_MAX_LAYERS];
     long long r = net->L[0].rows_in + n_seg;
     for (size_t i = 0; i < nl; ++i) {
         in_after[i] = r;
@@ -738,6 +738,9 @@ int run_segments_fused(idf_net* net, const void* d_segments, long long n_seg, bo
         F.stride_x = P.in_w == 1 ? 1 : P.l.stride; F.pad_x = P.in_w == 1 ? 0 : P.l.pad;
         F.relu = P.l.relu; F.shift = P.l.shift; F.round_bf16 = P.out_elem == E_BF16;
         F.Win = P.in_w; F.Wout = P.out_w; F.ring_rows = P.ring_rows; F.count_events = P.use_sparse; F.out_elem = P.out_elem;
+        F.w_soff = net->fused_w_soff[i]; F.b_soff = net->fused_b_soff[i];
+        F.w_bytes = (int)(P.wq_packed.empty() || P.use_sparse ? P.w_packed.size() : P.wq_packed.size());
+        F.w_src = (long long)(P.wq_packed.empty() || P.use_sparse ? P.w_off : P.wq_off);
         F.state_soff = net->fused_state_soff[i]; F.rowbuf_soff = net->fused_rowbuf_soff[i];
         F.w_off = (long long)(net->dtype == IDF_I8_I32 ? P.w_off : P.w_off / 4);
         F.wq_off = net->dtype == IDF_I8_I32 ? (P.wq_packed.empty() ? -1 : (long long)P.wq_off) : 0;
@@ -1071,6 +1074,17 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                 off = up16(off + (size_t)G * P.out_w * P.out_c * rs);
                 widest = std::max(widest, (size_t)G * P.out_w * P.out_c);
             }
+            // the parameters too, where they are few
+            for (const auto& P : net->L) {
+                // (int layers of four-channel words read those, but only while an input row reaches at most three rows)
+                const bool words = !P.wq_packed.empty() && !P.use_sparse;
+                const size_t wb = words ? P.wq_packed.size() : P.w_packed.size();
+                const bool on_chip = P.l.kind == IDF_CONV && wb <= 16 * 1024 && (!words || P.ring_rows <= 3) && off + wb + (size_t)P.out_c * 4 + 32 <= FUSED_SMEM_LIMIT;
+                net->fused_w_soff.push_back(on_chip ? (int)off : -1);
+                if (on_chip) off = up16(off + wb);
+                net->fused_b_soff.push_back(on_chip && !P.b_packed.empty() ? (int)off : -1);
+                if (on_chip && !P.b_packed.empty()) off = up16(off + (size_t)P.out_c * 4);
+            }
             net->fused_smem = off;
             net->fused_threads = (int)std::min<size_t>(512, std::max<size_t>(64, (widest + 31) / 32 * 32));
             net->fused_ok = off <= FUSED_SMEM_LIMIT;
@@ -1095,6 +1109,12 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
         off = align_up(off + P.state_bytes_all);
     }
     net->state_region_bytes = off - net->state_region_off;
+    // (behind the state, so that a reset is one memset)
+    net->counters_off = off;
+    off = align_up(off + net->L.size() * sizeof(unsigned long long));
+    net->status_off = off;
+    off = align_up(off + sizeof(unsigned int));
+    net->reset_bytes = off - net->state_region_off;
     if (net->eager) { net->eager_in_off = off; off = align_up(off + (size_t)net->n_streams * net->in_w * net->in_c * 4); }
     for (size_t i = 0; i + 1 < net->L.size(); ++i) {
         LayerPlan& P = net->L[i];
@@ -1112,11 +1132,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
             if (P.l.kind == IDF_CONV && P.tc.ok) biggest = std::max(biggest, P.state_bytes_all);
         if (biggest) { net->ring_scratch_off = off; off = align_up(off + biggest); }
     }
-    net->counters_off = off;
-    off = align_up(off + net->L.size() * sizeof(unsigned long long));
-    net->status_off = off;
-    off = align_up(off + sizeof(unsigned int));
-    net->workspace_bytes = off;
+    net->workspace_bytes = off + 1024;      // (a group of positions may reach a little past the last row of a buffer)
     *out = net;
     return IDF_OK;
 }
@@ -1201,9 +1217,7 @@ int idf_stream_reset(idf_net* net)
     if (!net) return fail(IDF_ERR_ARG, "net must not be NULL");
     if (net->phase == CREATED) return fail(IDF_ERR_STATE, "reset before stream_open");
     for (auto& P : net->L) { P.rows_in = 0; P.rows_done = 0; P.tc_launches = 0; P.pending = 0; P.e_hi = -1; }
-    cudaError_t e = cudaMemsetAsync(net->ws + net->status_off, 0, sizeof(unsigned int), net->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(net->ws + net->state_region_off, 0, net->state_region_bytes, net->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(net->ws + net->counters_off, 0, net->L.size() * sizeof(unsigned long long), net->stream);
+    cudaError_t e = cudaMemsetAsync(net->ws + net->state_region_off, 0, net->reset_bytes, net->stream);
     if (e != cudaSuccess) { net->phase = CREATED; return fail(IDF_ERR_CUDA, "stream_reset: %s", cudaGetErrorString(e)); }
     net->phase = OPEN;
     net->launches = 0;

@@ -31,6 +31,23 @@ __device__ __forceinline__ bool bounds_ok(unsigned int* status, long long idx, l
 // process-wide debug switches (bits of idf_debug_flag), set through idf_set_debug_flags
 unsigned debug_flags();
 
+#ifdef __CUDACC__
+// Launch of a kernel that begins with griddepcontrol.wait: it may be scheduled while its predecessor in the stream drains.  (Every
+// kernel launched this way waits before it touches anything but parameters, so completion stays ordered along the whole stream.)
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = (debug_flags() & 8u) ? 0 : 1;      // 8: IDF_DEBUG_NO_PDL
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+#endif
+
 inline size_t elem_size(int e) { return e == E_F32 || e == E_I32 ? 4 : (e == E_BF16 ? 2 : 1); }
 
 // How one conv layer advances by a block of input rows.  All row indices are absolute
@@ -150,6 +167,9 @@ struct FusedLayer {
     int Cin, Cout, Kh, Kw, stride, pad, stride_x, pad_x, relu, shift, round_bf16, Win, Wout, ring_rows;
     int count_events;      // the layer reports its input events (sparse-path layers)
     int out_elem;          // element type of the rows the layer emits (pool state in global memory has this type)
+    int w_soff, b_soff, w_bytes;   // shared memory, in bytes: the layer's weights (w_bytes of them, in the form the kernel reads) and bias, or -1: they are
+                           // read from global memory
+    long long w_src;       // where they come from: BYTE offset from FusedArgs::weights
     int state_soff, rowbuf_soff;   // shared memory, in bytes: ring [slot][G][Wout][Cout] words or pool row [G][Wout][C]; emitted row [G][Wout][Cout]
     long long w_off;       // weights [Kh][Kw][Cin][Cout]: element offset from FusedArgs::weights (fp32 or int8 elements)
     long long wq_off;      // int nets: the same weights, four input channels to a word [Kh][Kw][Cin/4][Cout], BYTE offset; -1: none

@@ -106,7 +106,7 @@ __device__ bool fused_feed(const FusedArgs& a, int i, const typename RowOf<TS>::
         return second;
     }
     // conv: Eq. 4 for every event of the row, tap by tap, then Eq. 2-3 for the row this input row completes
-    const TS* __restrict__ bias = L.bias_off >= 0 ? (const TS*)((const unsigned char*)a.weights + L.bias_off) : nullptr;
+    const TS* bias = L.bias_off < 0 ? nullptr : L.b_soff >= 0 ? (const TS*)(smem + L.b_soff) : (const TS*)((const unsigned char*)a.weights + L.bias_off);
     TS* ring = (TS*)(smem + L.state_soff);
     const int row_elems = L.Wout * L.Cout;
     // taps ky = ph, ph + s, ... < Kh; tap j reaches the row j below the newest one (if that many rows exist)
@@ -117,8 +117,8 @@ __device__ bool fused_feed(const FusedArgs& a, int i, const typename RowOf<TS>::
     const bool quads = (L.Cin & 3) == 0 && !L.count_events && L.wq_off >= 0;
     if (nt <= FUSED_TAPS && quads) {
         // four input channels at a time (dp4a / four FMAs), the input fetched once for all taps
-        const int* __restrict__ wq = (const int*)((const unsigned char*)a.weights + L.wq_off);     // int nets: [ky][kx][ci/4][co] packed words
-        const float* __restrict__ wf = (const float*)a.weights + L.w_off;                          // float nets: [ky][kx][ci][co]
+        const int* wq = L.w_soff >= 0 ? (const int*)(smem + L.w_soff) : (const int*)((const unsigned char*)a.weights + L.wq_off);     // int nets: [ky][kx][ci/4][co] packed words
+        const float* wf = L.w_soff >= 0 ? (const float*)(smem + L.w_soff) : (const float*)a.weights + L.w_off;                        // float nets: [ky][kx][ci][co]
         for (int e = threadIdx.x; e < G * row_elems; e += blockDim.x) {
             const int co = e % L.Cout, t = e / L.Cout, x = t % L.Wout, g = t / L.Wout;
             TS acc[FUSED_TAPS] = {0, 0, 0};
@@ -131,15 +131,15 @@ __device__ bool fused_feed(const FusedArgs& a, int i, const typename RowOf<TS>::
                         const int v = ((const int*)ip)[c4];
 #pragma unroll
                         for (int j = 0; j < FUSED_TAPS; ++j)
-                            if (j < nt) acc[j] = __dp4a(v, __ldg(wq + (((k.ph + j * L.stride) * L.Kw + kx) * Cq + c4) * L.Cout + co), acc[j]);
+                            if (j < nt) acc[j] = __dp4a(v, wq[(((k.ph + j * L.stride) * L.Kw + kx) * Cq + c4) * L.Cout + co], acc[j]);
                     } else {
                         const float4 v = ((const float4*)ip)[c4];
 #pragma unroll
                         for (int j = 0; j < FUSED_TAPS; ++j)
                             if (j < nt) {
                                 const float* wp = wf + (((k.ph + j * L.stride) * L.Kw + kx) * L.Cin + 4 * c4) * L.Cout + co;
-                                acc[j] += __ldg(wp) * v.x; acc[j] += __ldg(wp + L.Cout) * v.y;
-                                acc[j] += __ldg(wp + 2 * L.Cout) * v.z; acc[j] += __ldg(wp + 3 * L.Cout) * v.w;
+                                acc[j] += wp[0] * v.x; acc[j] += wp[L.Cout] * v.y;
+                                acc[j] += wp[2 * L.Cout] * v.z; acc[j] += wp[3 * L.Cout] * v.w;
                             }
                     }
                 }
@@ -160,7 +160,7 @@ __device__ bool fused_feed(const FusedArgs& a, int i, const typename RowOf<TS>::
             }
         }
     } else {
-        const TW* __restrict__ w = (const TW*)a.weights + L.w_off;
+        const TW* w = L.w_soff >= 0 ? (const TW*)(smem + L.w_soff) : (const TW*)a.weights + L.w_off;
         for (int e = threadIdx.x; e < G * row_elems; e += blockDim.x) {
             const int co = e % L.Cout, t = e / L.Cout, x = t % L.Wout, g = t / L.Wout;
             for (int j = 0; j < nt; ++j) {
@@ -226,7 +226,7 @@ __device__ void fused_cascade(const FusedArgs& a, int i, unsigned char* smem, La
 }
 
 template <typename TS>
-__global__ void __launch_bounds__(512) depth_first_kernel(const FusedArgs a)
+__global__ void __launch_bounds__(512) depth_first_kernel(const __grid_constant__ FusedArgs a)
 {
     typedef typename RowOf<TS>::T TR;
     extern __shared__ __align__(16) unsigned char fsmem[];
@@ -242,37 +242,63 @@ __global__ void __launch_bounds__(512) depth_first_kernel(const FusedArgs a)
     }
     int out_row = a.out_row0;
     if (threadIdx.x < FUSED_MAX_LAYERS) ev_local[threadIdx.x] = 0;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // ---- the group's rolling state comes on chip
+    // parameters come on chip while the previous kernel of the stream still runs: they do not depend on it
     for (int i = 0; i < a.n_layers; ++i) {
         const FusedLayer& L = a.layer[i];
-        const int row_elems = L.Wout * L.Cout;
-        if (L.kind == 0) {
-            TS* st = (TS*)(fsmem + L.state_soff);
-            const TS* gr = (const TS*)L.state;
-            for (int e = threadIdx.x; e < L.ring_rows * G * row_elems; e += blockDim.x) {
+        if (L.w_soff >= 0) {
+            const uint32_t* src = (const uint32_t*)((const unsigned char*)a.weights + L.w_src);
+            for (int e = threadIdx.x; e < (L.w_bytes + 3) / 4; e += blockDim.x) ((uint32_t*)(fsmem + L.w_soff))[e] = src[e];
+        }
+        if (L.b_soff >= 0)
+            for (int e = threadIdx.x; e < L.Cout; e += blockDim.x)
+                ((uint32_t*)(fsmem + L.b_soff))[e] = ((const uint32_t*)((const unsigned char*)a.weights + L.bias_off))[e];
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // ---- the group's rolling state and the first segment come on chip: one run over the elements of all layers, so that a launch for a
+    // single segment pays the latency of one load, not of one per layer
+    TR* inrow = (TR*)(fsmem + a.in_soff);
+    const int in_elems = a.in_w * a.in_c;
+    {
+        int total = G * in_elems * (a.n_seg > 0);
+        for (int i = 0; i < a.n_layers; ++i) {
+            const FusedLayer& L = a.layer[i];
+            total += (L.kind == 0 ? L.ring_rows : 1) * G * L.Wout * L.Cout;
+        }
+        for (int t = threadIdx.x; t < total; t += blockDim.x) {
+            int e = t, i = 0;
+            for (; i < a.n_layers; ++i) {
+                const FusedLayer& L = a.layer[i];
+                const int n = (L.kind == 0 ? L.ring_rows : 1) * G * L.Wout * L.Cout;
+                if (e < n) break;
+                e -= n;
+            }
+            if (i == a.n_layers) {
+                const long long at = (long long)g0 * in_elems + e;
+                if (IDF_OK_AT(a.status, at, (long long)a.n_seg * a.S * in_elems)) inrow[e] = load_elem<TR>(a.in, at, a.in_elem);
+                continue;
+            }
+            const FusedLayer& L = a.layer[i];
+            const int row_elems = L.Wout * L.Cout;
+            if (L.kind == 0) {
                 const int slot = e / (G * row_elems), q = e - slot * (G * row_elems);
                 const long long at = ((long long)slot * a.S + g0) * row_elems + q;
-                if (IDF_OK_AT(a.status, at, (long long)L.ring_rows * a.S * row_elems)) st[e] = gr[at];
-            }
-        } else {
-            TR* st = (TR*)(fsmem + L.state_soff);
-            for (int e = threadIdx.x; e < G * row_elems; e += blockDim.x) {
+                if (IDF_OK_AT(a.status, at, (long long)L.ring_rows * a.S * row_elems)) ((TS*)(fsmem + L.state_soff))[e] = ((const TS*)L.state)[at];
+            } else {
                 const long long at = (long long)g0 * row_elems + e;
-                if (IDF_OK_AT(a.status, at, (long long)a.S * row_elems)) st[e] = load_elem<TR>(L.state, at, L.out_elem);
+                if (IDF_OK_AT(a.status, at, (long long)a.S * row_elems)) ((TR*)(fsmem + L.state_soff))[e] = load_elem<TR>(L.state, at, L.out_elem);
             }
         }
     }
     __syncthreads();
     // ---- segments, one at a time, each through every layer it can reach
-    TR* inrow = (TR*)(fsmem + a.in_soff);
-    const int in_elems = a.in_w * a.in_c;
     for (int seg = 0; seg < a.n_seg; ++seg) {
-        for (int e = threadIdx.x; e < G * in_elems; e += blockDim.x) {
-            const long long at = ((long long)seg * a.S + g0) * in_elems + e;
-            if (IDF_OK_AT(a.status, at, (long long)a.n_seg * a.S * in_elems)) inrow[e] = load_elem<TR>(a.in, at, a.in_elem);
+        if (seg > 0) {
+            for (int e = threadIdx.x; e < G * in_elems; e += blockDim.x) {
+                const long long at = ((long long)seg * a.S + g0) * in_elems + e;
+                if (IDF_OK_AT(a.status, at, (long long)a.n_seg * a.S * in_elems)) inrow[e] = load_elem<TR>(a.in, at, a.in_elem);
+            }
+            __syncthreads();
         }
-        __syncthreads();
         if (fused_feed<TS>(a, 0, inrow, fsmem, clk[0], G, ev_local)) fused_cascade<TS>(a, 0, fsmem, clk, G, g0, out_row, ev_local);
     }
     // ---- end of input: rows that wait only for bottom zero padding are complete as they stand, in depth order
@@ -282,7 +308,7 @@ __global__ void __launch_bounds__(512) depth_first_kernel(const FusedArgs a)
             const FusedLayer& L = a.layer[i];
             if (L.kind != 0) continue;                   // (an unpaired pooling row is dropped)
             const int row_elems = L.Wout * L.Cout;
-            const TS* bias = L.bias_off >= 0 ? (const TS*)((const unsigned char*)a.weights + L.bias_off) : nullptr;
+            const TS* bias = L.bias_off < 0 ? nullptr : L.b_soff >= 0 ? (const TS*)(fsmem + L.b_soff) : (const TS*)((const unsigned char*)a.weights + L.bias_off);
             for (int n = 0; n < L.n_flush; ++n) {
                 TS* ring = (TS*)(fsmem + L.state_soff);
                 TR* rowbuf = (TR*)(fsmem + L.rowbuf_soff);
@@ -337,8 +363,7 @@ cudaError_t launch_depth_first(const FusedArgs& a, int int_net, int threads, siz
         if (e != cudaSuccess) return e;
         attr_set[int_net ? 1 : 0][dev] = true;
     }
-    kf<<<grid, threads, smem_bytes, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kf, grid, (unsigned)threads, smem_bytes, st, a);
 }
 
 }  // namespace idf

@@ -57,6 +57,7 @@ template <typename TI, typename TW, typename TS, typename TO>
 __global__ void __launch_bounds__(256) conv_rows_kernel(ConvArgs a, long long int_begin, long long int_end, unsigned edge_blocks)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const TI* __restrict__ in = (const TI*)a.in;
     const TW* __restrict__ w = (const TW*)a.w;
     const TS* __restrict__ bias = (const TS*)a.bias;
@@ -158,6 +159,7 @@ template <typename TS, typename TO>
 __global__ void __launch_bounds__(256) conv_flush_kernel(ConvArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const TS* __restrict__ bias = (const TS*)a.bias;
     TS* ring = (TS*)a.ring;
     TO* out = (TO*)a.out;
@@ -194,8 +196,7 @@ static cudaError_t launch_rows(const ConvArgs& a, cudaStream_t st)
         if (tot <= 0) return cudaSuccess;
         long long blocks = (tot + 255) / 256;
         if (blocks > 148LL * 64) blocks = 148LL * 64;
-        conv_flush_kernel<TS, TO><<<(unsigned)blocks, 256, 0, st>>>(a);
-        return cudaGetLastError();
+        return launch_pdl(conv_flush_kernel<TS, TO>, (unsigned)blocks, 256, 0, st, a);
     }
     const long long total = (long long)a.ring_rows * a.S * a.Wout * a.Cout;
     if (total == 0 || a.o_end <= a.o_begin) return cudaSuccess;
@@ -213,8 +214,7 @@ static cudaError_t launch_rows(const ConvArgs& a, cudaStream_t st)
     } else {
         int_begin = int_end = 0;
     }
-    conv_rows_kernel<TI, TW, TS, TO><<<(unsigned)(blocks + int_blocks), 256, 0, st>>>(a, int_begin, int_end, (unsigned)blocks);
-    return cudaGetLastError();
+    return launch_pdl(conv_rows_kernel<TI, TW, TS, TO>, (unsigned)(blocks + int_blocks), 256, 0, st, a, int_begin, int_end, (unsigned)blocks);
 }
 
 cudaError_t launch_conv_simple(const ConvArgs& a, int dtype, cudaStream_t st)
@@ -260,6 +260,7 @@ template <typename TI, typename TW, typename TS, typename TO, bool RING_IN_SMEM>
 __global__ void __launch_bounds__(SPARSE_MAX_THREADS) conv_sparse_kernel(ConvArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ short ev_x[SPARSE_MAX_EVENTS], ev_ci[SPARSE_MAX_EVENTS];   // position and channel of the event
     __shared__ TS ev_val[SPARSE_MAX_EVENTS];
@@ -524,11 +525,10 @@ static cudaError_t launch_sparse_t(const ConvArgs& a, cudaStream_t st)
         auto k = conv_sparse_kernel<TI, TW, TS, TO, true>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes);
         if (e != cudaSuccess) return e;
-        k<<<a.S, nthr, ring_bytes, st>>>(a);
+        return launch_pdl(k, a.S, nthr, ring_bytes, st, a);
     } else {
-        conv_sparse_kernel<TI, TW, TS, TO, false><<<a.S, nthr, 0, st>>>(a);
+        return launch_pdl(conv_sparse_kernel<TI, TW, TS, TO, false>, a.S, nthr, 0, st, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_conv_sparse(const ConvArgs& a, int dtype, cudaStream_t st)
@@ -555,6 +555,7 @@ __global__ void __launch_bounds__(256) unfold_rows_kernel(const T* __restrict__ 
                                                           long long in_elems, unsigned int* status)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int V = 16 / (int)sizeof(T);
     const int vecs = kpad / V;
     const long long total = n_pos * vecs;
@@ -613,6 +614,7 @@ __global__ void __launch_bounds__(256) unfold_rows_staged_kernel(const T* __rest
                                                                  long long in_elems, unsigned int* status)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __shared__ __align__(16) unsigned char raw[UNFOLD_ROW_BYTES];
     constexpr int V = 16 / (int)sizeof(T);
     const int vecs = kpad / V;
@@ -655,24 +657,22 @@ cudaError_t launch_unfold(const ConvArgs& a, int n_rows, int kpad, void* out, cu
         n_rs <= 0x7fffffffLL && (long long)a.Wout * (kpad * esize / 16) <= 0x7fffffffLL) {
         const unsigned grid = (unsigned)(n_rs < 148LL * 8 ? n_rs : 148LL * 8);
         if (a.in_elem == E_BF16)
-            unfold_rows_staged_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.in, (__nv_bfloat16*)out, (int)n_rs, a.Win, a.Wout,
+            return launch_pdl(unfold_rows_staged_kernel<__nv_bfloat16>, grid, 256, 0, st, (const __nv_bfloat16*)a.in, (__nv_bfloat16*)out, (int)n_rs, a.Win, a.Wout,
                                                                          a.Cin, a.Kw, a.stride_x, a.pad_x, kpad, a.in_elems, a.status);
         else if (a.in_elem == E_I8)
-            unfold_rows_staged_kernel<int8_t><<<grid, 256, 0, st>>>((const int8_t*)a.in, (int8_t*)out, (int)n_rs, a.Win, a.Wout, a.Cin, a.Kw,
+            return launch_pdl(unfold_rows_staged_kernel<int8_t>, grid, 256, 0, st, (const int8_t*)a.in, (int8_t*)out, (int)n_rs, a.Win, a.Wout, a.Cin, a.Kw,
                                                                   a.stride_x, a.pad_x, kpad, a.in_elems, a.status);
         else
             return cudaErrorInvalidValue;
-        return cudaGetLastError();
     }
     if (a.in_elem == E_BF16)
-        unfold_rows_kernel<__nv_bfloat16><<<(unsigned)blocks, 256, 0, st>>>((const __nv_bfloat16*)a.in, (__nv_bfloat16*)out, n_pos,
+        return launch_pdl(unfold_rows_kernel<__nv_bfloat16>, (unsigned)blocks, 256, 0, st, (const __nv_bfloat16*)a.in, (__nv_bfloat16*)out, n_pos,
                                                                           a.Win, a.Wout, a.Cin, a.Kw, a.stride_x, a.pad_x, kpad, a.in_elems, a.status);
     else if (a.in_elem == E_I8)
-        unfold_rows_kernel<int8_t><<<(unsigned)blocks, 256, 0, st>>>((const int8_t*)a.in, (int8_t*)out, n_pos, a.Win, a.Wout,
+        return launch_pdl(unfold_rows_kernel<int8_t>, (unsigned)blocks, 256, 0, st, (const int8_t*)a.in, (int8_t*)out, n_pos, a.Win, a.Wout,
                                                                    a.Cin, a.Kw, a.stride_x, a.pad_x, kpad, a.in_elems, a.status);
     else
         return cudaErrorInvalidValue;
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -689,6 +689,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) pool_rows_kernel(PoolArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const T* __restrict__ in = (const T*)a.in;
     T* state = (T*)a.state;
     T* out = (T*)a.out;
@@ -733,6 +734,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) pool_rows_vec_kernel(PoolArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int V = 16 / (int)sizeof(T);
     const T* __restrict__ in = (const T*)a.in;
     T* state = (T*)a.state;
@@ -795,13 +797,11 @@ static cudaError_t launch_pool_t(const PoolArgs& a, cudaStream_t st)
         const long long tv = (a.o_end - a.o_begin) * a.S * a.Wout * (a.C / V);
         long long blocks = (tv + 255) / 256;
         if (blocks > 148LL * 64) blocks = 148LL * 64;
-        pool_rows_vec_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(a);
-        return cudaGetLastError();
+        return launch_pdl(pool_rows_vec_kernel<T>, (unsigned)blocks, 256, 0, st, a);
     }
     long long blocks = (total + 255) / 256;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
-    pool_rows_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(pool_rows_kernel<T>, (unsigned)blocks, 256, 0, st, a);
 }
 
 cudaError_t launch_pool(const PoolArgs& a, cudaStream_t st)
@@ -828,6 +828,7 @@ template <typename TI, typename TS>
 __global__ void __launch_bounds__(256) avg_rows_kernel(AvgArgs a)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const TI* __restrict__ in = (const TI*)a.in;
     TS* sum = (TS*)a.sum;
     const long long total = (long long)a.S * a.C;
@@ -854,12 +855,11 @@ cudaError_t launch_avg(const AvgArgs& a, cudaStream_t st)
     long long blocks = (total + 255) / 256;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
     switch (a.elem) {
-        case E_F32: avg_rows_kernel<float, float><<<(unsigned)blocks, 256, 0, st>>>(a); break;
-        case E_BF16: avg_rows_kernel<__nv_bfloat16, float><<<(unsigned)blocks, 256, 0, st>>>(a); break;
-        case E_I8: avg_rows_kernel<int8_t, int><<<(unsigned)blocks, 256, 0, st>>>(a); break;
+        case E_F32: return launch_pdl(avg_rows_kernel<float, float>, (unsigned)blocks, 256, 0, st, a);
+        case E_BF16: return launch_pdl(avg_rows_kernel<__nv_bfloat16, float>, (unsigned)blocks, 256, 0, st, a);
+        case E_I8: return launch_pdl(avg_rows_kernel<int8_t, int>, (unsigned)blocks, 256, 0, st, a);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace idf

@@ -156,6 +156,13 @@ class Net:
         self._ws = None
         self.n_layers = n
         self._avg_sink = int(self._layers[n - 1].kind) == GLOBAL_AVG
+        # what the push calls need each time, looked up once (a push of one segment takes a few microseconds in all)
+        L = lib()
+        self._push, self._push_last, self._reset = L.idf_stream_push, L.idf_stream_push_last, L.idf_stream_reset
+        self._act_dtype, self._out_dtype = self.act_torch_dtype, self.out_torch_dtype
+        self._seg_shape = (self.n_streams, self.in_w, self.in_c)
+        self._em, self._tot = ctypes.c_int(), ctypes.c_longlong()
+        self._em_ref, self._tot_ref = ctypes.byref(self._em), ctypes.byref(self._tot)
 
     # -- queries ---------------------------------------------------------------------------------
     @property
@@ -219,32 +226,37 @@ class Net:
 
     def reset(self):
         """New streams on the workspace of the last open(): state and counters to zero, parameters stay."""
-        _check(lib().idf_stream_reset(self._h))
+        rc = self._reset(self._h)
+        if rc:
+            _check(rc)
 
     def alloc_out(self, in_rows: int, device="cuda:0") -> torch.Tensor:
         _, w, c = self.out_shape(in_rows)
         r = int(lib().idf_out_rows_needed(self._h, in_rows))
         return torch.zeros((self.n_streams, max(r, 1), w, c), dtype=self.out_torch_dtype, device=device)
 
+    def _check_io(self, segments: torch.Tensor, out: torch.Tensor):
+        assert segments.is_cuda and segments.is_contiguous() and out.is_cuda and out.is_contiguous()
+        assert segments.dtype is self._act_dtype and out.dtype is self._out_dtype
+        shape = segments.shape
+        assert shape[1:] == self._seg_shape, shape
+        return shape[0], out.shape[1]
+
     def push(self, segments: torch.Tensor, out: torch.Tensor) -> int:
         """segments: device tensor [n_seg][n_streams][in_w][in_c] in the activation type."""
-        assert segments.is_cuda and segments.is_contiguous() and out.is_cuda and out.is_contiguous()
-        assert segments.dtype == self.act_torch_dtype and out.dtype == self.out_torch_dtype
-        assert tuple(segments.shape[1:]) == (self.n_streams, self.in_w, self.in_c), segments.shape
-        em = ctypes.c_int()
-        _check(lib().idf_stream_push(self._h, segments.data_ptr(), segments.shape[0], out.data_ptr(), out.shape[1],
-                                     ctypes.byref(em)))
-        return int(em.value)
+        n, cap = self._check_io(segments, out)
+        rc = self._push(self._h, segments.data_ptr(), n, out.data_ptr(), cap, self._em_ref)
+        if rc:
+            _check(rc)
+        return self._em.value
 
     def push_last(self, segments: torch.Tensor, out: torch.Tensor) -> int:
         """The last segments and the end of input in one call; returns the total number of output rows."""
-        assert segments.is_cuda and segments.is_contiguous() and out.is_cuda and out.is_contiguous()
-        assert segments.dtype == self.act_torch_dtype and out.dtype == self.out_torch_dtype
-        assert tuple(segments.shape[1:]) == (self.n_streams, self.in_w, self.in_c), segments.shape
-        tot = ctypes.c_longlong()
-        _check(lib().idf_stream_push_last(self._h, segments.data_ptr(), segments.shape[0], out.data_ptr(), out.shape[1],
-                                          ctypes.byref(tot)))
-        return int(tot.value)
+        n, cap = self._check_io(segments, out)
+        rc = self._push_last(self._h, segments.data_ptr(), n, out.data_ptr(), cap, self._tot_ref)
+        if rc:
+            _check(rc)
+        return self._tot.value
 
     def set_out_base(self, first_row: int):
         """Later output rows are written at index (row - first_row) of the output buffer; see idf_stream_set_out_base."""
@@ -278,7 +290,7 @@ class Net:
         _check(lib().idf_state_restore(self._h, snapshot.data_ptr(), snapshot.numel()))
 
     def close(self):
-        if self._h:
+        if getattr(self, "_h", None):
             lib().idf_net_destroy(self._h)
             self._h = None
 
