@@ -738,6 +738,7 @@ int run_segments_fused(idf_net* net, const void* d_segments, long long n_seg, bo
         F.stride_x = P.in_w == 1 ? 1 : P.l.stride; F.pad_x = P.in_w == 1 ? 0 : P.l.pad;
         F.relu = P.l.relu; F.shift = P.l.shift; F.round_bf16 = P.out_elem == E_BF16;
         F.Win = P.in_w; F.Wout = P.out_w; F.ring_rows = P.ring_rows; F.count_events = P.use_sparse; F.out_elem = P.out_elem;
+        F.m_cout = 0xffffffffu / (unsigned)P.out_c + 1u; F.m_wout = 0xffffffffu / (unsigned)P.out_w + 1u;
         F.w_soff = net->fused_w_soff[i]; F.b_soff = net->fused_b_soff[i];
         F.w_bytes = (int)(P.wq_packed.empty() || P.use_sparse ? P.w_packed.size() : P.wq_packed.size());
         F.w_src = (long long)(P.wq_packed.empty() || P.use_sparse ? P.w_off : P.wq_off);

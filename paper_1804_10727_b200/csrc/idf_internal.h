@@ -169,6 +169,7 @@ struct FusedLayer {
     int out_elem;          // element type of the rows the layer emits (pool state in global memory has this type)
     int w_soff, b_soff, w_bytes;   // shared memory, in bytes: the layer's weights (w_bytes of them, in the form the kernel reads) and bias, or -1: they are
                            // read from global memory
+    unsigned int m_cout, m_wout;   // 0xffffffff / Cout + 1 and the same of Wout
     long long w_src;       // where they come from: BYTE offset from FusedArgs::weights
     int state_soff, rowbuf_soff;   // shared memory, in bytes: ring [slot][G][Wout][Cout] words or pool row [G][Wout][C]; emitted row [G][Wout][Cout]
     long long w_off;       // weights [Kh][Kw][Cin][Cout]: element offset from FusedArgs::weights (fp32 or int8 elements)
