@@ -47,6 +47,7 @@ struct LayerPlan {
     long long tc_launches = 0;
     std::vector<unsigned char> wq_packed;      // int nets, Cin % 4 == 0: [Kh][Kw][Cin/4][Cout] words of four int8 (all-layers launch)
     size_t wq_off = 0;
+    TimePlan time;                             // 1D layers on the tensor cores (time.ok; weights: wtc_packed)
     WinPlan win;                               // thin layers: the window kernel (win.ok)
     std::vector<unsigned char> wwin_packed;    // its banded weight matrix
     size_t wwin_off = 0;
@@ -237,6 +238,10 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
         ce = cudaErrorNotSupported;
         if (P.win.ok && n_in > 0) {
             ce = launch_conv_win(a, P.win, net->dtype, P.w_map_win, P.use_sparse, net->stream);
+            if (ce == cudaSuccess) P.tc_launches += 1;
+        }
+        if (ce == cudaErrorNotSupported && P.time.ok && P.tc.ok && n_in > 0) {
+            ce = launch_conv_time(a, P.time, net->dtype, net->ws + P.wtc_off, net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
         if (ce == cudaErrorNotSupported && P.tc.ok && !P.use_sparse && n_in > 0) {
@@ -787,7 +792,7 @@ const char* idf_last_error(void) { return g_err.c_str(); }
 
 int idf_set_debug_flags(unsigned int flags)
 {
-    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED | IDF_DEBUG_NO_TILED_EAGER))
+    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED | IDF_DEBUG_NO_TILED_EAGER | IDF_DEBUG_NO_TIME_TILES))
         return fail(IDF_ERR_ARG, "unknown debug flag in 0x%x", flags);
     g_debug_flags.store(flags, std::memory_order_relaxed);
     return IDF_OK;
@@ -924,6 +929,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                         planned = plan_as(x_win, g * l.cin, x_kw, 1, x_pad, pair);
                 }
                 if (!planned) { g = 1; shift = 0; planned = plan_as(w, l.cin, l.kw, sx, px, 0); }
+                if (planned && w == 1 && !(debug_flags() & IDF_DEBUG_NO_TIME_TILES)) time_make_plan(spec->dtype, l.cin, l.cout, l.kh, l.stride, &P.time);
                 if (planned) {
                     const size_t tap_elems = (size_t)l.cout * P.x_cin;
                     P.wtc_packed.assign((size_t)l.kh * P.x_kw * tap_elems * es, 0);

@@ -245,6 +245,15 @@ void win_pack_weights(const WinPlan& p, int dtype, const void* w, int Cin, int C
 int win_encode_weights(const WinPlan& p, int dtype, const void* d_w, void* map_out);
 cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, const void* w_map, int count_events, cudaStream_t st);
 
+// Static part of the plan of the 1D kernel (time rows x streams as the M dimension); tile sizes are chosen per launch.
+struct TimePlan {
+    int ok = 0;
+    int swb = 0, KB = 0, n_kb = 0;   // bytes and input channels of a K-block row, K blocks
+};
+bool time_make_plan(int dtype, int Cin, int Cout, int Kh, int stride, TimePlan* p);
+// d_w: the layer's tensor-core weights [tap slot][Cout][Cin] (tc_weight_slot)
+cudaError_t launch_conv_time(const ConvArgs& a, const TimePlan& p, int dtype, const void* d_w, cudaStream_t st);
+
 // x-unfold: out[row][s][x'][kx*Cin + ci] = in[row][s][x'*stride_x - pad_x + kx][ci] (0 outside the row or
 // beyond Kw*Cin), kpad channels per position, in the activation type
 cudaError_t launch_unfold(const ConvArgs& a, int n_rows, int kpad, void* out, cudaStream_t st);

@@ -83,16 +83,6 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t 
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-__device__ __forceinline__ void st_global_v4(void* p, const uint32_t* v)
-{
-    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
-}
-__device__ __forceinline__ void st_global_32(void* p, const uint32_t* v, int wide)
-{
-    if (wide) st_global_v8(p, *(const uint32_t(*)[8])v);
-    else { st_global_v4(p, v); st_global_v4((unsigned char*)p + 16, v + 4); }
-}
-
 // Walks the steps this CTA takes.  A work item is a tile of 128 windows and the steps [a0, a0 + na), then from b0 on (n in all).
 struct WinWalk {
     int it, i, n, a0, na, b0, tile;
@@ -123,39 +113,6 @@ struct WinWalk {
     }
 };
 
-template <int OUT>
-__device__ __forceinline__ void win_emit16f(const uint32_t* v, const float* bias_c, int relu, unsigned char* dst, int wide)
-{
-    float f[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
-    if (bias_c) {
-#pragma unroll
-        for (int j4 = 0; j4 < 4; ++j4) {
-            const float4 b4 = ((const float4*)bias_c)[j4];
-            f[4 * j4] += b4.x; f[4 * j4 + 1] += b4.y; f[4 * j4 + 2] += b4.z; f[4 * j4 + 3] += b4.w;
-        }
-    }
-    if (OUT == E_BF16) {
-        uint32_t pk[8];
-        if (relu) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
-        }
-        st_global_32(dst, pk, wide);
-    } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t w[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(relu ? fmaxf(f[8 * h + j], 0.f) : f[8 * h + j]);
-            st_global_32(dst + 32 * h, w, wide);
-        }
-    }
-}
 // AX 0: a window runs along x; 1: along the rows (1D nets).  RWT: words of a run of a 3-row layer, known at compile time
 // (the whole window is then fetched one step ahead and leaves in 16-byte stores), or 0.
 template <int DT, int AX, int RWT>
@@ -483,11 +440,11 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                             if (hi) st_global_v4(d1, pk + 4);
                         }
                     } else if (a.out_elem == E_BF16) {
-                        if (lo) win_emit16f<E_BF16>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
-                        if (hi) win_emit16f<E_BF16>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
+                        if (lo) emit16f<E_BF16>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
+                        if (hi) emit16f<E_BF16>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
                     } else {
-                        if (lo) win_emit16f<E_F32>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
-                        if (hi) win_emit16f<E_F32>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
+                        if (lo) emit16f<E_F32>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
+                        if (hi) emit16f<E_F32>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
                     }
                 }
                 first = k - n_chunk;
@@ -537,9 +494,9 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                         pack_i8<16>(v, (const int*)b, a.relu, a.shift, pk);
                         st_global_v4(out + e, pk);
                     } else if (a.out_elem == E_BF16) {
-                        win_emit16f<E_BF16>(v, (const float*)b, a.relu, out + 2 * e, a.out_wide);
+                        emit16f<E_BF16>(v, (const float*)b, a.relu, out + 2 * e, a.out_wide);
                     } else {
-                        win_emit16f<E_F32>(v, (const float*)b, a.relu, out + 4 * e, a.out_wide);
+                        emit16f<E_F32>(v, (const float*)b, a.relu, out + 4 * e, a.out_wide);
                     }
                 }
                 if (ok && !waited) ok = wait_acc();

@@ -305,6 +305,50 @@ __device__ __forceinline__ void pack_i8(const uint32_t* v, const int* bias_c, in
     else pack_i8_as<W, false, false>(v, bias_c, relu, rnd, shift, pk);
 }
 
+__device__ __forceinline__ void st_global_v4(void* p, const uint32_t* v)
+{
+    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t* v, int wide)
+{
+    if (wide) st_global_v8(p, *(const uint32_t(*)[8])v);
+    else { st_global_v4(p, v); st_global_v4((unsigned char*)p + 16, v + 4); }
+}
+
+// f(c + b) of 16 fp32 sums as bf16 or fp32, straight to global memory (wide: dst is 32-byte aligned)
+template <int OUT>
+__device__ __forceinline__ void emit16f(const uint32_t* v, const float* bias_c, int relu, unsigned char* dst, int wide)
+{
+    float f[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+    if (bias_c) {
+#pragma unroll
+        for (int j4 = 0; j4 < 4; ++j4) {
+            const float4 b4 = ((const float4*)bias_c)[j4];
+            f[4 * j4] += b4.x; f[4 * j4 + 1] += b4.y; f[4 * j4 + 2] += b4.z; f[4 * j4 + 3] += b4.w;
+        }
+    }
+    if (OUT == E_BF16) {
+        uint32_t pk[8];
+        if (relu) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
+        }
+        st_global_32(dst, pk, wide);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(relu ? fmaxf(f[8 * h + j], 0.f) : f[8 * h + j]);
+            st_global_32(dst + 32 * h, w, wide);
+        }
+    }
+}
 template <int DT> struct Acc;
 template <> struct Acc<1> { typedef float S; };
 template <> struct Acc<2> { typedef int S; };
