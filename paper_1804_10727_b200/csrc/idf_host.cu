@@ -240,7 +240,14 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
             ce = launch_conv_win(a, P.win, net->dtype, P.w_map_win, P.use_sparse, net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
-        if (ce == cudaErrorNotSupported && P.time.ok && P.tc.ok && n_in > 0) {
+        // 1D layers: time x streams as the tile where the row-ring kernel's tile of 128 streams would be partly empty (a last group of
+        // 26 of 128 included) or the launch has few rows, which it walks one after the other: 48 streams, 20 rows of 128 -> 128
+        // channels 25 against 9 us.  On long blocks of full tiles the ring kernel wins (1024 streams, 1977 rows: 507 against 533 us): its
+        // MMAs of 256 columns (two to four taps at once) fetch three operand bytes where 128 columns fetch four, and the
+        // shared memory is what both are short of.
+        const long long tiles = (S + 127) / 128 * 128;
+        const bool by_time = o_end - o_begin <= 256 || S * 5 < tiles * 4;
+        if (ce == cudaErrorNotSupported && P.time.ok && by_time && P.tc.ok && n_in > 0) {
             ce = launch_conv_time(a, P.time, net->dtype, net->ws + P.wtc_off, net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
