@@ -239,6 +239,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t bar_w = bar_empty + 8u * a.nstage;
     const uint32_t bar_ready = bar_w + 8u * taps;
     const uint32_t bar_free = bar_ready + 8u * a.nslot;
+    const uint32_t bar_start = bar_free + 8u * a.nslot;    // every slot the launch uses holds what its first row starts from
 
     const int nt = blockIdx.x % a.n_nt;
     const int mt_all = blockIdx.x / a.n_nt;
@@ -267,7 +268,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (threadIdx.x == 0) {
         s_abort = 0;
         s_issued = 0;
-        if (!IDF_OK_AT(a.status, (bar_free - smem_u32(smem_raw)) + 8u * a.nslot - 1, a.smem_bytes)) s_abort = 1;
+        if (!IDF_OK_AT(a.status, (bar_start - smem_u32(smem_raw)) + 7, a.smem_bytes)) s_abort = 1;
         // The weights come first: they do not depend on earlier kernels of the stream (their fetch overlaps the
         // previous kernel's tail under programmatic dependent launch), and a launch that brings a single row has
         // little else to hide their latency behind.  One copy per K block carries all taps of the CTA's channel
@@ -279,6 +280,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             tma_load_3d(sW + (uint32_t)(kb * taps) * w_tile_bytes, &tmW, bar_w, kb * a.KB, n0, 0);
         for (int i = 0; i < a.nstage; ++i) { mbar_init(bar_full + 8u * i, 1); mbar_init(bar_empty + 8u * i, 1); }
         for (int i = 0; i < a.nslot; ++i) { mbar_init(bar_ready + 8u * i, 1); mbar_init(bar_free + 8u * i, 4); }
+        mbar_init(bar_start, 4 * MAX_GROUPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -322,7 +324,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     // a new output row starts when ph == 0: its slot's previous row must have been read out
                     const bool fresh = (ri > 0 && ph == 0 && hi >= nslot && hi < c_n_orows);
                     q[0] = fresh ? bar_free + 8u * (uint32_t)slot_hi : 0u;
-                    q[1] = (uint32_t)(u_hi & 1);
+                    q[1] = (uint32_t)((u_hi & 1) ^ 1);              // phase u_hi - 1 of the slot: its row before this one has left
                     // the row completed by input row ri is (t0 - (Kh-1)) / s when that is a whole number >= 0
                     const int tf = t0 - (a.Kh - 1);
                     const int of = tf >= 0 ? tf / s : -1;
@@ -400,9 +402,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t a_stage_units = a_stage_bytes >> 4;
             const int nstage = a.nstage, n_kb = a.n_kb;
             bool ok = true;
-            // every slot this launch uses has been cleared once (a short launch visits fewer rows than there are slots)
-            for (int slot = 0; slot < (c_n_orows < nslot ? c_n_orows : nslot) && ok; ++slot)
-                ok = mbar_wait(bar_free + 8u * slot, 0, abort_flag);
+            // Every slot holds what its first row starts from.  This is a barrier of its own, not the slots' first free phase: the
+            // producer may be a slot's whole turn ahead, and a parity would not tell it that phase from the one it needs.
+            ok = mbar_wait(bar_start, 0, abort_flag);
             ok = ok && mbar_wait(bar_w, 0, abort_flag);          // the CTA's weight slice has landed
             // (paired positions: no swizzle, 8 rows of 16 bytes are 128 bytes, and the second half of a K step is the next position)
             const uint64_t adesc_base = (a.pair ? ((uint64_t)1 << 16) | ((uint64_t)8 << 32) | ((uint64_t)1 << 46) : desc_hi) | (uint64_t)((sA & 0x3FFFFu) >> 4);
@@ -568,11 +570,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     __syncwarp();
                     tmem_st16(tlane + (uint32_t)(slot * a.Ntile + c), v);
                 }
-                tmem_st_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_free + 8u * slot);   // one arrival per warp
             }
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_start);   // one arrival per warp
         }
         // Rows left open by this block go back to the ring in global memory; those that meet in one ring slot stay in
         // one group, in order.  (Rows begun by an earlier block were read above, before the first MMA, so nothing
@@ -794,7 +796,12 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     const bool wide_for_1d = true;
     for (int nt = 256; nt >= 16; nt >>= 1) {
         if (Cout % nt) continue;
-        if ((ring_rows + 1) * nt > 512) continue;
+        // TMEM slots.  An epilogue group tells the uses of a slot apart by the parity of its barrier, so it must have seen the row that
+        // used the slot before a row of its own: no group may skip as many rows as there are slots.  Its first row comes after at
+        // most the rows begun by an earlier block (Kh - 1 at stride 1, at most ring_rows) and a turn of all groups, by rows or by pairs.
+        const int n_cin = ring_rows == Kh ? Kh - 1 : ring_rows;
+        const int slots = 512 / nt > 16 ? 16 : 512 / nt;
+        if (slots < ring_rows + 1 || slots < n_cin + (pooled ? 2 : 1) * MAX_GROUPS) continue;
         if ((ring_rows + 256 / nt - 1) / (256 / nt) + 1 > 4) continue;   // at most 4 MMA segments per input row
         const size_t wb = (size_t)taps * p->n_kb * nt * p->swb;
         if (wb + 3 * a_stage + (size_t)stage_rows * nt * out_esize + 10240 > SMEM_LIMIT) continue;   // one staging tile at least
@@ -843,7 +850,7 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     if (nstage > 8) nstage = 8;
     if (nstage < 2) return false;
     p->nstage = nstage;
-    p->smem_bytes = 1024 + wb + (size_t)nstage * a_stage + tail_have + tail_pad + 8 * (2 * nstage + taps + 2 * p->nslot) + 64;
+    p->smem_bytes = 1024 + wb + (size_t)nstage * a_stage + tail_have + tail_pad + 8 * (2 * nstage + taps + 2 * p->nslot + 1) + 64;
     p->w_bytes = (size_t)taps * Cout * Cin * esize;
     p->ok = 1;
     return true;
