@@ -202,6 +202,7 @@ struct TcPlan {
     int BX = 0, BS = 0;      // a 128-row M tile = BS streams x BX consecutive x positions
     int BXP = 0;             // positions per stream held in the shared-memory tile (BX + kx halo)
     int shift_mode = 0;      // kx taps read one haloed tile at row offsets instead of one box per kx
+    int light = 0;           // for the build of the kernel of which an SM holds two CTAs
     int pair = 0;            // positions of 16 bytes, two to a K step
     int sx = 1;              // x stride (> 1 only without shift_mode: the tensor map walks the input row in steps of sx)
     int a_stage_bytes = 0;

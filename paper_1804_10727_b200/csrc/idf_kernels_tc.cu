@@ -29,9 +29,13 @@ namespace idf {
 
 namespace {
 
-constexpr int MAX_GROUPS = 3;                // epilogue groups (four warps each) taking output rows in turn
-constexpr int TC_THREADS = 64 + 128 * MAX_GROUPS;
-constexpr int ROWQ = 64;                     // row-schedule queue: two chunks of 32 rows
+// Two builds of the kernel: one CTA per SM with three epilogue groups (four warps each, taking output rows in turn), and a light
+// one with two groups, half the shared and tensor memory and at most 102 registers, of which an SM holds two.  tc_make_plan says
+// which layers take it and what it measured.
+constexpr int FULL_GROUPS = 3, LIGHT_GROUPS = 2;
+constexpr int tc_threads(int groups) { return 64 + 128 * groups; }
+constexpr int tc_rowq(int groups) { return groups == FULL_GROUPS ? 64 : 32; }      // row-schedule queue: two chunks
+constexpr size_t LIGHT_SMEM = 113408;        // dynamic shared memory of a light CTA: half an SM less the static part
 
 // Where an emitted row goes first: a shared-memory tile [tile row][panel of pwb bytes], written in
 // the swizzle the output tensor map expects, from which one thread sends it out with a TMA store.
@@ -208,12 +212,13 @@ struct TcArgs {
 
 // KX3: the common case of 128-byte rows with three kx taps read row-shifted from one haloed box, known at compile time
 // (the MMA warp's loop is what the kernel's speed hangs on: every constant it sees helps)
-template <int DT, int KSTEPS, int KX3>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+template <int DT, int KSTEPS, int KX3, int GROUPS>
+__global__ void __launch_bounds__(tc_threads(GROUPS), GROUPS == FULL_GROUPS ? 1 : 2)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                const __grid_constant__ CUtensorMap tmO, const TcArgs a)
 {
     typedef typename Acc<DT>::S TS;
+    constexpr int ROWQ = tc_rowq(GROUPS), CHUNK = ROWQ / 2;
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
@@ -280,7 +285,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             tma_load_3d(sW + (uint32_t)(kb * taps) * w_tile_bytes, &tmW, bar_w, kb * a.KB, n0, 0);
         for (int i = 0; i < a.nstage; ++i) { mbar_init(bar_full + 8u * i, 1); mbar_init(bar_empty + 8u * i, 1); }
         for (int i = 0; i < a.nslot; ++i) { mbar_init(bar_ready + 8u * i, 1); mbar_init(bar_free + 8u * i, 4); }
-        mbar_init(bar_start, 4 * MAX_GROUPS);
+        mbar_init(bar_start, 4 * GROUPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -313,10 +318,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int stage = 0, t = 0;
         uint32_t phase = 0;
         bool ok = true;
-        for (int r_chunk = 0; r_chunk < n_rows && ok; r_chunk += 32) {
+        for (int r_chunk = 0; r_chunk < n_rows && ok; r_chunk += CHUNK) {
             {
                 const int ri = r_chunk + lane;
-                if (ri < n_rows) {
+                if (lane < CHUNK && ri < n_rows) {
                     uint32_t* q = s_rowq[ri & (ROWQ - 1)];
                     const int t0 = c_base_ty + ri;
                     const int hi = t0 / s, ph = t0 - hi * s;
@@ -357,7 +362,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
             __syncwarp();
             if (lane == 0) {
-                const int r_end = r_chunk + 32 < n_rows ? r_chunk + 32 : n_rows;
+                const int r_end = r_chunk + CHUNK < n_rows ? r_chunk + CHUNK : n_rows;
                 for (int ri = r_chunk; ri < r_end && ok; ++ri) {
                     // A row that starts a new output row needs that row's slot read out and cleared.  Waiting
                     // here, before the row's first copy, means the MMA thread learns it from the copy's
@@ -452,8 +457,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 uint32_t next_ok = 1u;
                 if (!(last_row && row_end)) next_ok = mbar_test(bar_full + 8u * n_stage, n_phase);
                 uint4 nh = hdr, na = sa, nb = sb, nc = sc;
-                // schedule entries are published 32 rows at a time, ahead of the first copy of those rows
-                const bool early_info = row_end && !last_row && ((ri + 1) & 31) != 0;
+                // schedule entries are published a chunk of rows at a time, ahead of the first copy of those rows
+                const bool early_info = row_end && !last_row && ((ri + 1) & (CHUNK - 1)) != 0;
                 const uint4* qn = (const uint4*)s_rowq[(ri + 1) & (ROWQ - 1)];
                 if (early_info) { nh = qn[0]; na = qn[1]; nb = qn[2]; nc = qn[3]; }
                 // ---- the other kx taps of the tile (row-shifted reads of the same box)
@@ -508,7 +513,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int s = s0 + bs, x = x0 + bx;
         const bool in_tile = (bs < a.BS) && (bx < a.BX);
         const bool valid = in_tile && (s < a.S) && (x < a.Wout);
-        const bool wide = (a.Ntile & 31) == 0;
+        const bool wide = GROUPS == FULL_GROUPS && (a.Ntile & 31) == 0;     // (32 columns at a time take more registers than the light build has)
         const TS* bias = a.bias ? (const TS*)a.bias + n0 : nullptr;
         const long long row_elems = (long long)a.Wout * a.Cout;
         TS* ring_pos = (TS*)a.ring + (long long)s * row_elems + (long long)x * a.Cout + n0;   // + ring slot * S * row_elems
@@ -546,7 +551,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int slot = 0; slot < (c_n_orows < a.nslot ? c_n_orows : a.nslot); ++slot) {
                 const int rslot = rs;
                 if (++rs == a.ring_rows) rs = 0;
-                if (slot % MAX_GROUPS != grp) continue;
+                if (slot % GROUPS != grp) continue;
                 // (carried_row is the same in all threads: the tensor-memory stores below are warp-wide instructions and
                 // every branch around them must be uniform; what differs per thread is only whether it has values to load)
                 const bool carried_row = c_r0_positive && (slot * a.stride - c_base_ty < 0);
@@ -658,7 +663,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
 #endif
             {
-                if (wide) {
+                if (GROUPS == FULL_GROUPS && wide) {
                     for (int c = 0; c < a.Ntile; c += 32) {
                         uint32_t v[32];
                         if (!fine) continue;
@@ -732,10 +737,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
-}  // namespace
-
-bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, int Kw, int stride_x, int ring_rows,
-                  int out_esize, int pooled, int pair, TcPlan* p)
+// The plan for one of the two builds.
+bool make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, int Kw, int stride_x, int ring_rows,
+               int out_esize, int pooled, int pair, int light, TcPlan* p)
 {
     *p = TcPlan{};
     if (dtype != 1 && dtype != 2) return false;
@@ -756,6 +760,9 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     // bytes) and a K step is two neighbouring positions: the leading-dimension offset of the A descriptor is one row.  Cin and Kw
     // are those of the pairs: 32 bytes, half the taps (rounded up; the odd one has zero weights).  No x-unfold pass is needed
     // (16 -> 32 channels int8, 4096 streams of 26-wide rows with pool: 0.183 -> 0.149 ms).
+    p->light = light;
+    const size_t limit = light ? LIGHT_SMEM : SMEM_LIMIT, slack = light ? 1536 : 10240;
+    const int tmem_max = light ? 256 : 512;
     p->pair = pair;
     if (pair && (row_bytes != 32 || stride_x != 1)) return false;
     p->shift_mode = Kw > 1 && stride_x == 1;
@@ -799,14 +806,14 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
         // TMEM slots.  An epilogue group tells the uses of a slot apart by the parity of its barrier, so it must have seen the row that
         // used the slot before a row of its own: no group may skip as many rows as there are slots.  Its first row comes after at
         // most the rows begun by an earlier block (Kh - 1 at stride 1, at most ring_rows) and a turn of all groups, by rows or by pairs.
-        const int n_cin = ring_rows == Kh ? Kh - 1 : ring_rows;
-        const int slots = 512 / nt > 16 ? 16 : 512 / nt;
-        if (slots < ring_rows + 1 || slots < n_cin + (pooled ? 2 : 1) * MAX_GROUPS) continue;
+        const int n_cin = ring_rows == Kh ? Kh - 1 : ring_rows, groups = light ? LIGHT_GROUPS : FULL_GROUPS;
+        const int slots = tmem_max / nt > 16 ? 16 : tmem_max / nt;
+        if (slots < ring_rows + 1 || slots < n_cin + (pooled ? 2 : 1) * groups) continue;
         if ((ring_rows + 256 / nt - 1) / (256 / nt) + 1 > 4) continue;   // at most 4 MMA segments per input row
         const size_t wb = (size_t)taps * p->n_kb * nt * p->swb;
-        if (wb + 3 * a_stage + (size_t)stage_rows * nt * out_esize + 10240 > SMEM_LIMIT) continue;   // one staging tile at least
+        if (wb + (light ? 2 : 3) * a_stage + (size_t)stage_rows * nt * out_esize + slack > limit) continue;   // one staging tile at least
         const int units = p->n_mt * (Cout / nt);
-        if (units >= 120) { best = nt; break; }          // enough CTAs for the 148 SMs: take the widest such tile
+        if (units >= (light ? 1 : 120)) { best = nt; break; }          // enough CTAs for the 148 SMs: take the widest such tile
         // 1D nets come in long blocks of rows, which row chunks spread over the SMs: there the widest tile that fits
         // wins, because every channel slice fetches the Δ-rows again (audio1d's 128-channel layers with 16-channel
         // tiles moved 4.2 GB per layer through the L2)
@@ -816,7 +823,7 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     if (!best) return false;
     p->Ntile = best;
     p->n_nt = Cout / best;
-    p->nslot = 512 / best;
+    p->nslot = tmem_max / best;
     if (p->nslot > 16) p->nslot = 16;
     // as many resident rows as tensor memory holds: the fewer input rows whose window of ring rows
     // wraps around the slot array, the fewer split MMAs
@@ -834,18 +841,19 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     p->out_bufs = 1;
     // layers with many short K blocks per row (little MMA work per tile) need a deeper pipeline to cover the
     // copy latency more than they need a second epilogue group
-    const size_t want_stages = p->n_kb >= 4 ? 4 : 3;
-    for (int g = MAX_GROUPS; g > 1; --g)
-        if (wb + want_stages * a_stage + (size_t)g * p->out_stage_bytes + 10240 <= SMEM_LIMIT) { p->out_groups = g; break; }
+    const size_t want_stages = light ? 2 : (p->n_kb >= 4 ? 4 : 3);
+    for (int g = light ? LIGHT_GROUPS : FULL_GROUPS; g > 1; --g)
+        if (wb + want_stages * a_stage + (size_t)g * p->out_stage_bytes + slack <= limit) { p->out_groups = g; break; }
     // a second staging tile per group where it still leaves one more Δ-row stage than wanted
-    if (wb + (want_stages + 1) * a_stage + 2 * (size_t)p->out_groups * p->out_stage_bytes + 10240 <= SMEM_LIMIT) p->out_bufs = 2;
+    if (!light && wb + (want_stages + 1) * a_stage + 2 * (size_t)p->out_groups * p->out_stage_bytes + slack <= limit) p->out_bufs = 2;
     // the MMAs' run past a small box (see a_stage) must end inside this CTA's shared memory: what follows the
     // last stage (the staging tiles) covers it, or padding is added behind them
     const size_t overrun = (size_t)(128 + halo) * pos_bytes > box_pitch ? (size_t)(128 + halo) * pos_bytes - box_pitch : 0;
     const size_t tail_have = (size_t)p->out_groups * p->out_bufs * p->out_stage_bytes;
     const size_t tail_pad = overrun > tail_have ? (overrun - tail_have + 1023) / 1024 * 1024 : 0;
-    if (SMEM_LIMIT < 8192 + wb + 1024 + tail_have + tail_pad + 2 * a_stage) return false;
-    const size_t room = SMEM_LIMIT - 8192 - wb - 1024 - tail_have - tail_pad;   // static shared memory and alignment slack stay free
+    const size_t reserve = light ? 1536 : 8192 + 1024;
+    if (limit < reserve + wb + tail_have + tail_pad + 2 * a_stage) return false;
+    const size_t room = limit - reserve - wb - tail_have - tail_pad;   // static shared memory and alignment slack stay free
     int nstage = (int)(room / a_stage);
     if (nstage > 8) nstage = 8;
     if (nstage < 2) return false;
@@ -853,6 +861,27 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
     p->smem_bytes = 1024 + wb + (size_t)nstage * a_stage + tail_have + tail_pad + 8 * (2 * nstage + taps + 2 * p->nslot + 1) + 64;
     p->w_bytes = (size_t)taps * Cout * Cin * esize;
     p->ok = 1;
+    return true;
+}
+
+}  // namespace
+
+// Which build.  A layer of few input channels has little tensor-core work per row and is bound by its epilogue and by the waits
+// between the roles of one CTA; a second CTA on the SM adds a fourth group and fills those waits.  Its price is half the room:
+// where that costs a narrower channel tile the input is read again for each, and the full build is the better one
+// (int8 64 -> 64 with pool, 2048 streams of 126-wide rows: 0.80 ms full, 0.89 light with half the tile; bf16 128 -> 128, 64 x 112: 0.201
+// and 0.228; bf16 256 -> 256, 64 x 56: 0.256 and 0.346).  With the same tile the light build wins as soon as there are more CTAs
+// than SMs (int8 32 -> 64 stride 2, 254-wide rows: 128 streams 44 us full, 47 light; 192: 82 and 53; 2048: 531 and 339;
+// int8 16 -> 32 with pool, 26-wide rows: 512 streams 28 and 30, 768: 47 and 37, 4096: 152 and 111; bf16 16 -> 32, 128-wide rows: 128
+// streams 50 and 49, 256: 92 and 57, 1024: 313 and 200; one-row pushes of int8 64 -> 32, 128-wide rows: 128 streams 12 and 13, 1024: 47 and 29).
+bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, int Kw, int stride_x, int ring_rows,
+                  int out_esize, int pooled, int pair, TcPlan* p)
+{
+    if (!make_plan(dtype, S, Win, Wout, Cin, Cout, Kh, Kw, stride_x, ring_rows, out_esize, pooled, pair, 0, p)) return false;
+    TcPlan light;
+    if (make_plan(dtype, S, Win, Wout, Cin, Cout, Kh, Kw, stride_x, ring_rows, out_esize, pooled, pair, 1, &light) &&
+        light.Ntile == p->Ntile && light.n_mt * light.n_nt > 148)
+        *p = light;
     return true;
 }
 
@@ -990,23 +1019,26 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const 
     }
     const unsigned grid = (unsigned)(p.n_mt * p.n_nt * t.n_chunks);
     typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TcArgs);
-    static const KernelFn kernels[2][4] = {
-        {conv_tc_kernel<1, 1, 0>, conv_tc_kernel<1, 2, 0>, conv_tc_kernel<1, 4, 0>, conv_tc_kernel<1, 4, 1>},
-        {conv_tc_kernel<2, 1, 0>, conv_tc_kernel<2, 2, 0>, conv_tc_kernel<2, 4, 0>, conv_tc_kernel<2, 4, 1>}};
+    static const KernelFn kernels[4][4] = {
+        {conv_tc_kernel<1, 1, 0, 3>, conv_tc_kernel<1, 2, 0, 3>, conv_tc_kernel<1, 4, 0, 3>, conv_tc_kernel<1, 4, 1, 3>},
+        {conv_tc_kernel<2, 1, 0, 3>, conv_tc_kernel<2, 2, 0, 3>, conv_tc_kernel<2, 4, 0, 3>, conv_tc_kernel<2, 4, 1, 3>},
+        {conv_tc_kernel<1, 1, 0, 2>, conv_tc_kernel<1, 2, 0, 2>, conv_tc_kernel<1, 4, 0, 2>, conv_tc_kernel<1, 4, 1, 2>},
+        {conv_tc_kernel<2, 1, 0, 2>, conv_tc_kernel<2, 2, 0, 2>, conv_tc_kernel<2, 4, 0, 2>, conv_tc_kernel<2, 4, 1, 2>}};
     const int kidx = p.swb == 32 ? 0 : (p.swb == 64 ? 1 : ((p.shift_mode && a.Kw == 3) ? 3 : 2));
-    const KernelFn fn = kernels[dtype - 1][kidx];
-    static bool attr_set[2][4][64] = {};
+    const int kind = dtype - 1 + (p.light ? 2 : 0);
+    const KernelFn fn = kernels[kind][kidx];
+    static bool attr_set[4][4][64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!attr_set[dtype - 1][kidx][dev]) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SMEM_LIMIT - 6144));
+    if (!attr_set[kind][kidx][dev]) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(p.light ? LIGHT_SMEM : SMEM_LIMIT - 6144));
         if (e != cudaSuccess) return e;
-        attr_set[dtype - 1][kidx][dev] = true;
+        attr_set[kind][kidx][dev] = true;
     }
     // programmatic dependent launch: the kernel may be scheduled while its predecessor drains; it
     // touches nothing but its weights until griddepcontrol.wait
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = p.smem_bytes; cfg.stream = st;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(tc_threads(p.light ? LIGHT_GROUPS : FULL_GROUPS)); cfg.dynamicSmemBytes = p.smem_bytes; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
