@@ -544,37 +544,39 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // Every ring slot in tensor memory starts from what its row has so far (all MMAs accumulate): zero, or, for a
         // row begun by an earlier block, the partial sums that block left in the ring in global memory.  Taking those
         // up here, while weights and the first rows are still on their way, keeps the ring's read latency out of the
-        // path between the last MMA and the emission; the three groups share the slots.
+        // path between the last MMA and the emission.  A launch that brings one row waits for little else, so the groups share
+        // the carried rows by columns and a thread's loads go out together, not one piece of 16 columns after the other.
         {
+            constexpr int PIECES = GROUPS == FULL_GROUPS ? 3 : 2;
             const long long carry_off0 = (const TS*)a.ring_in - (const TS*)a.ring;
-            int rs = (a.ring_slot0 + c_oa) % a.ring_rows;
-            for (int slot = 0; slot < (c_n_orows < a.nslot ? c_n_orows : a.nslot); ++slot) {
-                const int rslot = rs;
-                if (++rs == a.ring_rows) rs = 0;
-                if (slot % GROUPS != grp) continue;
-                // (carried_row is the same in all threads: the tensor-memory stores below are warp-wide instructions and
-                // every branch around them must be uniform; what differs per thread is only whether it has values to load)
-                const bool carried_row = c_r0_positive && (slot * a.stride - c_base_ty < 0);
-                bool carried = carried_row && valid;
-                const TS* rp = ring_pos + (long long)rslot * ring_slot_stride + carry_off0;
-#ifdef IDF_BOUNDS
-                if (carried && !IDF_OK_AT(a.status, (rp - carry_off0 - (const TS*)a.ring) + a.Ntile - 1, a.ring_elems)) carried = false;
-#endif
-                for (int c = 0; c < a.Ntile; c += 16) {
-                    uint32_t v[16];
-                    if (carried) {
-                        uint32_t lo[8], hi[8];
-                        ld_global_v8(rp + c, lo);
-                        ld_global_v8(rp + c + 8, hi);
+            const int n_init = c_n_orows < a.nslot ? c_n_orows : a.nslot;
+            const int per_slot = 31 - __clz(a.Ntile >> 4);                              // log2 of the pieces of a slot (Ntile is a power of two)
+            for (int i0 = grp * PIECES; i0 < n_init << per_slot; i0 += GROUPS * PIECES) {
+                uint32_t v[PIECES][16];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) { v[j] = lo[j]; v[8 + j] = hi[j]; }
+                for (int u = 0; u < PIECES; ++u) {
+                    const int slot = (i0 + u) >> per_slot, c = ((i0 + u) - (slot << per_slot)) * 16;
+                    // (slot and carried_row are the same in all threads: the tensor-memory stores below are warp-wide instructions and
+                    // every branch around them must be uniform; what differs per thread is only whether it has values to load)
+                    const bool carried_row = slot < n_init && c_r0_positive && slot * a.stride - c_base_ty < 0;
+                    bool carried = carried_row && valid;
+                    const TS* rp = ring_pos + carry_off0 + c;
+                    if (carried_row) rp += (long long)((a.ring_slot0 + c_oa + slot) % a.ring_rows) * ring_slot_stride;
+#ifdef IDF_BOUNDS
+                    if (carried && !IDF_OK_AT(a.status, (rp - carry_off0 - (const TS*)a.ring) + 15, a.ring_elems)) carried = false;
+#endif
+                    if (carried) {
+                        ld_global_v8(rp, *(uint32_t(*)[8])v[u]);
+                        ld_global_v8(rp + 8, *(uint32_t(*)[8])(v[u] + 8));
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = 0u;
+                        for (int j = 0; j < 16; ++j) v[u][j] = 0u;
                     }
-                    __syncwarp();
-                    tmem_st16(tlane + (uint32_t)(slot * a.Ntile + c), v);
                 }
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < PIECES; ++u)
+                    if (i0 + u < n_init << per_slot) tmem_st16(tlane + (uint32_t)((i0 + u) << 4), v[u]);
             }
             tmem_st_wait();
             tc_fence_before();

@@ -19,7 +19,7 @@
 // Steps that exchange rows with the ring (begun by an earlier block, or left open by this one) are the same MMAs with
 // the missing input rows as zeros; the epilogue then adds what the ring holds and parks what stays open.  Where two
 // such rows can meet in one ring slot, those of a tile are one work item and a slot's words belong to one thread, which
-// takes the rows in order.  A freed slot is left zero.  All else are independent work items, dealt round robin to one
+// takes the rows in order.  A freed slot is left zero where the event scatter shares the ring.  All else are independent work items, dealt round robin to one
 // CTA per SM.  Layers that report their input events (Eq. 3: non-zero components) count them while the runs pass by.
 //
 // Measured on B200, against the kernels that served these layers before (event scatter on CUDA cores; one im2col row per
@@ -64,6 +64,8 @@ struct WinArgs {
     // visited rows share a ring slot, so the other steps ([0, e0_end) and [e1_begin, n_steps)) of a tile are one work item;
     // all else are independent work items of R steps
     int n_steps, e0_end, e1_begin, R, ordered, n_items;
+    int clear;                   // leave the slots of emitted rows zero (the scatter kernel starts its rows from what the ring holds)
+    int parts, part_cols;        // a work item is all N columns of its windows (1 part), or one of `parts` runs of part_cols
     long long in_elems, out_elems, ring_elems;
 };
 
@@ -85,13 +87,19 @@ __device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t 
 }
 // Walks the steps this CTA takes.  A work item is a tile of 128 windows and the steps [a0, a0 + na), then from b0 on (n in all).
 struct WinWalk {
-    int it, i, n, a0, na, b0, tile;
+    int it, i, n, a0, na, b0, tile, part;
     __device__ __forceinline__ void open(const WinArgs& a)
     {
         i = 0;
         if (it >= a.n_items) { n = 0; return; }
-        const int grp = it / a.n_tiles;
+        int grp = it / a.n_tiles;
         tile = it - grp * a.n_tiles;
+        part = 0;
+        if (a.parts > 1) {
+            const int g = grp / a.parts;
+            part = grp - g * a.parts;
+            grp = g;
+        }
         if (a.ordered && grp == 0) {
             a0 = 0; na = a.e0_end; b0 = a.e1_begin; n = a.e0_end + (a.n_steps - a.e1_begin);
         } else {
@@ -177,7 +185,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             live = col < a.ncol;
             const int s = AX == 0 ? col / a.nxw : col, xw = AX == 0 ? col - s * a.nxw : 0;
             b0 = (xw * a.P * a.stride_x - a.pad_x) * a.Cin * ES;
-            own = live ? (xw == a.nxw - 1 ? 4 * WIN_MAX_WORDS : a.P * a.Cin * ES) : 0;   // (events: bytes of a run that are this window's to count)
+            own = live && w.part == 0 ? (xw == a.nxw - 1 ? 4 * WIN_MAX_WORDS : a.P * a.Cin * ES) : 0;   // (events: bytes of a run that are this window's to count)
             in_s = (const unsigned char*)a.in + (long long)s * row_bytes;
         };
         int stage = set;                                                            // steps go round the stages (and the two sets)
@@ -338,8 +346,9 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         // ------------------------------ MMA issuer ---------------------------------------------
         const uint64_t desc_hi = make_smem_desc(0, a.swb);
         const uint32_t idesc = (DT == 1 ? ((1u << 4) | (1u << 7) | (1u << 10)) : ((2u << 4) | (1u << 7) | (1u << 10))) |
-                               ((128u >> 4) << 24) | ((uint32_t)(a.N >> 3) << 17);
-        const uint64_t bdesc = desc_hi | (uint64_t)((sW & 0x3FFFFu) >> 4);
+                               ((128u >> 4) << 24) | ((uint32_t)(a.part_cols >> 3) << 17);
+        const uint64_t bdesc0 = desc_hi | (uint64_t)((sW & 0x3FFFFu) >> 4);
+        const uint32_t part_units = (uint32_t)a.part_cols * a.swb >> 4;       // (a multiple of eight rows: the swizzle pattern starts over)
         bool ok = mbar_wait(bar_w, 0, abort_flag);
         const bool issuer = elect_one();
         int t = 0, stage = 0;
@@ -353,6 +362,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             if (issuer) {
                 const uint64_t adesc = desc_hi | (uint64_t)(((sA + (uint32_t)stage * stage_bytes) & 0x3FFFFu) >> 4);
                 const uint32_t d = tmem_base + 256u * acc;
+                const uint64_t bdesc = bdesc0 + (uint64_t)((uint32_t)w.part * part_units);
                 if (a.ksteps == 1) umma_tile<DT, 1, true>(d, adesc, bdesc, idesc);
                 else if (a.ksteps == 2) umma_tile<DT, 2, true>(d, adesc, bdesc, idesc);
                 else if (a.ksteps == 3) umma_tile<DT, 3, true>(d, adesc, bdesc, idesc);
@@ -369,7 +379,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         const int m = q * 32 + lane;
         const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16);
         const int oes = a.out_elem == E_F32 ? 4 : (a.out_elem == E_BF16 ? 2 : 1);
-        const int n_chunk = (a.N + 31) >> 5;
+        const int n_chunk = (a.part_cols + 31) >> 5;
         unsigned char* out = (unsigned char*)a.out;
         uint32_t* ring = (uint32_t*)a.ring;
         const long long ring_row = (long long)a.Wout * a.Cout;
@@ -390,7 +400,8 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
             }
             const int step = w.step();
             const int acc = t & 1;
-            const uint32_t trow = tlane + 256u * acc;
+            const int k_part = w.part * n_chunk;                                     // the item's first piece of 32 columns
+            const uint32_t trow = tlane + 256u * acc - 32u * (uint32_t)k_part;
             const long long o_row = o_base + (a.out_row_first + (AX == 0 ? step : step * a.P)) * a.out_row_stride;
             auto wait_acc = [&]() {
                 int got = 1;
@@ -404,8 +415,8 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                 if (!wait_acc()) { ok = false; break; }
                 const int n_col = n_pos * a.Cout;
                 unsigned char* dst = out + o_row * oes;
-                int k = first;
-                for (; k < n_chunk; k += WIN_EPI_GROUPS) {
+                int k = k_part + first;
+                for (; k < k_part + n_chunk; k += WIN_EPI_GROUPS) {
                     const int c = 32 * k;
                     uint32_t v[32];
                     // where the two halves (16 channels of one output each) go: side by side in a row (2D), or a row each (1D)
@@ -447,12 +458,12 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                         if (hi) emit16f<E_F32>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
                     }
                 }
-                first = k - n_chunk;
+                first = k - k_part - n_chunk;
             } else {
                 // A step that exchanges rows with the ring, 16 columns at a time.  The columns' groups are fixed here; in an
                 // ordered 1D item the group goes by ring slot (a column run is a row of its own there).
                 bool waited = false;
-                for (int k = 0; k < 2 * n_chunk; ++k) {
+                for (int k = 2 * k_part; k < 2 * (k_part + n_chunk); ++k) {
                     const int c = 16 * k;
                     const int p = (int)(((uint32_t)k * a.inv_c16) >> 16), co = c - p * a.Cout;
                     const int o = AX == 0 ? step : step * a.P + p;                  // visited row (the same in all lanes)
@@ -481,7 +492,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                         st_global_v8(ring + ri + 8, *(uint32_t(*)[8])(v + 8));
                         continue;
                     }
-                    if (carried) {                                                 // the slot is free again
+                    if (carried && a.clear) {                                      // the slot is free again
                         const uint32_t z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
                         st_global_v8(ring + ri, z);
                         st_global_v8(ring + ri + 8, z);
@@ -606,6 +617,7 @@ cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, cons
     WinArgs t{};
     t.in = a.in; t.bias = a.bias; t.ring = a.ring; t.out = a.out; t.status = a.status;
     t.events = count_events ? a.event_counter : nullptr;
+    t.clear = count_events;
     t.out_row_stride = a.out_row_stride; t.out_stream_stride = a.out_stream_stride;
     t.out_row_first = a.o_begin - a.out_row_base;
     t.n_in = (int)(a.r1 - a.r0); t.n_rows = (int)(a.o_end - a.o_begin); t.done_rel = (int)(a.done_end - a.o_begin);
@@ -634,7 +646,14 @@ cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, cons
     const int n_free = t.ordered ? t.e1_begin - t.e0_end : t.n_steps;
     const long long R = (long long)n_free * t.n_tiles / (148 * 4);
     t.R = (int)(R < 1 ? 1 : (R > 16 ? 16 : R));
-    const long long n_items = (long long)(t.ordered + (n_free + t.R - 1) / t.R) * t.n_tiles;
+    long long n_items = (long long)(t.ordered + (n_free + t.R - 1) / t.R) * t.n_tiles;
+    // A launch of few items (a row pushed at a time: three visited rows, all of them exchanged with the ring, whose 64-byte pieces are
+    // what takes the time) spreads an item's columns over several CTAs, which build the same windows, until every SM has an item
+    // (3 -> 64 bf16, 64 streams of 224-wide rows pushed one by one, 84 items: 14.1 us whole, 10.5 in two parts, 11.2 in four).
+    t.parts = 1;
+    while (!t.ordered && t.R == 1 && p.N % (64 * t.parts) == 0 && n_items * t.parts < 148) t.parts *= 2;
+    t.part_cols = p.N / t.parts;
+    n_items *= t.parts;
     if (n_items > 0x3fffffffLL) return cudaErrorNotSupported;
     t.n_items = (int)n_items;
     typedef void (*KernelFn)(const CUtensorMap, const WinArgs);
