@@ -67,7 +67,12 @@ __device__ __forceinline__ uint32_t word_max(uint32_t x, uint32_t y)
 {
     if (OP == 0) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y)); return r; }
     if (OP == 1) return __float_as_uint(fmaxf(__uint_as_float(x), __uint_as_float(y)));
-    return __vmaxs4(x, y);
+    // two bytes at a time: of a 16-bit maximum the upper byte is right whatever the lower bytes are
+    uint32_t h, l, r;
+    asm("max.s16x2 %0, %1, %2;" : "=r"(h) : "r"(x), "r"(y));
+    asm("max.s16x2 %0, %1, %2;" : "=r"(l) : "r"(x << 8), "r"(y << 8));
+    asm("prmt.b32 %0, %1, %2, 0x3715;" : "=r"(r) : "r"(h), "r"(l));
+    return r;
 }
 // 2x2 max-pooling folded into the emission of a conv layer's rows.  A thread owns one (stream, x)
 // position; its x neighbour is the next lane.  The x-pooled first row of a pair waits in the group's
@@ -283,9 +288,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         mbar_expect_tx(bar_w, (uint32_t)(taps * a.n_kb) * w_tile_bytes);
         for (int kb = 0; kb < a.n_kb; ++kb)
             tma_load_3d(sW + (uint32_t)(kb * taps) * w_tile_bytes, &tmW, bar_w, kb * a.KB, n0, 0);
-        for (int i = 0; i < a.nstage; ++i) { mbar_init(bar_full + 8u * i, 1); mbar_init(bar_empty + 8u * i, 1); }
-        for (int i = 0; i < a.nslot; ++i) { mbar_init(bar_ready + 8u * i, 1); mbar_init(bar_free + 8u * i, 4); }
-        mbar_init(bar_start, 4 * GROUPS);
+    }
+    // (one barrier to a lane: one thread initialising them all takes longer than everything else up to here)
+    if (warp == 2) {
+        if (lane < a.nstage) { mbar_init(bar_full + 8u * lane, 1); mbar_init(bar_empty + 8u * lane, 1); }
+        if (lane < a.nslot) { mbar_init(bar_ready + 8u * lane, 1); mbar_init(bar_free + 8u * lane, 4); }
+        if (lane == 31) mbar_init(bar_start, 4 * GROUPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
