@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -1306,20 +1307,46 @@ int idf_run_host(idf_net* net, const void* h_segments, int n_seg, void* d_segmen
     if (n_seg < 0) return fail(IDF_ERR_ARG, "negative count");
     // Pipeline over row blocks: while block b is computed on the handle's stream, block b + 1 travels to the
     // device on a second stream and the output rows block b - 1 completed travel back on a third.
-    // Half a row block per step: the first block's way in and the last block's way out are the part of the copies
-    // that nothing overlaps, and they shrink with the block, while the launches grow only a little more numerous
-    // (vgg2d: 2.20 -> 1.98 ms per batch; a quarter block is slower again).
-    const long long pipe = net->row_block >= 2 ? net->row_block / 2 : 1;
-    // ... and the first and the last step take half of that again when there are steps enough
+    const LayerPlan& P = net->L.back();
+    const size_t seg_bytes = (size_t)net->n_streams * net->in_w * net->in_c * elem_size(net->L[0].in_elem);
+    const size_t orow_bytes = (size_t)P.out_w * P.out_c * elem_size(P.out_elem);
+    // How many steps.  The first step's way in and the last one's way out are the part of the copies that nothing overlaps, so they
+    // shrink with the steps; but every step costs a launch of every layer (about 5 us, and up to 5 more where a CTA fetches
+    // much weight).  The sum is least at sqrt(copy time / step cost) steps: 64 vgg2d streams of 224 rows, 71 MB, 4 steps 1.81 ms,
+    // 3 steps 1.88, 6 1.94, 10 2.23.  Six are enough for any size (1024 events2d streams, 386 MB: 6 steps 5.68 ms, 12 5.88: each row of
+    // steps leaves as a strided copy, whose runs get short).
+    // A short first step lets the computing start early, a long one follows, and they grow shorter to the end: where
+    // the way out takes nearly as long as the computing, a step's rows should be out before the next step's are.  (Many steps mean that
+    // the copies are what it takes: then they are alike, half of one at both ends.)
     std::vector<long long> cut;                      // segment index where step b starts; cut.back() = n_seg
     {
-        const long long edge = (n_seg >= 3 * pipe && pipe >= 2) ? pipe / 2 : 0;
-        long long pos = 0;
+        double step_us = 0.0;
+        long long rows_out = n_seg;
+        for (const LayerPlan& Q : net->L) {
+            rows_out = layer_rows_at_flush(Q, rows_out);
+            if (Q.l.kind == IDF_CONV) step_us += 5.0 + 5.0 * std::min(1.0, (double)Q.w_packed.size() / 150e3);
+        }
+        const double copy_us = ((double)seg_bytes * n_seg + (double)orow_bytes * net->n_streams * rows_out) / 55e3;
+        const double x = step_us > 0.0 ? std::sqrt(copy_us / step_us) : 0.0;
         cut.push_back(0);
-        if (edge) { pos = edge; cut.push_back(pos); }
-        while (pos < n_seg - edge) { pos = std::min<long long>(pos + pipe, n_seg - edge); cut.push_back(pos); }
-        if (edge) cut.push_back(n_seg);
-        if (cut.size() < 2) cut.push_back(n_seg);
+        if (x >= 1.0 && n_seg >= 21) {
+            const int n = (int)std::max(3.0, std::min({x + 0.3, 6.0, n_seg / 7.0}));     // (not fewer than seven rows or so to a step)
+            const bool few = n < 6;
+            const double mid = few ? 1.4 : 1.0, late = few ? 0.75 : 1.0, last = few ? 0.4 : 0.5, total = 0.5 + mid * (n - 3) + late + last;
+            double w = 0.5;
+            for (int k = 1; k < n; ++k) {
+                cut.push_back((long long)(n_seg * w / total));
+                w += k == n - 2 ? late : mid;
+            }
+        } else {
+            // little to copy: half a row block to a step, half of that first and last when there are steps enough
+            const long long pipe = net->row_block >= 2 ? net->row_block / 2 : 1;
+            const long long edge = (n_seg >= 3 * pipe && pipe >= 2) ? pipe / 2 : 0;
+            long long pos = 0;
+            if (edge) { pos = edge; cut.push_back(pos); }
+            while (pos < n_seg - edge) { pos = std::min<long long>(pos + pipe, n_seg - edge); if (pos < n_seg) cut.push_back(pos); }
+        }
+        cut.push_back(n_seg);
     }
     const long long nb = (long long)cut.size() - 1;
     if (!net->copy_in) {
@@ -1332,9 +1359,6 @@ int idf_run_host(idf_net* net, const void* h_segments, int n_seg, void* d_segmen
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return fail(IDF_ERR_CUDA, "cudaEventCreate failed");
         net->order_events.push_back(e);
     }
-    const LayerPlan& P = net->L.back();
-    const size_t seg_bytes = (size_t)net->n_streams * net->in_w * net->in_c * elem_size(net->L[0].in_elem);
-    const size_t orow_bytes = (size_t)P.out_w * P.out_c * elem_size(P.out_elem);
     const size_t opitch = (size_t)out_capacity_rows * orow_bytes;
     cudaError_t e = cudaEventRecord(net->order_events[0], net->stream);      // earlier work on the caller's stream comes first
     if (e == cudaSuccess) e = cudaStreamWaitEvent(net->copy_in, net->order_events[0], 0);
