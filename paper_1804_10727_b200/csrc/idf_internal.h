@@ -225,6 +225,7 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
                   int out_esize, int pooled, int pair, TcPlan* p);
 int tc_weight_slot(int ky, int kx, int Kh, int stride);
 int tc_encode_weights(const TcPlan& p, int dtype, const void* d_w, int taps, int Cin, int Cout, void* map_out);
+cudaError_t launch_ring_copy(void* dst, const void* src, long long words, cudaStream_t st);   // words: a multiple of four
 cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const void* w_map, int n_in_rows,
                            unsigned int* status, cudaStream_t st);
 

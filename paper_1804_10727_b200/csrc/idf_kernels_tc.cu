@@ -1054,8 +1054,7 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const 
     }
     t.ring_in = a.ring;
     if (t.n_chunks > 1 && a.r0 > 0) {
-        const size_t ring_bytes = (size_t)a.ring_rows * a.S * a.Wout * a.Cout * 4;
-        cudaError_t ce = cudaMemcpyAsync(a.ring_scratch, a.ring, ring_bytes, cudaMemcpyDeviceToDevice, st);
+        cudaError_t ce = launch_ring_copy(a.ring_scratch, a.ring, (long long)a.ring_rows * a.S * a.Wout * a.Cout, st);
         if (ce != cudaSuccess) return ce;
         t.ring_in = a.ring_scratch;
     }

@@ -353,7 +353,7 @@ cudaError_t launch_conv_time(const ConvArgs& a, const TimePlan& p, int dtype, co
     if (n_tt > 1 && t.carried) {
         // rows begun by an earlier block and rows left open by this one may share a ring slot and lie in different CTAs
         if (!a.ring_scratch) return cudaErrorNotSupported;
-        cudaError_t ce = cudaMemcpyAsync(a.ring_scratch, a.ring, (size_t)a.ring_rows * a.S * a.Cout * 4, cudaMemcpyDeviceToDevice, st);
+        cudaError_t ce = launch_ring_copy(a.ring_scratch, a.ring, (long long)a.ring_rows * a.S * a.Cout, st);
         if (ce != cudaSuccess) return ce;
         t.ring_in = a.ring_scratch;
     }
