@@ -56,7 +56,9 @@ inline size_t elem_size(int e) { return e == E_F32 || e == E_I32 ? 4 : (e == E_B
 // Row bookkeeping (0-based): input row r reaches output rows o with 0 <= r + pad - o*stride < Kh
 // through tap ky = r + pad - o*stride; row o is complete once input row o*stride - pad + Kh - 1 has
 // been applied (or at flush if only bottom padding is missing); its ring slot is o % ring_rows.
-// A free ring slot holds zeros; the state excludes the bias, which joins at emission.
+// A free ring slot may hold what its last row left there: whoever begins a row does not read its slot.  Only layers that report
+// their events (event scatter) start rows from what the slot holds; every kernel that serves them leaves a freed slot zero.
+// The state excludes the bias, which joins at emission.
 struct ConvArgs {
     const void* in;        // input rows of this block: [r - r0][S][Win][Cin]
     long long in_stream_elems;   // elements from one stream's row to the next (0: Win*Cin)

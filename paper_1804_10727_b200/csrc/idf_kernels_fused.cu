@@ -147,6 +147,9 @@ __device__ __forceinline__ bool fused_feed(const FusedArgs& a, int i, const type
     for (int ky = c.ph; ky < Kh; ky += stride) ++nt;
     if (nt > c.hi_sat + 1) nt = c.hi_sat + 1;
     const bool completes = c.phf == 0 && c.tf_neg == 0;      // ... and the oldest row reached then has its last tap
+    // The newest row begins with its tap 0, in a slot that may hold what an earlier row left (the per-layer kernels do not clear the
+    // slots they empty): it starts from 0.  (Rows begun by input row 0 with a later tap find slots as the reset left them.)
+    const bool begins = c.ph == 0;
     const int Cq = Cin >> 2;
     const bool quads = (Cin & 3) == 0 && !count && wq_off >= 0;
     if (nt <= FUSED_TAPS && (quads || Cin <= 4)) {
@@ -174,6 +177,7 @@ __device__ __forceinline__ bool fused_feed(const FusedArgs& a, int i, const type
                     if (slot < 0) slot += ring_rows;
                     at[j] = (slot * G + g) * row_elems + x * Cout + co;
                     old[j] = ring[at[j]];
+                    if (j == 0 && begins) old[j] = 0;
                     acc[j] = 0;
                 }
                 const TS b = bias ? bias[co] : (TS)0;
@@ -213,7 +217,7 @@ __device__ __forceinline__ bool fused_feed(const FusedArgs& a, int i, const type
 #pragma unroll
                 for (int j = 0; j < FUSED_TAPS; ++j) {
                     const TS s = old[j] + acc[j];
-                    const bool frees = completes && j == nt - 1;               // the slot is free for the row ring_rows further on
+                    const bool frees = completes && j == nt - 1;               // (left zero: the event scatter starts its rows from the ring)
                     if (j < nt) ring[at[j]] = frees ? (TS)0 : s;
                     if (j == nt - 1) done = s;
                 }
@@ -244,7 +248,7 @@ __device__ __forceinline__ bool fused_feed(const FusedArgs& a, int i, const type
                 }
                 TS* cp = ring + (slot * G + g) * row_elems + x * Cout + co;
                 if (--slot < 0) slot += ring_rows;
-                const TS s = *cp + acc;
+                const TS s = (j == 0 && begins ? (TS)0 : *cp) + acc;
                 if (completes && j == nt - 1) {
                     rowbuf[e] = fused_act(s, bias ? bias[co] : (TS)0, relu, shift, round_bf16);
                     *cp = 0;
