@@ -21,6 +21,7 @@
 // thread: 521 us there, but 61 us per push on the small launches.
 #include "../../include/idf.h"
 #include "idf_ptx.h"
+#include "idf_time_tiles.h"
 
 namespace idf {
 
@@ -31,9 +32,6 @@ namespace {
 constexpr int TIME_GROUPS = 4;
 constexpr int TIME_THREADS = 32 * (2 + 4 * TIME_GROUPS + 1);
 constexpr int TIME_W_WARP = 2 + 4 * TIME_GROUPS;
-constexpr int TIME_SB = 8, TIME_TM = 16;     // streams and output rows of an M tile
-constexpr int TIME_MAX_W = 40;               // weight tiles in shared memory
-constexpr size_t TIME_SMEM = 226304;         // dynamic shared memory per CTA (227 KB less the static part)
 
 struct TimeArgs {
     const void* bias;
@@ -317,36 +315,18 @@ cudaError_t launch_conv_time(const ConvArgs& a, const TimePlan& p, int dtype, co
     t.out_row_stride = a.out_row_stride; t.out_stream_stride = a.out_stream_stride; t.out_row_first = a.o_begin - a.out_row_base;
     t.out_elems = a.out_elems; t.ring_elems = a.ring_elems;
     t.S = a.S; t.Cout = a.Cout; t.Kh = a.Kh; t.stride = a.stride; t.relu = a.relu; t.shift = a.shift; t.out_elem = a.out_elem;
-    t.out_wide = ((uintptr_t)a.out & 31) == 0 && (dtype == 1 || a.Cout % 32 == 0);
     t.n_rows = (int)(a.o_end - a.o_begin); t.done_rel = (int)(a.done_end - a.o_begin);
     t.base_ty = (int)(a.r0 + a.pad - a.o_begin * a.stride); t.carried = a.r0 > 0;
     t.ring_slot0 = (int)(a.o_begin % a.ring_rows); t.ring_rows = a.ring_rows;
     t.KB = p.KB; t.n_kb = p.n_kb; t.swb = p.swb;
     t.n_g = (a.S + TIME_SB - 1) / TIME_SB;
-    // Tile sizes.  128 outputs per MMA run at the pipe's full rate and four M tiles amortise a weight tile; where a launch has too few
-    // items for the SMs, channel slices are narrowed (the weights are what a lone CTA waits for).  Up to 64 rows are one item per
-    // stream group whatever its size: rows taken from the ring and rows parked in it then meet in one CTA.
-    int N = a.Cout;
-    while (N > 128) N = N % 32 == 0 ? N / 2 : 16;
-    if (a.Cout % N != 0 || N % 16 != 0) N = 16;
-    const long long big_items = (long long)t.n_g * ((t.n_rows + 63) / 64);
-    while (N > 32 && N % 32 == 0 && big_items * (a.Cout / N) < 100) N /= 2;
-    int MT = (t.n_rows + TIME_TM - 1) / TIME_TM;
-    if (MT > 4) MT = 4;
-    const size_t w_bytes = ((size_t)N * p.swb + 1023) / 1024 * 1024;
-    auto window = [&](int mt) { return (mt * TIME_TM - 1) * a.stride + a.Kh; };
-    auto a_bytes = [&](int mt) { return ((size_t)window(mt) * TIME_SB * p.swb + 1023) / 1024 * 1024; };
-    while (MT > 1 && (window(MT) > 256 || 1024 + 2 * a_bytes(MT) + 3 * w_bytes > TIME_SMEM)) --MT;
-    const int n_tiles = a.Kh * p.n_kb;
-    int n_w = (int)((TIME_SMEM - 1024 - 2 * a_bytes(MT)) / w_bytes);
-    if (n_w > TIME_MAX_W) n_w = TIME_MAX_W;
-    t.resident = n_w >= n_tiles;
-    t.n_w = t.resident ? n_tiles : (n_w > 8 ? 8 : n_w);
-    t.N = N; t.n_nt = a.Cout / N; t.MT = MT; t.window = window(MT);
-    t.a_bytes = (int)a_bytes(MT); t.w_bytes = (int)w_bytes;
+    const TimeTiles tiles = time_tiles(dtype, a.S, t.n_rows, a.Cout, a.Kh, a.stride, p.swb, p.n_kb);
+    const int N = tiles.N, MT = tiles.MT;
+    t.N = N; t.n_nt = a.Cout / N; t.MT = MT; t.window = tiles.window; t.resident = tiles.resident; t.n_w = tiles.n_w;
+    t.a_bytes = (int)tiles.a_bytes; t.w_bytes = (int)tiles.w_bytes;
     t.n_sets = 2 * MT * N <= 512 ? 2 : 1;
-    t.cparts = MT == 1 ? 4 : (MT == 2 ? 2 : 1);
-    while (t.cparts > 1 && (N % (16 * t.cparts)) != 0) t.cparts /= 2;
+    t.cparts = tiles.cparts;
+    t.out_wide = ((uintptr_t)a.out & 31) == 0 && tiles.wide;
     const int n_tt = (t.n_rows + MT * TIME_TM - 1) / (MT * TIME_TM);
     if ((long long)n_tt * t.n_g > 0x3fffffffLL) return cudaErrorNotSupported;
     t.n_items = n_tt * t.n_g;

@@ -27,6 +27,11 @@ CASES = [
     ("i8_64_128", "i8", c1(64, 128, 9), 100, 10),
     ("i8_128_80", "i8", c1(128, 80, 3, 1, 1, 0), 65, 5),
     ("i8_32_144_s4", "i8", c1(32, 144, 9, 4), 130, 6),            # channel slices of 16
+    ("i8_64_96", "i8", c1(64, 96, 5), 77, 4),                     # slices of 48, some of them between 32-byte boundaries
+    ("i8_64_96_many", "i8", c1(64, 96, 3, 1, 1), 100, 820),       # slices of 96, also in shares of 48
+    ("i8_32_160", "i8", c1(32, 160, 3, 1, 1), 80, 9),             # of 80
+    ("i8_32_192", "i8", c1(32, 192, 3, 1, 1, 0), 66, 7),          # of 96 and 48
+    ("i8_32_224", "i8", c1(32, 224, 5, 2, 2), 140, 5),            # of 112
 ]
 
 
