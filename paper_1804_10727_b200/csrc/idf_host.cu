@@ -923,7 +923,8 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                 };
                 // Groups of g positions: tap kx lies at position (kx + shift) of a run of groups that starts x_pad groups to the
                 // left.  The last group of a row may reach into the next stream's row, or past the buffer: only where no output
-                // reads there (its weights are zero), the buffer is the library's own and any bits are a number (int8).
+                // reads there (its weights are zero), the buffer is the library's own and any bits are a number (int8).  Nor may bf16
+                // positions of the row itself meet a zero weight: an infinity or a NaN would reach outputs that do not read it.
                 int g = sx > 1 ? sx : ((size_t)l.cin * es == 16 ? 2 : 1), shift = 0;
                 bool planned = false;
                 if (g > 1 && w > 1 && ((size_t)w * l.cin * es) % 16 == 0) {
@@ -933,7 +934,8 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                     const int x_kw = (l.kw + shift + g - 1) / g;
                     const int whole = w / g, x_win = pair ? w : (need <= whole * g ? whole : (w + g - 1) / g);
                     const bool spill = !pair && x_win * g > w;
-                    if (!spill || (need <= w && i > 0 && spec->dtype == IDF_I8_I32))
+                    const bool zero_taps = shift > 0 || x_kw * g != l.kw;
+                    if (spec->dtype == IDF_I8_I32 ? !spill || (need <= w && i > 0) : !spill && !zero_taps)
                         planned = plan_as(x_win, g * l.cin, x_kw, 1, x_pad, pair);
                 }
                 if (!planned) { g = 1; shift = 0; planned = plan_as(w, l.cin, l.kw, sx, px, 0); }
