@@ -54,7 +54,7 @@ struct WinArgs {
     int n_in, n_rows, done_rel, base_ty, carried;      // input rows, visited output rows, emitted ones; tap ky of visited row o reads
                                  // input row o*stride + ky - base_ty; carried: rows with o*stride < base_ty were begun by an earlier block
     int ring_slot0, ring_rows;   // ring slot of visited row 0
-    int S, Win, Wout, Cin, Cout, Kh, stride, stride_x, pad_x, relu, shift, out_elem;
+    int S, Win, Wout, Cin, Cout, Kh, Kw, stride, stride_x, pad_x, relu, shift, out_elem;
     int P, nxw, ncol, n_tiles;   // outputs per window, windows per row, windows per output row of all streams, tiles of 128
     int run_words;               // words of a tap row's run
     int swb, ksteps, N;
@@ -120,6 +120,53 @@ struct WinWalk {
         return true;
     }
 };
+
+// A window is one row of A for all its outputs: an infinity or a NaN in it meets the zeros of B and turns the sums of outputs that do
+// not read it into NaN - in all Cout columns, so a look at the first of 16 finds them.  Such 16 columns (k-th of the window; bf16 layers) are
+// worked out here instead, one by one, from the output's own taps: added to what the ring holds, parked or emitted.  A call, by the thread
+// concerned, behind the look: inlined, or with the sums put back in tensor memory, it cost the launches without such values 1-5 %
+// (vgg2d one row per push 9.30 ms without any of it, 9.35 so, 9.41-9.77 the other ways; one push 1.35, 1.35, 1.36-1.37).
+template <int AX>
+__device__ __noinline__ void own_taps_only(const WinArgs& a, uint32_t sW, int k, int s, int xw, int step)
+{
+    const __nv_bfloat16* in = (const __nv_bfloat16*)a.in;
+    const int p = 16 * k / a.Cout, o = AX == 0 ? step : step * a.P + p;
+    const int x = AX == 0 ? xw * a.P + p : 0, ty = o * a.stride - a.base_ty;            // ty: the first tap's input row
+    const bool emit = o < a.done_rel, carried = a.carried && ty < 0;
+    float* ring = (float*)a.ring;
+#pragma unroll 1
+    for (int n = 16 * k; n < 16 * k + 16; ++n) {
+        const int co = n - p * a.Cout;
+        const uint32_t phase = a.swb == 128 ? (uint32_t)(n & 7) : (a.swb == 64 ? (uint32_t)((n >> 1) & 3) : (uint32_t)((n >> 2) & 1));
+        float sum = 0.f;
+#pragma unroll 1
+        for (int ky = 0; ky < a.Kh; ++ky) {
+            if ((unsigned)(ty + ky) >= (unsigned)a.n_in) continue;
+#pragma unroll 1
+            for (int i = 0; i < a.Kw * a.Cin; ++i) {
+                const int e = AX == 0 ? (x * a.stride_x - a.pad_x) * a.Cin + i : i;     // value of the stream's row
+                if ((unsigned)e >= (unsigned)(a.Win * a.Cin)) continue;
+                const long long at = ((long long)(ty + ky) * a.S + s) * a.Win * a.Cin + e;
+                if (!IDF_OK_AT(a.status, at, a.in_elems)) continue;
+                const uint32_t b = 2u * (uint32_t)(AX == 0 ? 2 * ky * a.run_words + p * a.stride_x * a.Cin + i : (p * a.stride + ky) * a.Cin + i);
+                unsigned short w;
+                asm volatile("ld.shared.u16 %0, [%1];" : "=h"(w) : "r"(sW + (uint32_t)(n * a.swb) + (((b >> 4) ^ phase) << 4) + (b & 15u)));
+                sum = fmaf(__bfloat162float(__ushort_as_bfloat16(w)), __bfloat162float(in[at]), sum);
+            }
+        }
+        const long long ri = ((long long)((a.ring_slot0 + o) % a.ring_rows) * a.S + s) * a.Wout * a.Cout + (long long)x * a.Cout + co;
+        if ((carried || !emit) && !IDF_OK_AT(a.status, ri, a.ring_elems)) continue;
+        if (carried) sum += ring[ri];
+        if (!emit) { ring[ri] = sum; continue; }
+        if (a.bias) sum += ((const float*)a.bias)[co];
+        if (a.relu) sum = a.out_elem == E_BF16 ? (sum < 0.f ? 0.f : sum) : fmaxf(sum, 0.f);      // (as emit16f)
+        const long long at = (a.out_row_first + o) * a.out_row_stride + (long long)s * a.out_stream_stride + (long long)x * a.Cout + co;
+        if (!IDF_OK_AT(a.status, at, a.out_elems)) continue;
+        if (a.out_elem == E_BF16) ((__nv_bfloat16*)a.out)[at] = __float2bfloat16_rn(sum);
+        else ((float*)a.out)[at] = sum;
+    }
+}
+__device__ __forceinline__ bool is_nan(uint32_t v) { return __uint_as_float(v) != __uint_as_float(v); }
 
 // AX 0: a window runs along x; 1: along the rows (1D nets).  RWT: words of a run of a 3-row layer, known at compile time
 // (the whole window is then fetched one step ahead and leaves in 16-byte stores), or 0.
@@ -450,12 +497,18 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                             if (lo) st_global_v4(d0, pk);
                             if (hi) st_global_v4(d1, pk + 4);
                         }
-                    } else if (a.out_elem == E_BF16) {
-                        if (lo) emit16f<E_BF16>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
-                        if (hi) emit16f<E_BF16>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
                     } else {
-                        if (lo) emit16f<E_F32>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
-                        if (hi) emit16f<E_F32>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
+                        if (a.out_elem == E_BF16) {
+                            if (lo) emit16f<E_BF16>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
+                            if (hi) emit16f<E_BF16>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
+                        } else {
+                            if (lo) emit16f<E_F32>(v, (const float*)b_lo, a.relu, d0, a.out_wide);
+                            if (hi) emit16f<E_F32>(v + 16, (const float*)b_hi, a.relu, d1, a.out_wide);
+                        }
+                        const bool odd_lo = lo && is_nan(v[0]), odd_hi = hi && is_nan(v[16]);
+                        if (odd_lo || odd_hi)
+#pragma unroll 1
+                            for (int h = odd_lo ? 0 : 1; h < (odd_hi ? 2 : 1); ++h) own_taps_only<AX>(a, sW, 2 * k + h, s, xw, step);
                     }
                 }
                 first = k - k_part - n_chunk;
@@ -484,6 +537,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
                     __syncwarp();
                     tmem_ld<16>(trow + c, v);
                     if (!have) continue;
+                    if (DT == 1 && is_nan(v[0])) { own_taps_only<AX>(a, sW, k, s, xw, step); continue; }
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
                         v[j] = DT == 1 ? __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(r[j])) : v[j] + r[j];
@@ -623,7 +677,7 @@ cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, cons
     t.n_in = (int)(a.r1 - a.r0); t.n_rows = (int)(a.o_end - a.o_begin); t.done_rel = (int)(a.done_end - a.o_begin);
     t.base_ty = (int)(a.r0 + a.pad - a.o_begin * a.stride); t.carried = a.r0 > 0;
     t.ring_slot0 = (int)(a.o_begin % a.ring_rows); t.ring_rows = a.ring_rows;
-    t.S = a.S; t.Win = a.Win; t.Wout = a.Wout; t.Cin = a.Cin; t.Cout = a.Cout; t.Kh = a.Kh; t.stride = a.stride;
+    t.S = a.S; t.Win = a.Win; t.Wout = a.Wout; t.Cin = a.Cin; t.Cout = a.Cout; t.Kh = a.Kh; t.Kw = a.Kw; t.stride = a.stride;
     t.stride_x = a.stride_x; t.pad_x = a.pad_x; t.relu = a.relu; t.shift = a.shift; t.out_elem = a.out_elem;
     t.P = p.P; t.nxw = p.nxw; t.run_words = p.run_words; t.swb = p.swb; t.ksteps = p.ksteps; t.N = p.N;
     t.inv_c16 = (65536u + a.Cout / 16 - 1) / (a.Cout / 16);
