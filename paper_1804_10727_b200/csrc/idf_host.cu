@@ -1149,7 +1149,12 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
             if (P.l.kind == IDF_CONV && P.tc.ok) biggest = std::max(biggest, P.state_bytes_all);
         if (biggest) { net->ring_scratch_off = off; off = align_up(off + biggest); }
     }
-    net->workspace_bytes = off + 1024;      // (a group of positions may reach a little past the last row of a buffer)
+    // the last group of positions of a full buffer's last row may reach past it
+    size_t spill = 1024;
+    for (const auto& P : net->L)
+        if (P.tc.ok && !P.unfold && !P.tc.pair && (long long)P.x_win * P.x_cin > (long long)P.in_w * P.in_c)
+            spill = std::max(spill, ((size_t)P.x_win * P.x_cin - (size_t)P.in_w * P.in_c) * elem_size(P.in_elem));
+    net->workspace_bytes = align_up(off + spill);
     *out = net;
     return IDF_OK;
 }

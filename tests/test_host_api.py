@@ -153,3 +153,22 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(idf, "LIB_PATH", tmp_path / "libidf.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         idf.lib()
+
+
+def test_workspace_covers_the_last_group_of_positions():
+    """An x-strided int8 layer takes positions in groups; at an odd width the last group of a buffer's last row reaches one position
+    past it.  That position lies in the workspace however many channels it has: the workspace that no stream accounts for (its size
+    extrapolated to 0 streams) is larger by it than at the next even width, beyond the 1024 bytes that are always there."""
+    cin = 2048
+    layers = (conv(16, cin, 1, shift=8), Layer(cin=cin, cout=16, kh=2, kw=1, stride=2, shift=8))
+    ws = [np.zeros((l.cout, l.kh, l.kw, l.cin), np.int8) for l in layers]
+
+    def beside_streams(width):
+        sizes = []
+        for S in (256, 512):                                    # (every buffer is then whole 256-byte blocks)
+            net = idf.Net("i8", layers, width, 16, S, ws, [None, None], row_block=16)
+            sizes.append(net.workspace_bytes)
+            net.close()
+        return 2 * sizes[0] - sizes[1]
+
+    assert 1024 + beside_streams(3) - beside_streams(4) >= cin
