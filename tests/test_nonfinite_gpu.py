@@ -25,6 +25,8 @@ CASES = [
     ("window_5x5_stride2", conv(2, 32, 5, stride=2, pad=2, relu=0), 16, 33, 4),
     ("window_1d", conv(1, 32, 9, one_d=True, relu=0), 203, 1, 130),
     ("window_1d_stride2", conv(1, 32, 9, stride=2, one_d=True, relu=0), 203, 1, 1030),
+    ("time_1d", conv(32, 32, 9, one_d=True, relu=0), 120, 1, 20),            # shifted views of whole rows: no zero weights
+    ("time_1d_stride2_pad", conv(64, 32, 9, stride=2, pad=4, one_d=True, relu=0), 120, 1, 20),
     ("window_1d_pad", conv(2, 48, 5, pad=2, one_d=True, relu=0), 50, 1, 3),
 ]
 
