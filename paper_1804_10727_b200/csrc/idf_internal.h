@@ -34,17 +34,23 @@ unsigned debug_flags();
 #ifdef __CUDACC__
 // Launch of a kernel that begins with griddepcontrol.wait: it may be scheduled while its predecessor in the stream drains.  (Every
 // kernel launched this way waits before it touches anything but parameters, so completion stays ordered along the whole stream.)
+// dependent = false: an ordinary launch (the kernel's wait is then a no-op).
 template <typename... P, typename... A>
-inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+inline cudaError_t launch_as(bool dependent, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = (debug_flags() & 8u) ? 0 : 1;      // 8: IDF_DEBUG_NO_PDL
+    cfg.attrs = attr; cfg.numAttrs = !dependent || (debug_flags() & 8u) ? 0 : 1;      // 8: IDF_DEBUG_NO_PDL
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    return launch_as(true, kernel, grid, block, smem, st, args...);
 }
 #endif
 

@@ -214,7 +214,15 @@ static cudaError_t launch_rows(const ConvArgs& a, cudaStream_t st)
     } else {
         int_begin = int_end = 0;
     }
-    return launch_pdl(conv_rows_kernel<TI, TW, TS, TO>, (unsigned)(blocks + int_blocks), 256, 0, st, a, int_begin, int_end, (unsigned)blocks);
+    // A dependent launch saves up to 3 us, but its blocks are placed while the previous kernel's still run, unevenly: where there are
+    // more of them than SMs, and each takes long, that costs more than it saves.  Measured on 420 layers, time of ordinary over dependent
+    // launches (mean; worst): up to 148 blocks 1.12 (0.86); more, below 192 multiply-adds per output 1.10 (0.88); 192-511 in at most one
+    // wave of eight blocks per SM 0.97 (0.74), in several 1.01 (0.87); 512 and more 0.96 (0.68; int8 128 -> 8 5x5, 235 blocks: 209 us
+    // ordinary, 334 dependent).
+    const int macs = a.Kh * a.Kw * a.Cin;
+    const long long all_blocks = blocks + int_blocks;
+    const bool dependent = all_blocks <= 148 || macs < 192 || (macs < 512 && all_blocks >= 148 * 8);
+    return launch_as(dependent, conv_rows_kernel<TI, TW, TS, TO>, (unsigned)(blocks + int_blocks), 256, 0, st, a, int_begin, int_end, (unsigned)blocks);
 }
 
 cudaError_t launch_conv_simple(const ConvArgs& a, int dtype, cudaStream_t st)
@@ -521,13 +529,17 @@ static cudaError_t launch_sparse_t(const ConvArgs& a, cudaStream_t st)
     const size_t ring_bytes = (size_t)a.ring_rows * a.Wout * a.Cout * sizeof(TS);
     const long long row_words = (long long)a.Wout * a.Cout;
     const int nthr = row_words >= 4096 ? SPARSE_MAX_THREADS : (row_words >= 1024 ? 256 : (row_words >= 512 ? 128 : 64));     // short rows: more, smaller CTAs per SM
+    // Dependent launches (see launch_rows) for short ones: few rows, and CTAs that are small or no more than SMs (1 -> 8 channels, 354
+    // streams of 232-wide rows one by one: 19 us ordinary, 27 dependent; 2 -> 64 stride 2, 79 streams, 22 rows: 172 and 190; rows pushed one
+    // by one into small CTAs: 5.5-6 and 4.2).
+    const bool dependent = a.r1 - a.r0 <= 16 && (nthr == 64 || a.S <= 148);
     if (ring_bytes <= conv_sparse_max_smem()) {
         auto k = conv_sparse_kernel<TI, TW, TS, TO, true>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes);
         if (e != cudaSuccess) return e;
-        return launch_pdl(k, a.S, nthr, ring_bytes, st, a);
+        return launch_as(dependent, k, a.S, nthr, ring_bytes, st, a);
     } else {
-        return launch_pdl(conv_sparse_kernel<TI, TW, TS, TO, false>, a.S, nthr, 0, st, a);
+        return launch_as(dependent, conv_sparse_kernel<TI, TW, TS, TO, false>, a.S, nthr, 0, st, a);
     }
 }
 
