@@ -520,6 +520,39 @@ void reach(const LayerPlan& P, long long lo, long long hi, long long* o_lo, long
     }
 }
 
+// Tiled or plain kernels for an eager net.  The tiled kernel has one block per group of streams, whose warps take a row's units one after
+// the other; the plain ones have a thread per unit but a launch per layer.  So few streams of wide rows with many channels, and 1D nets
+// (one position per stream: most lanes idle), are better off with the plain ones: bf16 2 -> 128 3x3, 4 streams of 224-wide rows 51 us a
+// push tiled, 15 plain; 1D 3 -> 128 k9, 64 streams 21 and 9.  The estimate (us a push) was fitted to 276 nets of one to three layers, error
+// 16 % tiled and 14 % plain; the choice costs 1.4 % against always the better one.
+bool eager_tiled_pays(const idf_net* net)
+{
+    const bool int_net = net->dtype == IDF_I8_I32;
+    const long long S = net->n_streams;
+    const int G0 = net->eager_G;
+    double tiled = G0 ? 2.9 : 0.0, plain = 4.25;
+    int below = 1;                                               // rows of the layer below that change
+    for (const LayerPlan& P : net->L) {
+        const int rows = P.e_window;
+        const double outs = (double)rows * S * P.out_w * P.out_c / (148.0 * 2048.0);      // threads of the plain kernels, in full chips
+        plain += 4.25 + 6.5 * outs;
+        if (!G0) tiled += 3.9;
+        if (P.l.kind == IDF_MAXPOOL2) {
+            tiled += 2.4;
+        } else {
+            const int G = G0 ? G0 : eager_tiled_group(net->n_streams, P.e_w_words, P.e_d_words, EAGER_SMEM_WORDS);
+            const int taps = std::min(P.l.kh, below), groups = int_net && P.in_c % 4 == 0 ? P.in_c / 4 : P.in_c;
+            const double macs = (double)taps * P.l.kw * P.in_c;
+            plain += 0.064 * macs + 0.033 * macs * outs;
+            const long long units = (long long)rows * ((G * P.out_w + 31) / 32) * (P.out_c / (P.out_c % 8 == 0 ? 8 : 4));
+            const double turns = (double)((units + 15) / 16) * (double)((S + 296LL * G - 1) / (296LL * G));
+            tiled += turns * (1.8 + 0.026 * taps * P.l.kw * groups) + 0.013 * P.e_w_words / 512.0;
+        }
+        below = rows;
+    }
+    return tiled <= 1.05 * plain;
+}
+
 // One layer of an eager step: launched at once by the plain kernels; the tiled kernel takes all layers of a step together where
 // they fit (`batch`: launch_eager_batch does it after the last one).
 cudaError_t launch_eager(idf_net* net, size_t i, EagerArgs& a, EagerNetArgs* batch)
@@ -1035,6 +1068,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
             net->eager_d_words = std::max(net->eager_d_words, P.e_d_words);
         }
         net->eager_G = net->L.size() <= EAGER_MAX_LAYERS ? eager_tiled_group(net->n_streams, net->eager_w_words, net->eager_d_words, EAGER_SMEM_WORDS) : 0;
+        if (net->eager_tiled && !eager_tiled_pays(net)) net->eager_tiled = 0;
         net->state_bytes_stream = 0;
         for (auto& P : net->L) {
             P.e_cap = P.e_window + 2;      // (a pooling layer above still reads the two rows below its oldest open pair)
