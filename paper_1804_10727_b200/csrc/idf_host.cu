@@ -938,7 +938,15 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                                      l.path != IDF_PATH_SPARSE && (size_t)taps * l.cin * es <= 128 &&
                                      (!P.use_sparse || (w > 1 && l.stride == 1));
             const bool prefer_thin = (debug_flags() & IDF_DEBUG_PREFER_THIN) != 0;
-            if (win_allowed && (!pool_next || P.use_sparse || prefer_thin) &&
+            // Not where positions are whole K steps already and the tensor-core kernels take them as they are: 1D layers, whose time tiles
+            // are better on blocks of rows (int8 32 -> 128 k3, one stream of 2000: 42 us by windows, 9 by time tiles; rows one by one 4.2 both),
+            // and 1x1 layers whose windows hold one output or have few columns (int8 128 -> 48, 176 streams of 90-wide rows, 160 rows: 629 and
+            // 190 us; bf16 32 -> 16, 235 x 112: 218 and 80).
+            const size_t pos_bytes = (size_t)l.cin * es;
+            const bool whole_steps = pos_bytes == 32 || pos_bytes == 64 || pos_bytes == 128;
+            const size_t most_p = whole_steps ? std::min<size_t>(256 / (size_t)std::min(l.cout, 256), 128 / pos_bytes) : 0;     // outputs of a window
+            const bool as_they_are = whole_steps && !P.use_sparse && !prefer_thin && (w == 1 || (taps == 1 && (most_p <= 1 || most_p * l.cout <= 32)));
+            if (win_allowed && !as_they_are && (!pool_next || P.use_sparse || prefer_thin) &&
                 win_make_plan(spec->dtype, net->n_streams, P.out_w, l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, w == 1, &P.win)) {
                 P.wwin_packed.resize(P.win.w_bytes);
                 win_pack_weights(P.win, spec->dtype, weights[i], l.cin, l.cout, l.kh, l.kw, l.stride, w == 1 ? 1 : l.stride, P.wwin_packed.data());
