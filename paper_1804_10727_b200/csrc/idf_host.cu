@@ -97,7 +97,7 @@ struct idf_net {
     size_t eager_in_off = 0;               // the pushed segment as words (the input layer's announcement)
     std::vector<LayerPlan> L;
     size_t workspace_bytes = 0, state_region_off = 0, state_region_bytes = 0, reset_bytes = 0, counters_off = 0, status_off = 0;
-    size_t ring_scratch_off = 0;           // room for a copy of the largest tensor-core layer's ring (row-chunked launches)
+    size_t ring_scratch_off = 0;           // room for a copy of the largest tensor-core layer's ring (launches whose CTAs read rows that others rewrite)
     size_t state_bytes_stream = 0;
     unsigned char* ws = nullptr;
     cudaStream_t stream = nullptr;
@@ -1188,7 +1188,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
     {
         size_t biggest = 0;
         for (auto& P : net->L)
-            if (P.l.kind == IDF_CONV && P.tc.ok) biggest = std::max(biggest, P.state_bytes_all);
+            if (P.l.kind == IDF_CONV && (P.tc.ok || P.win.ok)) biggest = std::max(biggest, P.state_bytes_all);
         if (biggest) { net->ring_scratch_off = off; off = align_up(off + biggest); }
     }
     // the last group of positions of a full buffer's last row may reach past it

@@ -19,7 +19,7 @@
 // Steps that exchange rows with the ring (begun by an earlier block, or left open by this one) are the same MMAs with
 // the missing input rows as zeros; the epilogue then adds what the ring holds and parks what stays open.  Where two
 // such rows can meet in one ring slot, those of a tile are one work item and a slot's words belong to one thread, which
-// takes the rows in order.  A freed slot is left zero where the event scatter shares the ring.  All else are independent work items, dealt round robin to one
+// takes the rows in order, or the carried rows are read from a copy of the ring.  A freed slot is left zero where the event scatter shares the ring.  All else are independent work items, dealt round robin to one
 // CTA per SM.  Layers that report their input events (Eq. 3: non-zero components) count them while the runs pass by.
 //
 // Measured on B200, against the kernels that served these layers before (event scatter on CUDA cores; one im2col row per
@@ -46,6 +46,7 @@ struct WinArgs {
     const void* in;              // input rows of the block: [n_in][S][Win][Cin]
     const void* bias;
     void* ring;
+    const void* ring_in;         // where the rows begun by earlier blocks are read: the ring, or a copy of it
     void* out;
     unsigned int* status;
     unsigned long long* events;  // count the non-zero input components here (int8 layers), or nullptr
@@ -156,7 +157,7 @@ __device__ __noinline__ void own_taps_only(const WinArgs& a, uint32_t sW, int k,
         }
         const long long ri = ((long long)((a.ring_slot0 + o) % a.ring_rows) * a.S + s) * a.Wout * a.Cout + (long long)x * a.Cout + co;
         if ((carried || !emit) && !IDF_OK_AT(a.status, ri, a.ring_elems)) continue;
-        if (carried) sum += ring[ri];
+        if (carried) sum += ((const float*)a.ring_in)[ri];
         if (!emit) { ring[ri] = sum; continue; }
         if (a.bias) sum += ((const float*)a.bias)[co];
         if (a.relu) sum = a.out_elem == E_BF16 ? (sum < 0.f ? 0.f : sum) : fmaxf(sum, 0.f);      // (as emit16f)
@@ -429,6 +430,7 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
         const int n_chunk = (a.part_cols + 31) >> 5;
         unsigned char* out = (unsigned char*)a.out;
         uint32_t* ring = (uint32_t*)a.ring;
+        const uint32_t* ring_in = (const uint32_t*)a.ring_in;
         const long long ring_row = (long long)a.Wout * a.Cout;
         bool ok = true;
         int t = 0, first = grp;                                                    // this group's first chunk in the step at hand
@@ -529,8 +531,8 @@ conv_win_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__
 #pragma unroll
                     for (int j = 0; j < 16; ++j) r[j] = 0u;
                     if (have && carried) {                                         // (in flight while the accumulator is waited for)
-                        ld_global_v8(ring + ri, *(uint32_t(*)[8])r);
-                        ld_global_v8(ring + ri + 8, *(uint32_t(*)[8])(r + 8));
+                        ld_global_v8(ring_in + ri, *(uint32_t(*)[8])r);
+                        ld_global_v8(ring_in + ri + 8, *(uint32_t(*)[8])(r + 8));
                     }
                     if (!waited) { waited = true; ok = wait_acc(); }
                     if (!ok) break;
@@ -669,7 +671,7 @@ cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, cons
     if (!p.ok || a.pool_fused || a.o_end <= a.o_begin) return cudaErrorNotSupported;
     if (((uintptr_t)a.out & 15) != 0) return cudaErrorNotSupported;
     WinArgs t{};
-    t.in = a.in; t.bias = a.bias; t.ring = a.ring; t.out = a.out; t.status = a.status;
+    t.in = a.in; t.bias = a.bias; t.ring = a.ring; t.ring_in = a.ring; t.out = a.out; t.status = a.status;
     t.events = count_events ? a.event_counter : nullptr;
     t.clear = count_events;
     t.out_row_stride = a.out_row_stride; t.out_stream_stride = a.out_stream_stride;
@@ -696,6 +698,20 @@ cudaError_t launch_conv_win(const ConvArgs& a, const WinPlan& p, int dtype, cons
     t.e1_begin = c1 == t.n_rows && c1 % rows_per_step == 0 ? t.n_steps : c1 / rows_per_step;
     if (t.e1_begin < t.e0_end) t.e0_end = t.e1_begin = t.n_steps;                   // every step exchanges rows with the ring
     t.ordered = t.n_rows > t.ring_rows && (t.e0_end > 0 || t.e1_begin < t.n_steps);
+    // An ordered item takes its steps one after the other, 4-5 us each where outputs have many channels.  Where that is what the launch
+    // waits for, the carried rows are read from a copy of the ring instead, and every step is an item of its own (the copy is a launch of
+    // 2-3 us).  1D steps are runs of P rows that share ring slots all over, two of them pay; 2D steps are rows, three: 450 thin layers, mean
+    // time against never copying 0.93 (1D 16 -> 128 k2, 152 streams in fives: 7.4 -> 2.9 ms; 1 -> 96 k3, 231 streams in 17s: 2.2 -> 0.96;
+    // audio1d frames 1.302 -> 1.238, 5 vgg2d streams in 29s 0.487 -> 0.476).  Above 2000 steps the copy is the longer part.
+    const int n_exchange = t.e0_end + (t.n_steps - t.e1_begin);
+    if (t.ordered && !t.clear && a.ring_scratch && n_exchange >= (p.one_d ? 2 : 3) && (long long)t.n_steps * t.n_tiles <= 2000) {
+        if (t.carried) {
+            cudaError_t ce = launch_ring_copy(a.ring_scratch, a.ring, (long long)a.ring_rows * a.S * a.Wout * a.Cout, st);
+            if (ce != cudaSuccess) return ce;
+            t.ring_in = a.ring_scratch;
+        }
+        t.ordered = 0;
+    }
     // steps per work item: about four items per CTA, at most 16 (neighbouring rows share their input through the L1)
     const int n_free = t.ordered ? t.e1_begin - t.e0_end : t.n_steps;
     const long long R = (long long)n_free * t.n_tiles / (148 * 4);
