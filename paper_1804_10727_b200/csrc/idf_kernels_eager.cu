@@ -13,8 +13,9 @@
 // A push of one segment touches, in every layer, exactly the rows whose receptive field contains
 // that segment; the host works the row intervals out and launches one kernel per layer.
 //
-// Two sets of kernels: plain ones (a thread per unit, any shape and type), and tiled ones for the shapes that
-// eager_tiled_ok accepts, which keep no h ring for conv layers and pass d on in the activation type.
+// Two sets of kernels: plain ones (a thread per unit, any shape and type), and a tiled one for nets whose layers
+// eager_tiled_words accepts and for which it is the faster (eager_tiled_pays), which keeps no h ring for conv layers and
+// passes d on in the activation type.
 #include "../../include/idf.h"
 #include "idf_internal.h"
 

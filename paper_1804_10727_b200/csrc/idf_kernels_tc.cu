@@ -309,7 +309,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // The weights come first: they do not depend on earlier kernels of the stream (their fetch overlaps the
         // previous kernel's tail under programmatic dependent launch), and a launch that brings a single row has
         // little else to hide their latency behind.  One copy per K block carries all taps of the CTA's channel
-        // slice (the parameters are stored tap by tap in the order the stacked tiles want, see tc_pack_weights).
+        // slice (the parameters are stored tap by tap in the order the stacked tiles want, see tc_weight_slot).
         mbar_init(bar_w, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         mbar_expect_tx(bar_w, (uint32_t)(taps * a.n_kb) * w_tile_bytes);
@@ -840,7 +840,6 @@ bool make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, i
     // a launch that emits pooled rows stages half a tile of positions
     const int stage_rows = pooled ? 64 : 128;
     int best = 0, best_units = -1;
-    const bool wide_for_1d = true;
     for (int nt = 256; nt >= 16; nt >>= 1) {
         if (Cout % nt) continue;
         // TMEM slots.  An epilogue group tells the uses of a slot apart by the parity of its barrier, so it must have seen the row that
@@ -857,7 +856,7 @@ bool make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh, i
         // 1D nets come in long blocks of rows, which row chunks spread over the SMs: there the widest tile that fits
         // wins, because every channel slice fetches the Δ-rows again (audio1d's 128-channel layers with 16-channel
         // tiles moved 4.2 GB per layer through the L2)
-        if (Win == 1 && wide_for_1d) { best = nt; break; }
+        if (Win == 1) { best = nt; break; }
         if (units > best_units) { best_units = units; best = nt; }
     }
     if (!best) return false;
