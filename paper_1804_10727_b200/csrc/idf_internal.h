@@ -242,6 +242,7 @@ struct WinPlan {
     int ok = 0;
     int one_d = 0;           // the window runs along the rows (1D nets), else along x
     int P = 0;               // outputs per window
+    int widest = 0;          // the same before windows are narrowed for launches of few tiles
     int nxw = 0;             // windows per row
     int run_words = 0;       // 32-bit words of one tap row's run
     int n_words = 0;         // words of a whole window row (at most 32)

@@ -612,6 +612,7 @@ bool win_make_plan(int dtype, int S, int Wout, int Cin, int Cout, int Kh, int Kw
     int P = 256 / Cout, run = 0;
     while (P >= 1 && words(P, &run) > WIN_MAX_WORDS) --P;
     if (P < 1) return false;
+    p->widest = P;
     if (one_d) {
         while (P > 2 && ((long long)S + 127) / 128 * (64 / P) < 64) P = (P + 1) / 2;
     } else {

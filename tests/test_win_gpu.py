@@ -23,7 +23,7 @@ CASES = [
     ("bf16_1d_few", "bf16", (conv(2, 48, 5, pad=2, one_d=True),), 50, 1, 3),
     ("bf16_1d_all_exchange", "bf16", (conv(1, 128, 9, one_d=True),), 64, 1, 19),    # short blocks: every row meets the ring, carried ones from a copy
     ("i8_1d_all_exchange", "i8", (conv(8, 96, 9, pad=4, one_d=True),), 64, 1, 14),
-    ("bf16_5x5_all_exchange", "bf16", (conv(2, 16, 5, pad=2),), 24, 27, 40),
+    ("bf16_5x5_all_exchange", "bf16", (conv(2, 32, 5, pad=2),), 24, 27, 40),
     ("i8_1d", "i8", (conv(3, 16, 9, stride=3, one_d=True, path=1),), 100, 1, 140),
 ]
 
