@@ -337,7 +337,9 @@ typedef enum {
     IDF_DEBUG_NO_FUSED = 32,        /* never the single launch over all layers (state in shared memory)       */
     IDF_DEBUG_FORCE_FUSED = 64,     /* ... always, where a stream's state fits (by default: small pushes only) */
     IDF_DEBUG_NO_TILED_EAGER = 128, /* eager emission: the plain kernels for every shape                      */
-    IDF_DEBUG_NO_TIME_TILES = 256   /* 1D tensor-core layers on the row-ring kernel                           */
+    IDF_DEBUG_NO_TIME_TILES = 256,  /* 1D tensor-core layers on the row-ring kernel                           */
+    IDF_DEBUG_NO_CTA_PAIRS = 512,   /* wide layers on the row-ring kernel (1D ones as without CTA pairs)      */
+    IDF_DEBUG_FORCE_CTA_PAIRS = 1024 /* every launch of a layer that the CTA-pair kernel can take goes there  */
 } idf_debug_flag;
 int idf_set_debug_flags(unsigned int flags);
 

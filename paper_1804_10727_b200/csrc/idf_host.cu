@@ -48,6 +48,7 @@ struct LayerPlan {
     long long tc_launches = 0;
     std::vector<unsigned char> wq_packed;      // int nets, Cin % 4 == 0: [Kh][Kw][Cin/4][Cout] words of four int8 (all-layers launch)
     size_t wq_off = 0;
+    PairPlan pair;                             // wide layers on CTA pairs (pair.ok; weights: wtc_packed)
     TimePlan time;                             // 1D layers on the tensor cores (time.ok; weights: wtc_packed)
     WinPlan win;                               // thin layers: the window kernel (win.ok)
     std::vector<unsigned char> wwin_packed;    // its banded weight matrix
@@ -157,6 +158,19 @@ void as_planned(const LayerPlan& P, ConvArgs* t)
     t->Win = P.x_win; t->Cin = P.x_cin; t->Kw = P.x_kw; t->stride_x = P.x_stride; t->pad_x = P.x_pad;
 }
 
+// Whether a launch is one for the CTA-pair kernel.
+// Measured on 650 random layers against the row-ring kernel (mean time ring / pairs): 2D layers of a multiple of 128 output channels, all rows in one
+// launch 1.5 (the worst 0.91), 8 to 12 rows at a time 1.25, fewer 0.8 to 0.9 (such a launch mostly waits for the rows it exchanges with
+// the ring).  Of a multiple of 64 channels, two K blocks and more 1.5; with one K block 1.3, but 0.54 where the launch is large (int8
+// 64 -> 64, 2048 streams: MMAs of 64 columns wait for operands); of other channel counts 1.2 with some at 0.5.
+bool by_pairs(const LayerPlan& P, const ConvArgs& a)
+{
+    if (!P.pair.ok || a.r1 <= a.r0 || (debug_flags() & IDF_DEBUG_NO_CTA_PAIRS)) return false;
+    if (debug_flags() & IDF_DEBUG_FORCE_CTA_PAIRS) return true;
+    if (a.r1 - a.r0 < 8) return false;
+    return a.Cout % 128 == 0 || (a.Cout % 64 == 0 && P.pair.n_kb >= 2);
+}
+
 // Enqueue one layer on n_in input rows found at in_ptr (slots 0..n_in-1).  With `flush` (n_in == 0)
 // the layer learns that its input has ended and completes the rows that wait only for bottom padding.
 // Rows it emits go to the next layer's buffer starting at slot `out_slot` (or to the caller's output
@@ -250,6 +264,12 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
         const bool by_time = o_end - o_begin <= 256 || S * 5 < tiles * 4;
         if (ce == cudaErrorNotSupported && P.time.ok && by_time && P.tc.ok && n_in > 0) {
             ce = launch_conv_time(a, P.time, net->dtype, net->ws + P.wtc_off, net->stream);
+            if (ce == cudaSuccess) P.tc_launches += 1;
+        }
+        if (ce == cudaErrorNotSupported && by_pairs(P, a)) {
+            ConvArgs t = a;
+            as_planned(P, &t);
+            ce = launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
         if (ce == cudaErrorNotSupported && P.tc.ok && !P.use_sparse && n_in > 0) {
@@ -373,7 +393,9 @@ int launch_conv_pool(idf_net* net, size_t i, const void* in_ptr, long long n_in,
         net->launches += 1;
         t.in = net->ws + P.unf_off;
     }
-    ce = launch_conv_tc(t, P.tc_pool, net->dtype, P.w_map_pool, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
+    ce = by_pairs(P, a) ? launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream) : cudaErrorNotSupported;
+    if (ce == cudaErrorNotSupported)
+        ce = launch_conv_tc(t, P.tc_pool, net->dtype, P.w_map_pool, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
     if (net->timing) {
         if (ce == cudaSuccess) {
             cudaEventRecord(ev_b, net->stream);
@@ -833,7 +855,8 @@ const char* idf_last_error(void) { return g_err.c_str(); }
 
 int idf_set_debug_flags(unsigned int flags)
 {
-    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED | IDF_DEBUG_NO_TILED_EAGER | IDF_DEBUG_NO_TIME_TILES))
+    if (flags & ~(unsigned)(IDF_DEBUG_NO_TENSOR_CORES | IDF_DEBUG_NO_POOL_FUSION | IDF_DEBUG_NO_ROW_CHUNKS | IDF_DEBUG_NO_PDL | IDF_DEBUG_PREFER_THIN | IDF_DEBUG_NO_FUSED | IDF_DEBUG_FORCE_FUSED | IDF_DEBUG_NO_TILED_EAGER | IDF_DEBUG_NO_TIME_TILES |
+                            IDF_DEBUG_NO_CTA_PAIRS | IDF_DEBUG_FORCE_CTA_PAIRS))
         return fail(IDF_ERR_ARG, "unknown debug flag in 0x%x", flags);
     g_debug_flags.store(flags, std::memory_order_relaxed);
     return IDF_OK;
@@ -988,6 +1011,7 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
                 }
                 if (!planned) { g = 1; shift = 0; planned = plan_as(w, l.cin, l.kw, sx, px, 0); }
                 if (planned && w == 1 && !(debug_flags() & IDF_DEBUG_NO_TIME_TILES)) time_make_plan(spec->dtype, l.cin, l.cout, l.kh, l.stride, &P.time);
+                if (planned && P.x_stride == 1 && !P.tc.pair) pair_make_plan(spec->dtype, P.x_win, P.x_cin, l.cout, l.kh, P.x_kw, l.stride, &P.pair);
                 if (planned) {
                     const size_t tap_elems = (size_t)l.cout * P.x_cin;
                     P.wtc_packed.assign((size_t)l.kh * P.x_kw * tap_elems * es, 0);

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include "idf_pair_tiles.h"
 
 namespace idf {
 
@@ -264,6 +265,17 @@ struct TimePlan {
 bool time_make_plan(int dtype, int Cin, int Cout, int Kh, int stride, TimePlan* p);
 // d_w: the layer's tensor-core weights [tap slot][Cout][Cin] (tc_weight_slot)
 cudaError_t launch_conv_time(const ConvArgs& a, const TimePlan& p, int dtype, const void* d_w, cudaStream_t st);
+
+// Static part of the plan of the CTA-pair kernel (wide 2D layers of stride 1); tile sizes are chosen per launch (idf_pair_tiles.h).
+struct PairPlan {
+    int ok = 0;
+    int swb = 0, KB = 0, n_kb = 0;   // bytes and input channels of a K-block row, K blocks
+    // tiles of the row counts seen last, by their low bits (a stream's pushes repeat a few counts; working them out takes microseconds)
+    struct Seen { int rows = 0, pooled = 0; PairTiles tiles{}; } seen[4];
+};
+bool pair_make_plan(int dtype, int Win, int Cin, int Cout, int Kh, int Kw, int stride, PairPlan* p);
+// d_w: the layer's tensor-core weights [tap slot][Cout][Cin] (tc_weight_slot)
+cudaError_t launch_conv_pair(const ConvArgs& a, PairPlan& p, int dtype, const void* d_w, cudaStream_t st);
 
 // x-unfold: out[row][s][x'][kx*Cin + ci] = in[row][s][x'*stride_x - pad_x + kx][ci] (0 outside the row or
 // beyond Kw*Cin), kpad channels per position, in the activation type

@@ -66,19 +66,6 @@ __device__ __forceinline__ void stage_load(const StageSink& k, uint32_t col_byte
     if (V == 4) asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
     else asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr) : "memory");
 }
-// element-wise maximum of two 32-bit words holding OP = 0: two bf16, 1: one fp32, 2: four int8
-template <int OP>
-__device__ __forceinline__ uint32_t word_max(uint32_t x, uint32_t y)
-{
-    if (OP == 0) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y)); return r; }
-    if (OP == 1) return __float_as_uint(fmaxf(__uint_as_float(x), __uint_as_float(y)));
-    // two bytes at a time: of a 16-bit maximum the upper byte is right whatever the lower bytes are
-    uint32_t h, l, r;
-    asm("max.s16x2 %0, %1, %2;" : "=r"(h) : "r"(x), "r"(y));
-    asm("max.s16x2 %0, %1, %2;" : "=r"(l) : "r"(x << 8), "r"(y << 8));
-    asm("prmt.b32 %0, %1, %2, 0x3715;" : "=r"(r) : "r"(h), "r"(l));
-    return r;
-}
 // 2x2 max-pooling folded into the emission of a conv layer's rows.  A thread owns one (stream, x)
 // position; its x neighbour is the next lane.  The x-pooled first row of a pair waits in the group's
 // staging tile (or, across launches, in the pool layer's state in global memory) until the second

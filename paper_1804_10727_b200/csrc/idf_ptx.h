@@ -342,6 +342,19 @@ __device__ __forceinline__ void emit16f(const uint32_t* v, const float* bias_c, 
         }
     }
 }
+// element-wise maximum of two 32-bit words holding OP = 0: two bf16, 1: one fp32, 2: four int8
+template <int OP>
+__device__ __forceinline__ uint32_t word_max(uint32_t x, uint32_t y)
+{
+    if (OP == 0) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y)); return r; }
+    if (OP == 1) return __float_as_uint(fmaxf(__uint_as_float(x), __uint_as_float(y)));
+    // two bytes at a time: of a 16-bit maximum the upper byte is right whatever the lower bytes are
+    uint32_t h, l, r;
+    asm("max.s16x2 %0, %1, %2;" : "=r"(h) : "r"(x), "r"(y));
+    asm("max.s16x2 %0, %1, %2;" : "=r"(l) : "r"(x << 8), "r"(y << 8));
+    asm("prmt.b32 %0, %1, %2, 0x3715;" : "=r"(r) : "r"(h), "r"(l));
+    return r;
+}
 template <int DT> struct Acc;
 template <> struct Acc<1> { typedef float S; };
 template <> struct Acc<2> { typedef int S; };

@@ -40,6 +40,7 @@ EXPORTS = (
 )
 DEBUG_NO_TENSOR_CORES, DEBUG_NO_POOL_FUSION, DEBUG_NO_ROW_CHUNKS, DEBUG_NO_PDL, DEBUG_PREFER_THIN = 1, 2, 4, 8, 16
 DEBUG_NO_FUSED, DEBUG_FORCE_FUSED, DEBUG_NO_TILED_EAGER, DEBUG_NO_TIME_TILES = 32, 64, 128, 256
+DEBUG_NO_CTA_PAIRS, DEBUG_FORCE_CTA_PAIRS = 512, 1024
 
 
 class IdfLayer(ctypes.Structure):

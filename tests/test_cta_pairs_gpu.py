@@ -1,0 +1,68 @@
+"""Wide layers on CTA pairs (M = 256 tensor-core instructions over two CTAs): positions around the tile sizes (several streams to a tile,
+one, several tiles to a row, an odd last tile), rows of an item and remainders, one and several K blocks, channel slices, blocks that
+begin, continue and end streams (rows carried through the ring, also from its copy), pooled rows with pairs split across launches, odd
+widths, rows that wait only for padding; the row-ring kernel gives the same bytes (int8)."""
+import numpy as np
+import pytest
+
+from paper_1804_10727_b200 import idf
+from paper_1804_10727_b200.workloads import Layer, conv, POOL
+from helpers import assert_close, assert_equal, rand_net, with_shifts
+
+pytestmark = pytest.mark.gpu
+
+
+def rect(cin, cout, kh, kw, pad=0, relu=1):
+    return Layer("conv", cin, cout, kh, kw, 1, pad, relu, 0, 0)
+
+
+CASES = [
+    # (name, mode, layers, H, W, S)
+    ("bf16_64_64", "bf16", (conv(64, 64, 3, pad=1),), 19, 20, 13),
+    ("bf16_128_256_one_position_tile", "bf16", (conv(128, 256, 3, pad=1),), 9, 126, 1),
+    ("bf16_256_128_two_tiles_a_row", "bf16", (conv(256, 128, 3, pad=1),), 7, 130, 2),
+    ("bf16_128_96", "bf16", (conv(128, 96, 3),), 12, 39, 5),                     # slices of 32
+    ("bf16_64_64_k5", "bf16", (conv(64, 64, 5, pad=4),), 11, 24, 3),             # rows and columns of nothing but padding beside the map
+    ("bf16_64_64_k5x2", "bf16", (rect(64, 64, 5, 2, 1, 0),), 14, 30, 2),
+    ("bf16_pool_f32", "bf16", (conv(64, 64, 3, pad=1), POOL), 13, 30, 5),
+    ("bf16_pool_odd", "bf16", (conv(128, 128, 3, pad=1), POOL), 18, 65, 3),      # odd width, one stream to a tile
+    ("i8_64_64", "i8", (conv(64, 64, 3),), 15, 27, 9),                           # 64-byte positions
+    ("i8_128_256", "i8", (conv(128, 256, 3, pad=1),), 10, 18, 7),
+    ("i8_pool", "i8", (conv(128, 64, 3, pad=1), POOL), 17, 34, 4),
+    ("i8_pool_odd_rows", "i8", (conv(64, 128, 3), POOL), 18, 131, 1),
+]
+
+
+@pytest.mark.parametrize("name,mode,layers,H,W,S", CASES, ids=[c[0] for c in CASES])
+def test_cta_pairs_match_oracle(orc, debug_flags, name, mode, layers, H, W, S):
+    layers = with_shifts(layers, 9) if mode == "i8" else layers
+    x, ws, bs = rand_net(mode, layers, H, W, layers[0].cin, S=S, seed=len(name))
+    want = orc.forward(mode, layers, x, ws, bs)
+    check = assert_equal if mode == "i8" else assert_close                       # (one conv layer: fp32 output)
+    debug_flags(idf.DEBUG_FORCE_CTA_PAIRS)
+    for chunks, rb, last in ((None, 0, True), (None, 0, False), ([1] * H, 0, True), ([5, 1, 2], 0, True), ([H // 2], 4, False)):
+        net = idf.Net(mode, layers, W, layers[0].cin, S, ws, bs, row_block=rb)
+        got = idf.infer(net, x, chunks=chunks, last=last)
+        assert net.status()[0] > 0
+        check(got, want, f"{name}/{chunks and len(chunks)}/{rb}/{last}")
+        net.close()
+    if mode == "i8":
+        debug_flags(idf.DEBUG_NO_CTA_PAIRS)
+        net = idf.Net(mode, layers, W, layers[0].cin, S, ws, bs)
+        assert_equal(idf.infer(net, x, chunks=[4, 3], last=True), want, name + "/row ring")
+        net.close()
+
+
+def test_hidden_rows(orc, debug_flags):
+    """bf16 rows between layers, emitted and pooled by pairs: against the row-ring kernels, off by one rounding (2^-8 of the value; the
+    sums of the next layer average that out, so twice it over the largest output bounds them)."""
+    layers = (conv(64, 128, 3, pad=1), POOL, conv(128, 128, 3, pad=1), conv(128, 64, 3, pad=1), POOL)
+    x, ws, bs = rand_net("bf16", layers, 24, 40, 64, S=6, seed=3)
+    outs = []
+    for flags in (idf.DEBUG_FORCE_CTA_PAIRS, idf.DEBUG_NO_CTA_PAIRS):
+        debug_flags(flags)
+        net = idf.Net("bf16", layers, 40, 64, 6, ws, bs)
+        outs.append([idf.infer(net, x, chunks=c, last=True) for c in (None, [1] * 24, [7, 2, 9])])
+        net.close()
+    for got, want in zip(*outs):
+        assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(want).max()
