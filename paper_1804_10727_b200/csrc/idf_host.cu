@@ -158,16 +158,17 @@ void as_planned(const LayerPlan& P, ConvArgs* t)
     t->Win = P.x_win; t->Cin = P.x_cin; t->Kw = P.x_kw; t->stride_x = P.x_stride; t->pad_x = P.x_pad;
 }
 
-// Whether a launch is one for the CTA-pair kernel.
-// Measured on 650 random layers against the row-ring kernel (mean time ring / pairs): 2D layers of a multiple of 128 output channels, all rows in one
-// launch 1.5 (the worst 0.91), 8 to 12 rows at a time 1.25, fewer 0.8 to 0.9 (such a launch mostly waits for the rows it exchanges with
-// the ring).  Of a multiple of 64 channels, two K blocks and more 1.5; with one K block 1.3, but 0.54 where the launch is large (int8
-// 64 -> 64, 2048 streams: MMAs of 64 columns wait for operands); of other channel counts 1.2 with some at 0.5.
-bool by_pairs(const LayerPlan& P, const ConvArgs& a)
+// Whether a launch is one for the CTA-pair kernel; `ring`: the row-ring kernel's plan for it.
+// Measured on 650 random layers against that kernel (mean time ring / pairs): 2D layers of a multiple of 128 output channels, all rows in one
+// launch 1.5 (the worst 0.91), 8 to 12 rows at a time 1.25.  A launch of fewer rows mostly waits for the rows it exchanges with the
+// ring, 0.8 to 0.9 - unless the row-ring kernel takes it in two turns of the SMs (256 -> 256, 64 x 56, one row: 1.10; 30 such layers 1.2, 0.96 to 2.4).  Of
+// a multiple of 64 channels, two K blocks and more 1.5; with one K block 1.3, but 0.54 where the launch is large (int8 64 -> 64, 2048
+// streams: MMAs of 64 columns wait for operands); of other channel counts 1.2 with some at 0.5.
+bool by_pairs(const LayerPlan& P, const TcPlan& ring, const ConvArgs& a)
 {
     if (!P.pair.ok || a.r1 <= a.r0 || (debug_flags() & IDF_DEBUG_NO_CTA_PAIRS)) return false;
     if (debug_flags() & IDF_DEBUG_FORCE_CTA_PAIRS) return true;
-    if (a.r1 - a.r0 < 8) return false;
+    if (a.r1 - a.r0 < 8) return a.Cout % 128 == 0 && !ring.light && (long long)ring.n_mt * ring.n_nt > 148;
     return a.Cout % 128 == 0 || (a.Cout % 64 == 0 && P.pair.n_kb >= 2);
 }
 
@@ -266,7 +267,7 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
             ce = launch_conv_time(a, P.time, net->dtype, net->ws + P.wtc_off, net->stream);
             if (ce == cudaSuccess) P.tc_launches += 1;
         }
-        if (ce == cudaErrorNotSupported && by_pairs(P, a)) {
+        if (ce == cudaErrorNotSupported && by_pairs(P, P.tc, a)) {
             ConvArgs t = a;
             as_planned(P, &t);
             ce = launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream);
@@ -393,7 +394,7 @@ int launch_conv_pool(idf_net* net, size_t i, const void* in_ptr, long long n_in,
         net->launches += 1;
         t.in = net->ws + P.unf_off;
     }
-    ce = by_pairs(P, a) ? launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream) : cudaErrorNotSupported;
+    ce = by_pairs(P, P.tc_pool, a) ? launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream) : cudaErrorNotSupported;
     if (ce == cudaErrorNotSupported)
         ce = launch_conv_tc(t, P.tc_pool, net->dtype, P.w_map_pool, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
     if (net->timing) {

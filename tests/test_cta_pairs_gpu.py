@@ -53,6 +53,19 @@ def test_cta_pairs_match_oracle(orc, debug_flags, name, mode, layers, H, W, S):
         net.close()
 
 
+@pytest.mark.parametrize("S", [72, 76])                                          # 144 and 152 tiles of the row-ring kernel: one turn of the SMs, two
+def test_rows_one_by_one(orc, S):
+    """The rule for launches of few rows, on both sides of its line."""
+    layers = (conv(256, 256, 3, pad=1),)
+    x, ws, bs = rand_net("bf16", layers, 6, 30, 256, S=S, seed=S)
+    pick = np.r_[0:4, S - 1]
+    want = orc.forward("bf16", layers, x[pick], ws, bs)
+    net = idf.Net("bf16", layers, 30, 256, S, ws, bs)
+    for chunks in ([1] * 6, [2, 3, 1], [4, 2]):
+        assert_close(idf.infer(net, x, chunks=chunks, last=True)[pick], want, f"{S}/{len(chunks)}")
+    net.close()
+
+
 def test_hidden_rows(orc, debug_flags):
     """bf16 rows between layers, emitted and pooled by pairs: against the row-ring kernels, off by one rounding (2^-8 of the value; the
     sums of the next layer average that out, so twice it over the largest output bounds them)."""
