@@ -61,7 +61,7 @@ def test_rows_one_by_one(orc, S):
     pick = np.r_[0:4, S - 1]
     want = orc.forward("bf16", layers, x[pick], ws, bs)
     net = idf.Net("bf16", layers, 30, 256, S, ws, bs)
-    for chunks in ([1] * 6, [2, 3, 1], [4, 2]):
+    for chunks in ([1] * 6, [2, 3, 1], [4, 2], [6]):
         assert_close(idf.infer(net, x, chunks=chunks, last=True)[pick], want, f"{S}/{len(chunks)}")
     net.close()
 
