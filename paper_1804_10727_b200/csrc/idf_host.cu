@@ -351,7 +351,8 @@ int launch_conv_pool(idf_net* net, size_t i, const void* in_ptr, long long n_in,
     a.w = net->ws + P.w_off;
     a.bias = P.b_packed.empty() ? nullptr : net->ws + P.b_off;
     a.ring = net->ws + P.state_off;
-        a.ring_scratch = net->ring_scratch_off ? net->ws + net->ring_scratch_off : nullptr;
+    a.ring_scratch = net->ring_scratch_off ? net->ws + net->ring_scratch_off : nullptr;
+    if (a.ring_scratch && P.pair.ok) a.pool_scratch = (unsigned char*)a.ring_scratch + align_up(P.state_bytes_all);
     if (last) {
         a.out = final_out;
         a.out_row_stride = (long long)Q.out_w * Q.out_c;
@@ -1221,8 +1222,12 @@ int idf_net_create(const idf_spec* spec, const void* const* weights, const void*
         }
     {
         size_t biggest = 0;
-        for (auto& P : net->L)
-            if (P.l.kind == IDF_CONV && (P.tc.ok || P.win.ok)) biggest = std::max(biggest, P.state_bytes_all);
+        for (size_t i = 0; i < net->L.size(); ++i) {
+            const LayerPlan& P = net->L[i];
+            // (behind the ring: the pool layer's state, where the layer's launch on CTA pairs has the pool folded in)
+            const size_t pool = P.fuse_pool && P.pair.ok ? align_up(P.state_bytes_all) - P.state_bytes_all + net->L[i + 1].state_bytes_all : 0;
+            if (P.l.kind == IDF_CONV && (P.tc.ok || P.win.ok)) biggest = std::max(biggest, P.state_bytes_all + pool);
+        }
         if (biggest) { net->ring_scratch_off = off; off = align_up(off + biggest); }
     }
     // the last group of positions of a full buffer's last row may reach past it

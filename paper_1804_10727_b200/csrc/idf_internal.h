@@ -73,6 +73,7 @@ struct ConvArgs {
     const void* bias;      // [Cout] in the state type, or nullptr
     void* ring;            // [ring_rows][S][Wout][Cout] state words
     void* ring_scratch;    // tensor-core kernel: room for a copy of the ring (same size), or nullptr
+    void* pool_scratch;    // CTA pairs: room for a copy of the pool state row, or nullptr
     void* out;             // emitted rows
     long long out_row_stride, out_stream_stride, out_row_base;  // element strides; row o goes to (o - out_row_base)
     long long out_rows_extent;   // rows the output buffer holds per stream
@@ -235,6 +236,8 @@ bool tc_make_plan(int dtype, int S, int Win, int Wout, int Cin, int Cout, int Kh
 int tc_weight_slot(int ky, int kx, int Kh, int stride);
 int tc_encode_weights(const TcPlan& p, int dtype, const void* d_w, int taps, int Cin, int Cout, void* map_out);
 cudaError_t launch_ring_copy(void* dst, const void* src, long long words, cudaStream_t st);   // words: a multiple of four
+// a ring and a pool layer's state row in one launch (either may be empty)
+cudaError_t launch_state_copy(void* dst, const void* src, long long words, void* dst2, const void* src2, long long words2, cudaStream_t st);
 cudaError_t launch_conv_tc(const ConvArgs& a, const TcPlan& p, int dtype, const void* w_map, int n_in_rows,
                            unsigned int* status, cudaStream_t st);
 

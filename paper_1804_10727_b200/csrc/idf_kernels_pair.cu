@@ -41,6 +41,7 @@ struct PairArgs {
     const void* ring_in;         // where the rows begun by earlier blocks are read: the ring, or a copy of it
     void* out;
     void* pool_state;            // [S][Wout/2][Cout] in the output type: x-pooled first row of an open pair
+    const void* pool_in;         // where the one that an earlier launch left is read: the same, or a copy of it
     unsigned int* status;
     long long out_row_stride, out_stream_stride, out_row_first;    // elements; output row of row 0 (pooled: of the pair that row 0 begins)
     long long out_elems, ring_elems, pool_elems;
@@ -120,38 +121,6 @@ __device__ __forceinline__ void pair_mma(uint32_t tmem_d, uint32_t alo, uint32_t
                      "tcgen05.mma.cta_group::2.kind::i8 [%0], a1, b1, %5, q;\n\t}"
                      ::"r"(tmem_d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(fresh) : "memory");
 }
-
-// The work items of a cluster: an even share of all units, cut into items of at most R rows of one column of work.
-struct PairWalk {
-    int u, u_end;
-    int col, row0, nr;           // column of work, first row, rows
-    int j_lo, i_lo, i_hi;        // first accumulator in use; i in [i_lo, i_hi]: the input rows the block holds (input row row0 + i - base_ty)
-    __device__ __forceinline__ bool start(const PairArgs& a)
-    {
-        const unsigned c = blockIdx.x >> 1, n = gridDim.x >> 1;
-        u = (int)((long long)a.units * c / n);
-        u_end = (int)((long long)a.units * (c + 1) / n);
-        return next(a);
-    }
-    __device__ __forceinline__ bool next(const PairArgs& a)
-    {
-        if (u >= u_end) return false;
-        col = u / a.n_u;
-        const int r = u - col * a.n_u, rem = min(u_end - u, a.n_u - r), per = a.R / a.row_step;
-        const int pieces = (rem + per - 1) / per, take = (rem + pieces - 1) / pieces;
-        row0 = r * a.row_step;
-        nr = min(take * a.row_step, a.row_hi - row0);
-        u += take;
-        j_lo = max(a.row_lo - row0, 0);
-        i_lo = max(j_lo, a.base_ty - row0);
-        i_hi = min(nr + a.Kh - 2, a.n_in - 1 + a.base_ty - row0);
-        return true;
-    }
-    // input rows of accumulator j; none at all: the row has nothing to add
-    __device__ __forceinline__ int first_row(int j) const { return max(i_lo, j); }
-    __device__ __forceinline__ int last_row(const PairArgs& a, int j) const { return min(i_hi, j + a.Kh - 1); }
-    __device__ __forceinline__ bool has_taps(const PairArgs& a, int j) const { return first_row(j) <= last_row(a, j); }
-};
 
 // W sums of one position -> the words of W emitted values; returns their number
 template <int DT, int W>
@@ -341,8 +310,8 @@ __device__ __forceinline__ bool emit_pooled(const PairArgs& a, const PairSpot& p
             // the pair's other row came with an earlier launch, or comes with a later one
             const long long at = ((long long)p.s * wp + xp) * a.Cout + p.n0 + c + share;
             if (!here || !IDF_OK_AT(a.status, at, a.pool_elems - 4 * H / ES + 1)) continue;
-            unsigned char* st = (unsigned char*)a.pool_state + at * ES;
             if (!emit1) {
+                unsigned char* st = (unsigned char*)a.pool_state + at * ES;
                 if (a.pool_keep) {
 #pragma unroll
                     for (int j = 0; j < H; j += 4) st_global_v4(st + 4 * j, m + j);
@@ -351,7 +320,7 @@ __device__ __forceinline__ bool emit_pooled(const PairArgs& a, const PairSpot& p
             }
 #pragma unroll
             for (int j = 0; j < H; j += 4) {
-                const uint4 g = *(const uint4*)(st + 4 * j);
+                const uint4 g = *(const uint4*)((const unsigned char*)a.pool_in + at * ES + 4 * j);
                 m[j] = word_max<OP>(m[j], g.x); m[j + 1] = word_max<OP>(m[j + 1], g.y);
                 m[j + 2] = word_max<OP>(m[j + 2], g.z); m[j + 3] = word_max<OP>(m[j + 3], g.w);
             }
@@ -415,7 +384,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             bool ok = true;
             // (no item without input rows: the schedule goes by rows)
             auto skip = [&](bool m) { while (m && w.i_lo > w.i_hi) m = w.next(a); return m; };
-            bool more = w.start(a);
+            bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1);
             for (more = skip(more); more && ok;) {
                 const int mt = 2 * (w.col / a.n_nt) + (int)rank, xt = mt % a.n_xt, x0 = xt * a.BX - a.pad_x, s0 = (mt / a.n_xt) * a.BS;
                 PairWalk v = w;                                      // the item at hand
@@ -456,7 +425,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int t = 0, stage = 0;
             uint32_t ph = 1;
             bool ok = true;
-            for (bool more = w.start(a); more && ok; more = w.next(a)) {
+            for (bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1); more && ok; more = w.next(a)) {
                 const int n0 = (w.col % a.n_nt) * a.N + (int)rank * (a.N / 2);
                 for (int kb = 0; kb < a.n_kb && ok; ++kb)
                     for (int i = w.i_lo; i <= w.i_hi && ok; ++i)
@@ -499,7 +468,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             // stages: input row at hand; oldest tap row still wanted; next one to be waited for
             int sa = 0, tail = 0, head = 0;
             uint32_t pa = 0, ph_head = 0, free_ph = 0xffffffffu;
-            bool more = w.start(a), ok = true;
+            bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1), ok = true;
             while (more && w.i_lo > w.i_hi) more = w.next(a);
             // The tensor pipe runs only some instructions behind this warp, which therefore works nothing out: what a row wants done comes with
             // the row (the producer's schedule), and what the next row needs is looked at (barriers without blocking, its schedule entry
@@ -598,7 +567,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (lane == 0) mbar_arrive_cluster(free0 + 8u * j);
         };
         const bool wide = a.N >= 32 * PAIR_GROUPS;
-        for (bool more = w.start(a); more && ok; more = w.next(a)) {
+        for (bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1); more && ok; more = w.next(a)) {
             const int mt = 2 * (w.col / a.n_nt) + (int)rank, xt = mt % a.n_xt;
             p.n0 = (w.col % a.n_nt) * a.N;
             p.s = (mt / a.n_xt) * a.BS + bs;
@@ -696,12 +665,17 @@ cudaError_t launch_conv_pair(const ConvArgs& a, PairPlan& p, int dtype, const vo
     t.N = g.N; t.n_nt = a.Cout / g.N; t.R = g.R; t.KB = p.KB; t.n_kb = p.n_kb; t.swb = p.swb; t.n_a = g.n_a; t.n_b = g.n_b;
     t.a_bytes = (int)g.a_bytes; t.b_bytes = (int)(g.b_tile * a.Kw); t.b_tile = (int)g.b_tile; t.a_box_bytes = (int)g.a_box;
     t.row_step = g.row_step; t.n_u = g.n_u; t.units = (int)g.units;
-    if (t.carried && a.o_end - a.o_begin > a.ring_rows) {
-        // a row begun by an earlier block and one left open by this one may share a ring slot and lie in different CTAs
-        if (!a.ring_scratch) return cudaErrorNotSupported;
-        cudaError_t ce = launch_ring_copy(a.ring_scratch, a.ring, (long long)a.ring_rows * a.S * a.Wout * a.Cout, st);
+    t.pool_in = a.pool_state;
+    // a row begun by an earlier block and one left open by this one may share a ring slot and lie in different CTAs; so may the pooled rows
+    // that the block takes and parks (both copies are one launch)
+    const bool copy_ring = t.carried && a.o_end - a.o_begin > a.ring_rows, copy_pool = pooled && pair_pool_state_both(a.o_begin, a.done_end, a.pool_keep);
+    if (copy_ring || copy_pool) {
+        if (!a.ring_scratch || (copy_pool && !a.pool_scratch)) return cudaErrorNotSupported;
+        cudaError_t ce = launch_state_copy(a.ring_scratch, a.ring, copy_ring ? (long long)a.ring_rows * a.S * a.Wout * a.Cout : 0,
+                                           a.pool_scratch, a.pool_state, copy_pool ? a.pool_state_elems * elem_size(a.out_elem) / 4 : 0, st);
         if (ce != cudaSuccess) return ce;
-        t.ring_in = a.ring_scratch;
+        if (copy_ring) t.ring_in = a.ring_scratch;
+        if (copy_pool) t.pool_in = a.pool_scratch;
     }
     CUtensorMap tmA, tmW;
     {

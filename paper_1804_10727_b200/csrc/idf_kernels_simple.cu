@@ -874,23 +874,33 @@ cudaError_t launch_avg(const AvgArgs& a, cudaStream_t st)
     }
 }
 
-// Copy of a layer's ring for launches whose CTAs read rows that others rewrite.  As a kernel it takes part in the chain of dependent
+// Copy of a layer's ring (and of the pool layer's state row) for launches whose CTAs read rows that others rewrite.  As a kernel it takes part in the chain of dependent
 // launches, which a copy by the driver interrupts (vgg2d, 5 streams in groups of 29 rows: 507 us with driver copies, 488 so).
 namespace {
-__global__ void __launch_bounds__(256) ring_copy_kernel(uint4* dst, const uint4* src, unsigned int n)
+__global__ void __launch_bounds__(256) ring_copy_kernel(uint4* dst, const uint4* src, unsigned int n, uint4* dst2, const uint4* src2, unsigned int n2)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (unsigned int i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) dst[i] = src[i];
+    for (unsigned int i = blockIdx.x * 256u + threadIdx.x; i < n2; i += gridDim.x * 256u) dst2[i] = src2[i];
 }
 }  // namespace
 
+cudaError_t launch_state_copy(void* dst, const void* src, long long words, void* dst2, const void* src2, long long words2, cudaStream_t st)
+{
+    const long long n = words / 4, n2 = words2 / 4, most = n > n2 ? n : n2;
+    if (most > 0x7fffffffLL) {
+        cudaError_t e = words ? cudaMemcpyAsync(dst, src, (size_t)words * 4, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
+        if (e == cudaSuccess && words2) e = cudaMemcpyAsync(dst2, src2, (size_t)words2 * 4, cudaMemcpyDeviceToDevice, st);
+        return e;
+    }
+    const long long blocks = (most + 255) / 256;
+    return launch_pdl(ring_copy_kernel, (unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st, (uint4*)dst, (const uint4*)src, (unsigned int)n,
+                      (uint4*)dst2, (const uint4*)src2, (unsigned int)n2);
+}
 cudaError_t launch_ring_copy(void* dst, const void* src, long long words, cudaStream_t st)
 {
-    const long long n = words / 4;
-    if (n > 0x7fffffffLL) return cudaMemcpyAsync(dst, src, (size_t)words * 4, cudaMemcpyDeviceToDevice, st);
-    const long long blocks = (n + 255) / 256;
-    return launch_pdl(ring_copy_kernel, (unsigned)(blocks < 148 * 8 ? blocks : 148 * 8), 256, 0, st, (uint4*)dst, (const uint4*)src, (unsigned int)n);
+    return launch_state_copy(dst, src, words, nullptr, nullptr, 0, st);
 }
 
 }  // namespace idf

@@ -1,6 +1,13 @@
-// Tile sizes of the CTA-pair kernel (idf_kernels_pair.cu), chosen per launch.  Plain host code: no CUDA headers.
+// Tile sizes of the CTA-pair kernel (idf_kernels_pair.cu), chosen per launch, and the order in which its clusters take the work.  No CUDA
+// headers: the parts that the kernel runs compile as plain host code too.
 #pragma once
 #include <cstddef>
+
+#ifdef __CUDACC__
+#define IDF_ANYWHERE __host__ __device__ __forceinline__
+#else
+#define IDF_ANYWHERE inline
+#endif
 
 namespace idf {
 
@@ -87,6 +94,52 @@ inline PairTiles pair_tiles(int S, int Wout, int Cout, int Kh, int Kw, int swb, 
         }
     }
     return best;
+}
+
+// The work items of a cluster: an even share of all units, cut into items of at most R rows of one column of work.  Args: PairArgs, or what
+// a test has in its place.
+struct PairWalk {
+    int u, u_end;
+    int col, row0, nr;           // column of work, first row, rows
+    int j_lo, i_lo, i_hi;        // first accumulator in use; i in [i_lo, i_hi]: the input rows the block holds (input row row0 + i - base_ty)
+    static IDF_ANYWHERE int least(int x, int y) { return x < y ? x : y; }
+    static IDF_ANYWHERE int most(int x, int y) { return x > y ? x : y; }
+    template <class Args>
+    IDF_ANYWHERE bool start(const Args& a, unsigned c, unsigned n)      // cluster c of n
+    {
+        u = (int)((long long)a.units * c / n);
+        u_end = (int)((long long)a.units * (c + 1) / n);
+        return next(a);
+    }
+    template <class Args>
+    IDF_ANYWHERE bool next(const Args& a)
+    {
+        if (u >= u_end) return false;
+        col = u / a.n_u;
+        const int r = u - col * a.n_u, rem = least(u_end - u, a.n_u - r), per = a.R / a.row_step;
+        const int pieces = (rem + per - 1) / per, take = (rem + pieces - 1) / pieces;
+        row0 = r * a.row_step;
+        nr = least(take * a.row_step, a.row_hi - row0);
+        u += take;
+        j_lo = most(a.row_lo - row0, 0);
+        i_lo = most(j_lo, a.base_ty - row0);
+        i_hi = least(nr + a.Kh - 2, a.n_in - 1 + a.base_ty - row0);
+        return true;
+    }
+    // input rows of accumulator j; none at all: the row has nothing to add
+    IDF_ANYWHERE int first_row(int j) const { return most(i_lo, j); }
+    template <class Args>
+    IDF_ANYWHERE int last_row(const Args& a, int j) const { return least(i_hi, j + a.Kh - 1); }
+    template <class Args>
+    IDF_ANYWHERE bool has_taps(const Args& a, int j) const { return first_row(j) <= last_row(a, j); }
+};
+
+// Whether a launch with the max-pool folded in both takes the x-pooled first row of a pair out of the pool layer's state (it begins with the
+// pair's second row) and parks another one there (it ends with a first row).  The two pairs are different work items, mostly of different
+// clusters, and nothing orders them: such a launch takes the row from a copy.
+inline bool pair_pool_state_both(long long o_begin, long long done_end, int pool_keep)
+{
+    return pool_keep && (o_begin & 1) && (done_end & 1) && done_end > o_begin;
 }
 
 }  // namespace idf

@@ -4,6 +4,7 @@ begin, continue and end streams (rows carried through the ring, also from its co
 widths, rows that wait only for padding; the row-ring kernel gives the same bytes (int8)."""
 import numpy as np
 import pytest
+import torch
 
 from paper_1804_10727_b200 import idf
 from paper_1804_10727_b200.workloads import Layer, conv, POOL
@@ -79,3 +80,31 @@ def test_hidden_rows(orc, debug_flags):
         net.close()
     for got, want in zip(*outs):
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("push", [14, 36, 40])
+def test_pool_rows_taken_and_parked_in_one_launch(debug_flags, push):
+    """Launches that begin with a pair's second row and end with a pair's first (rows [35, 71), [71, 107)): the row an earlier launch left in
+    the pool state and the one parked there belong to different clusters, in no order; with shares that straddle columns of work the parking
+    cluster comes first.  The row-ring kernel gives the same bytes, every time."""
+    layers = with_shifts((conv(128, 128, 3, pad=1), POOL), 12)
+    S, H, W = 64, 112, 112
+    g = torch.Generator(device="cuda").manual_seed(push)
+    seg = torch.randint(-127, 128, (H, S, W, 128), generator=g, device="cuda", dtype=torch.int8)
+    _, ws, bs = rand_net("i8", layers, 1, 1, 128, S=1, seed=push)
+    net = idf.Net("i8", layers, W, 128, S, ws, bs)
+    net.open()
+    outs = []
+    for rep in range(11):
+        debug_flags(idf.DEBUG_NO_CTA_PAIRS if rep == 0 else 0)
+        out = net.alloc_out(H)
+        net.reset()
+        for r in range(0, H - push, push):
+            net.push(seg[r:r + push], out)
+        r = (H - 1) // push * push
+        net.push_last(seg[r:], out)
+        net.status()
+        outs.append(out)
+        assert torch.equal(out, outs[0]), f"{push} rows a push, run {rep}: {int((out != outs[0]).sum())} of {out.numel()} differ"
+    assert int(outs[0].ne(0).sum()) > outs[0].numel() // 4
+    net.close()

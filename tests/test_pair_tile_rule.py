@@ -45,9 +45,67 @@ int main() {
 """
 
 
-def test_tiles_fit(tmp_path):
+POOL_PROGRAM = r"""
+#include <cstdio>
+#include <initializer_list>
+#include <vector>
+#include "idf_pair_tiles.h"
+using namespace idf;
+struct Args { int units, n_u, R, row_step, row_lo, row_hi, Kh, base_ty, n_in; };
+int main() {
+    // launches of a 3x3 layer with padding and a pool: every output row belongs to one item; of pairs split over launches, the items that
+    // take the first row out of the pool state and that park one there
+    long long apart = 0, launches = 0;
+    for (int S : {1, 3, 64})
+        for (int Wout : {40, 56, 112, 131})
+            for (int o_begin : {0, 1, 35})
+                for (int rows : {1, 2, 3, 6, 7, 8, 35, 36, 37}) {
+                    const int r0 = o_begin ? o_begin + 1 : 0, r1 = r0 + rows, done_end = r1 - 1, o_end = r1 + 1, o0 = o_begin & ~1;
+                    if (done_end < o_begin) continue;
+                    const PairTiles t = pair_tiles(S, Wout, 128, 3, 3, 128, 2, o_end - o0, 1);
+                    if (!t.ok) { printf("no tiles\n"); return 1; }
+                    const Args a{(int)t.units, t.n_u, t.R, 2, o_begin - o0, o_end - o0, 3, r0 + 1 - o0, r1 - r0};
+                    const int cols = (int)(t.units / t.n_u), done = done_end - o0;
+                    std::vector<int> seen(cols * a.row_hi, 0), taker(cols, -1), parker(cols, -1);
+                    int item = 0;
+                    for (int c = 0; c < t.clusters; ++c) {
+                        PairWalk w;
+                        for (bool more = w.start(a, c, t.clusters); more; more = w.next(a), ++item)
+                            for (int j = w.j_lo; j < w.nr; ++j) {
+                                const int row = w.row0 + j;
+                                seen[w.col * a.row_hi + row]++;
+                                if (row >= done) continue;
+                                if ((row & 1) && row - 1 < a.row_lo) taker[w.col] = c;
+                                if (!(row & 1) && row + 1 >= done) parker[w.col] = c;
+                            }
+                    }
+                    ++launches;
+                    const bool both = pair_pool_state_both(o_begin, done_end, 1);
+                    for (int k = 0; k < cols; ++k) {
+                        for (int row = a.row_lo; row < a.row_hi; ++row)
+                            if (seen[k * a.row_hi + row] != 1) { printf("row %d of column %d: %d items\n", row, k, seen[k * a.row_hi + row]); return 1; }
+                        if (both != (taker[k] >= 0 && parker[k] >= 0)) { printf("S %d W %d rows [%d, %d): taken by %d, parked by %d, rule %d\n", S, Wout, o_begin, done_end, taker[k], parker[k], both); return 1; }
+                        apart += both && taker[k] != parker[k];
+                    }
+                }
+    printf("%lld launches, %lld columns with the two in different clusters\n", launches, apart);
+    return apart > 0 && !pair_pool_state_both(1, 7, 0) ? 0 : 1;
+}
+"""
+
+
+def run(program, tmp_path):
     src, exe = tmp_path / "rule.cpp", tmp_path / "rule"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_1804_10727_b200", "csrc"), str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+def test_tiles_fit(tmp_path):
+    run(PROGRAM, tmp_path)
+
+
+def test_launches_that_take_and_park_a_pool_row_are_known(tmp_path):
+    """Nothing orders the clusters: where one may read the pool state's words that another writes, the launch must read a copy."""
+    run(POOL_PROGRAM, tmp_path)
