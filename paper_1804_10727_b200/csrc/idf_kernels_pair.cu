@@ -379,7 +379,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // ------------------------------ input rows ---------------------------------------------
         if (lane == 0) {
             const uint32_t full0 = map_to_rank(a_full, 0);
-            int t = 0, stage = 0;
+            int stage = 0;
             uint32_t ph = 1;
             bool ok = true;
             // (no item without input rows: the schedule goes by rows)
@@ -391,7 +391,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 more = w.next(a);
                 more = skip(more);
                 for (int kb = 0; kb < a.n_kb && ok; ++kb)
-                    for (int i = v.i_lo; i <= v.i_hi; ++i, ++t) {
+                    for (int i = v.i_lo; i <= v.i_hi; ++i) {
                         // What the MMA warp has to do with this row, section by section (accumulators j_hi, j_hi - 1, ..): one bit each.
                         const int j_hi = min(v.nr - 1, i), j_end = max(v.j_lo, i - a.Kh + 1), n = j_hi - j_end + 1;
                         const uint32_t all = (1u << n) - 1u, oldest = 1u << (n - 1);
@@ -411,10 +411,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
             }
             // the first CTA's last commits must have arrived here before this CTA may leave
-            for (int k = 0; k < a.n_a && k < t && ok; ++k) {
-                ok = mbar_wait(a_empty + 8u * stage, ph, abort_flag);
-                if (++stage == a.n_a) { stage = 0; ph ^= 1u; }
-            }
+            if (ok) pair_drain(stage, ph, a.n_a, [&](int s, uint32_t parity) { return mbar_wait(a_empty + 8u * s, parity, abort_flag); });
         }
         __syncwarp();
     } else if (warp == PAIR_W_WARP) {
@@ -422,7 +419,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (lane == 0) {
             const uint32_t full0 = map_to_rank(b_full, 0);
             const uint32_t half = (uint32_t)(a.N / 2) * a.swb;
-            int t = 0, stage = 0;
+            int stage = 0;
             uint32_t ph = 1;
             bool ok = true;
             for (bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1); more && ok; more = w.next(a)) {
@@ -437,14 +434,10 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             // (slot of a tap in the parameters: see tc_weight_slot, stride 1)
                             for (int kx = 0; kx < a.Kw; ++kx)
                                 tma_pair_3d(sB + (uint32_t)(stage * a.b_bytes + kx * a.b_tile), &tmW, full0 + 8u * stage, kb * a.KB, n0, kx * a.Kh + a.Kh - 1 - (i - j));
-                            ++t;
                             if (++stage == a.n_b) { stage = 0; ph ^= 1u; }
                         }
             }
-            for (int k = 0; k < a.n_b && k < t && ok; ++k) {
-                ok = mbar_wait(b_empty + 8u * stage, ph, abort_flag);
-                if (++stage == a.n_b) { stage = 0; ph ^= 1u; }
-            }
+            if (ok) pair_drain(stage, ph, a.n_b, [&](int s, uint32_t parity) { return mbar_wait(b_empty + 8u * s, parity, abort_flag); });
             asm volatile("griddepcontrol.wait;" ::: "memory");
         }
         __syncwarp();

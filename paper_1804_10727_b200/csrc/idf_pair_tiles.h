@@ -134,6 +134,18 @@ struct PairWalk {
     IDF_ANYWHERE bool has_taps(const Args& a, int j) const { return first_row(j) <= last_row(a, j); }
 };
 
+// A producer's last waits: every stage of its ring of n is free again, `stage` and its parity `ph` being those of the next use.  All n are looked
+// at however many were used (a stage that never was passes at once: the phase before a barrier's first counts as over).
+template <class Wait>
+IDF_ANYWHERE bool pair_drain(int stage, unsigned ph, int n, Wait wait)
+{
+    for (int k = 0; k < n; ++k) {
+        if (!wait(stage, ph)) return false;
+        if (++stage == n) { stage = 0; ph ^= 1u; }
+    }
+    return true;
+}
+
 // Whether a launch with the max-pool folded in both takes the x-pooled first row of a pair out of the pool layer's state (it begins with the
 // pair's second row) and parks another one there (it ends with a first row).  The two pairs are different work items, mostly of different
 // clusters, and nothing orders them: such a launch takes the row from a copy.

@@ -93,6 +93,32 @@ int main() {
 }
 """
 
+DRAIN_PROGRAM = r"""
+#include <cstdio>
+#include <vector>
+#include "idf_pair_tiles.h"
+using namespace idf;
+int main() {
+    // a ring of n stages after t uses, one of its stages (or none) not yet given back; a barrier is the number of its completed phases,
+    // and a wait for a parity passes where the phase of that parity is the one before the current
+    for (int n = 1; n <= PAIR_MAX_B; ++n)
+        for (int t = 0; t <= 3 * n; ++t)
+            for (int late = -1; late < n && late < t; ++late) {
+                std::vector<unsigned> done(n, 0);
+                int stage = 0;
+                unsigned ph = 1;
+                for (int k = 0; k < t; ++k) {
+                    done[stage]++;
+                    if (++stage == n) { stage = 0; ph ^= 1u; }
+                }
+                if (late >= 0) done[late]--;
+                const bool over = pair_drain(stage, ph, n, [&](int s, unsigned parity) { return (done[s] & 1u) != parity; });
+                if (over != (late < 0)) { printf("%d stages, %d uses, stage %d late: over %d\n", n, t, late, over); return 1; }
+            }
+    return 0;
+}
+"""
+
 
 def run(program, tmp_path):
     src, exe = tmp_path / "rule.cpp", tmp_path / "rule"
@@ -109,3 +135,8 @@ def test_tiles_fit(tmp_path):
 def test_launches_that_take_and_park_a_pool_row_are_known(tmp_path):
     """Nothing orders the clusters: where one may read the pool state's words that another writes, the launch must read a copy."""
     run(POOL_PROGRAM, tmp_path)
+
+
+def test_closing_waits_cover_every_stage_in_use(tmp_path):
+    """No CTA leaves before the arrivals on its barriers are in, also where fewer stages were used than there are."""
+    run(DRAIN_PROGRAM, tmp_path)
