@@ -31,7 +31,6 @@ int tc_weight_slot(int ky, int kx, int Kh, int stride);
 namespace {
 
 constexpr int PAIR_GROUPS = 4;                             // emission groups of four warps, each with a share of an accumulator's columns
-constexpr int PAIR_MMA_WARPS = 2;                          // each issues for every other accumulator
 constexpr int PAIR_W_WARP = 1 + PAIR_MMA_WARPS, PAIR_EPI_WARP = PAIR_W_WARP + 1;
 constexpr int PAIR_THREADS = 32 * (PAIR_EPI_WARP + 4 * PAIR_GROUPS);
 
@@ -340,7 +339,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
     __shared__ uint4 s_sched[PAIR_MAX_A];                              // per input row at hand: what the MMA warp has to do with it
-    __shared__ __align__(8) unsigned long long s_bars[2 * PAIR_MAX_A + 2 * PAIR_MAX_B + 2 * PAIR_MAX_R + 1];
+    __shared__ __align__(8) unsigned long long s_bars[2 * PAIR_MAX_A + 2 * PAIR_MAX_B + 2 * PAIR_MAX_R + PAIR_MMA_WARPS];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -358,7 +357,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (lane < a.n_a) { mbar_init(a_full + 8u * lane, 1); mbar_init(a_empty + 8u * lane, PAIR_MMA_WARPS); }
         if (lane < a.n_b) { mbar_init(b_full + 8u * lane, 1); mbar_init(b_empty + 8u * lane, PAIR_MMA_WARPS); }
         if (lane < PAIR_MAX_R) { mbar_init(acc_full + 8u * lane, 1); mbar_init(acc_free + 8u * lane, 2 * 4 * PAIR_GROUPS); }
-        if (lane == 31) mbar_init(bar_done, 1);
+        if (lane < PAIR_MMA_WARPS) mbar_init(bar_done + 8u * lane, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -530,11 +529,14 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     entry(sa);
                 }
             }
-            if (!ok) {
-                // let what has been issued finish before either CTA gives its memory back
-                if (issuer) pair_commit(bar_done);
-                for (uint32_t i = 0; i < 4096 && !mbar_try_wait(bar_done, 0); ++i) __nanosleep(64);
-            }
+            // (what has been issued finishes before either CTA gives its memory back)
+            if (!ok)
+                pair_give_up(warp - 1, [&](int k) { if (issuer) pair_commit(bar_done + 8u * k); },
+                             [&](int k) {
+                                 if (mbar_try_wait(bar_done + 8u * k, 0)) return true;
+                                 __nanosleep(64);
+                                 return false;
+                             });
         }
         __syncwarp();
     } else {

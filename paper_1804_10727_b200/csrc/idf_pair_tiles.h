@@ -12,6 +12,7 @@
 namespace idf {
 
 constexpr int PAIR_MAX_A = 8, PAIR_MAX_B = 24, PAIR_MAX_R = 8;     // stages of input rows and of tap rows, rows of a work item
+constexpr int PAIR_MMA_WARPS = 2;                                  // issuing warps: each issues for every other accumulator
 constexpr int PAIR_CLUSTERS = 74;                                  // two SMs each
 constexpr double PAIR_ROW_CLK = 800, PAIR_ITEM_CLK = 600;          // cycles from one input row to the next with little to do in it, and between items
 constexpr size_t PAIR_SMEM = 230400;                               // dynamic shared memory per CTA (227 KB less the static part)
@@ -144,6 +145,15 @@ IDF_ANYWHERE bool pair_drain(int stage, unsigned ph, int n, Wait wait)
         if (++stage == n) { stage = 0; ph ^= 1u; }
     }
     return true;
+}
+
+// What an issuing warp does that gives up: all it has issued is committed to a barrier of its own (of one arrival: a shared one would tell it of
+// the other warp's instructions, and turn twice) and has a bounded time to finish.
+template <class Commit, class Over>
+IDF_ANYWHERE void pair_give_up(int issuer, Commit commit, Over over)
+{
+    commit(issuer);
+    for (int i = 0; i < 4096 && !over(issuer); ++i) {}
 }
 
 // Whether a launch with the max-pool folded in both takes the x-pooled first row of a pair out of the pool layer's state (it begins with the

@@ -119,6 +119,32 @@ int main() {
 }
 """
 
+GIVE_UP_PROGRAM = r"""
+#include <cstdio>
+#include "idf_pair_tiles.h"
+using namespace idf;
+int main() {
+    // barriers of one arrival; issuer k's instructions finish at its look number p, the other issuers' at look q
+    for (int k = 0; k < PAIR_MMA_WARPS; ++k)
+        for (int p = 0; p <= 6; ++p)
+            for (int q = 0; q <= 6; ++q) {
+                unsigned phases[PAIR_MMA_WARPS] = {};
+                int looks = 0, mine = -1, theirs[PAIR_MMA_WARPS];
+                for (int o = 0; o < PAIR_MMA_WARPS; ++o)                      // the barriers the others commit to
+                    if (o != k) pair_give_up(o, [&](int b) { theirs[o] = b; }, [](int) { return true; });
+                pair_give_up(k, [&](int b) { mine = b; }, [&](int b) {
+                    if (looks == p) phases[mine]++;
+                    for (int o = 0; o < PAIR_MMA_WARPS; ++o)
+                        if (o != k && looks == q) phases[theirs[o]]++;
+                    ++looks;
+                    return (phases[b] & 1u) == 1u;
+                });
+                if (looks != p + 1) { printf("issuer %d done at %d, the other at %d: left at %d\n", k, p, q, looks - 1); return 1; }
+            }
+    return 0;
+}
+"""
+
 
 def run(program, tmp_path):
     src, exe = tmp_path / "rule.cpp", tmp_path / "rule"
@@ -140,3 +166,7 @@ def test_launches_that_take_and_park_a_pool_row_are_known(tmp_path):
 def test_closing_waits_cover_every_stage_in_use(tmp_path):
     """No CTA leaves before the arrivals on its barriers are in, also where fewer stages were used than there are."""
     run(DRAIN_PROGRAM, tmp_path)
+
+
+def test_issuers_that_give_up_wait_for_their_own_instructions(tmp_path):
+    run(GIVE_UP_PROGRAM, tmp_path)
