@@ -338,10 +338,14 @@ typedef enum {
     IDF_DEBUG_FORCE_FUSED = 64,     /* ... always, where a stream's state fits (by default: small pushes only) */
     IDF_DEBUG_NO_TILED_EAGER = 128, /* eager emission: the plain kernels for every shape                      */
     IDF_DEBUG_NO_TIME_TILES = 256,  /* 1D tensor-core layers on the row-ring kernel                           */
-    IDF_DEBUG_NO_CTA_PAIRS = 512,   /* wide layers on the row-ring kernel (1D ones as without CTA pairs)      */
+    IDF_DEBUG_NO_CTA_PAIRS = 512,   /* wide layers on the row-ring kernel                                     */
     IDF_DEBUG_FORCE_CTA_PAIRS = 1024 /* every launch of a layer that the CTA-pair kernel can take goes there  */
 } idf_debug_flag;
 int idf_set_debug_flags(unsigned int flags);
+
+/* Debug only.  Per layer, how many of the launches that idf_stream_status counts went to the CTA-pair kernel since the last open or
+ * reset (host, n_layers entries; nothing is waited for): a launch that this kernel declines goes on to the next one without a word. */
+int idf_debug_pair_launches(const idf_net* net, long long* launches);
 
 /* Message for the most recent failure on the calling thread ("" if none). */
 const char* idf_last_error(void);

@@ -45,7 +45,7 @@ struct LayerPlan {
     alignas(64) unsigned char w_map[128];   // TMA descriptor of wtc in the workspace (made at open)
     TcPlan tc_pool;                         // plan of the launches that also emit the following max-pool's rows
     alignas(64) unsigned char w_map_pool[128];
-    long long tc_launches = 0;
+    long long tc_launches = 0, pair_launches = 0;      // launches on the tensor cores; those of them on CTA pairs
     std::vector<unsigned char> wq_packed;      // int nets, Cin % 4 == 0: [Kh][Kw][Cin/4][Cout] words of four int8 (all-layers launch)
     size_t wq_off = 0;
     PairPlan pair;                             // wide layers on CTA pairs (pair.ok; weights: wtc_packed)
@@ -273,7 +273,7 @@ int launch_layer(idf_net* net, size_t i, const void* in_ptr, long long n_in, boo
             ConvArgs t = a;
             as_planned(P, &t);
             ce = launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream);
-            if (ce == cudaSuccess) P.tc_launches += 1;
+            if (ce == cudaSuccess) { P.tc_launches += 1; P.pair_launches += 1; }
         }
         if (ce == cudaErrorNotSupported && P.tc.ok && !P.use_sparse && n_in > 0) {
             ConvArgs t = a;
@@ -398,6 +398,7 @@ int launch_conv_pool(idf_net* net, size_t i, const void* in_ptr, long long n_in,
         t.in = net->ws + P.unf_off;
     }
     ce = by_pairs(P, P.tc_pool, a) ? launch_conv_pair(t, P.pair, net->dtype, net->ws + P.wtc_off, net->stream) : cudaErrorNotSupported;
+    if (ce == cudaSuccess) P.pair_launches += 1;
     if (ce == cudaErrorNotSupported)
         ce = launch_conv_tc(t, P.tc_pool, net->dtype, P.w_map_pool, (int)n_in, (unsigned int*)(net->ws + net->status_off), net->stream);
     if (net->timing) {
@@ -1319,7 +1320,7 @@ int idf_stream_reset(idf_net* net)
 {
     if (!net) return fail(IDF_ERR_ARG, "net must not be NULL");
     if (net->phase == CREATED) return fail(IDF_ERR_STATE, "reset before stream_open");
-    for (auto& P : net->L) { P.rows_in = 0; P.rows_done = 0; P.tc_launches = 0; P.pending = 0; P.e_hi = -1; }
+    for (auto& P : net->L) { P.rows_in = 0; P.rows_done = 0; P.tc_launches = P.pair_launches = 0; P.pending = 0; P.e_hi = -1; }
     cudaError_t e = cudaMemsetAsync(net->ws + net->state_region_off, 0, net->reset_bytes, net->stream);
     if (e != cudaSuccess) { net->phase = CREATED; return fail(IDF_ERR_CUDA, "stream_reset: %s", cudaGetErrorString(e)); }
     net->phase = OPEN;
@@ -1507,6 +1508,13 @@ int idf_event_counts(idf_net* net, long long* events)
 }
 
 long long idf_launch_count(const idf_net* net) { return net ? net->launches : 0; }
+
+int idf_debug_pair_launches(const idf_net* net, long long* launches)
+{
+    if (!net || !launches) return fail(IDF_ERR_ARG, "net and launches must not be NULL");
+    for (size_t i = 0; i < net->L.size(); ++i) launches[i] = net->L[i].pair_launches;
+    return IDF_OK;
+}
 
 int idf_stream_status(idf_net* net, long long* tensor_core_launches)
 {

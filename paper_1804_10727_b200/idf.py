@@ -36,7 +36,7 @@ EXPORTS = (
     "idf_net_create", "idf_net_destroy", "idf_net_state_bytes", "idf_net_workspace_bytes", "idf_out_shape",
     "idf_stream_open", "idf_stream_reset", "idf_stream_push", "idf_stream_push_last", "idf_stream_finish", "idf_run_host", "idf_event_counts",
     "idf_launch_count", "idf_stream_status", "idf_set_timing", "idf_layer_times", "idf_conv_rows_noalloc", "idf_last_error",
-    "idf_state_snapshot_bytes", "idf_state_save", "idf_state_restore", "idf_stream_set_out_base", "idf_set_debug_flags", "idf_out_rows_needed",
+    "idf_state_snapshot_bytes", "idf_state_save", "idf_state_restore", "idf_stream_set_out_base", "idf_set_debug_flags", "idf_out_rows_needed", "idf_debug_pair_launches",
 )
 DEBUG_NO_TENSOR_CORES, DEBUG_NO_POOL_FUSION, DEBUG_NO_ROW_CHUNKS, DEBUG_NO_PDL, DEBUG_PREFER_THIN = 1, 2, 4, 8, 16
 DEBUG_NO_FUSED, DEBUG_FORCE_FUSED, DEBUG_NO_TILED_EAGER, DEBUG_NO_TIME_TILES = 32, 64, 128, 256
@@ -93,6 +93,7 @@ def lib():
         L.idf_state_save.argtypes = [vp, vp, sz]
         L.idf_state_restore.argtypes = [vp, vp, sz]
         L.idf_set_debug_flags.argtypes = [ctypes.c_uint]
+        L.idf_debug_pair_launches.argtypes = [vp, ctypes.POINTER(ll)]
         L.idf_out_rows_needed.argtypes = [vp, ll]; L.idf_out_rows_needed.restype = ll
         L.idf_last_error.restype = ctypes.c_char_p
         _lib = L
@@ -200,6 +201,12 @@ class Net:
         """Synchronise; raise if a kernel gave up on a bounded wait; return tensor-core launches per layer."""
         n = (ctypes.c_longlong * self.n_layers)()
         _check(lib().idf_stream_status(self._h, n))
+        return list(n)
+
+    def pair_launches(self):
+        """Debug: launches per layer on the CTA-pair kernel, of those that status() returns."""
+        n = (ctypes.c_longlong * self.n_layers)()
+        _check(lib().idf_debug_pair_launches(self._h, n))
         return list(n)
 
     def set_timing(self, on: bool):

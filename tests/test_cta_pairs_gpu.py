@@ -44,13 +44,14 @@ def test_cta_pairs_match_oracle(orc, debug_flags, name, mode, layers, H, W, S):
     for chunks, rb, last in ((None, 0, True), (None, 0, False), ([1] * H, 0, True), ([5, 1, 2], 0, True), ([H // 2], 4, False)):
         net = idf.Net(mode, layers, W, layers[0].cin, S, ws, bs, row_block=rb)
         got = idf.infer(net, x, chunks=chunks, last=last)
-        assert net.status()[0] > 0
+        assert net.pair_launches()[0] == net.status()[0] > 0                     # every launch that brings rows
         check(got, want, f"{name}/{chunks and len(chunks)}/{rb}/{last}")
         net.close()
     if mode == "i8":
         debug_flags(idf.DEBUG_NO_CTA_PAIRS)
         net = idf.Net(mode, layers, W, layers[0].cin, S, ws, bs)
         assert_equal(idf.infer(net, x, chunks=[4, 3], last=True), want, name + "/row ring")
+        assert net.status()[0] > 0 and net.pair_launches()[0] == 0
         net.close()
 
 
@@ -64,6 +65,8 @@ def test_rows_one_by_one(orc, S):
     net = idf.Net("bf16", layers, 30, 256, S, ws, bs)
     for chunks in ([1] * 6, [2, 3, 1], [4, 2], [6]):
         assert_close(idf.infer(net, x, chunks=chunks, last=True)[pick], want, f"{S}/{len(chunks)}")
+        few = sum(n < 6 for n in chunks)
+        assert net.pair_launches()[0] == len(chunks) - (few if S == 72 else 0) and net.status()[0] == len(chunks)
     net.close()
 
 
@@ -76,7 +79,11 @@ def test_hidden_rows(orc, debug_flags):
     for flags in (idf.DEBUG_FORCE_CTA_PAIRS, idf.DEBUG_NO_CTA_PAIRS):
         debug_flags(flags)
         net = idf.Net("bf16", layers, 40, 64, 6, ws, bs)
-        outs.append([idf.infer(net, x, chunks=c, last=True) for c in (None, [1] * 24, [7, 2, 9])])
+        outs.append([])
+        for c in (None, [1] * 24, [7, 2, 9]):
+            outs[-1].append(idf.infer(net, x, chunks=c, last=True))
+            tc, pairs = net.status(), net.pair_launches()
+            assert all(tc[i] > 0 and pairs[i] == (tc[i] if flags == idf.DEBUG_FORCE_CTA_PAIRS else 0) for i in (0, 2, 3)), (flags, c, tc, pairs)
         net.close()
     for got, want in zip(*outs):
         assert np.abs(got - want).max() <= 2.0 ** -7 * np.abs(want).max()
@@ -104,6 +111,7 @@ def test_pool_rows_taken_and_parked_in_one_launch(debug_flags, push):
         r = (H - 1) // push * push
         net.push_last(seg[r:], out)
         net.status()
+        assert (net.pair_launches()[0] > 0) == (rep > 0)
         outs.append(out)
         assert torch.equal(out, outs[0]), f"{push} rows a push, run {rep}: {int((out != outs[0]).sum())} of {out.numel()} differ"
     assert int(outs[0].ne(0).sum()) > outs[0].numel() // 4
