@@ -350,7 +350,8 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     if (threadIdx.x == 0) {
         s_abort = 0;
-        if (!IDF_OK_AT(a.status, sB + (uint32_t)(a.n_b * a.b_bytes) - smem_u32(smem_raw) - 1u, a.smem_bytes)) s_abort = 1;
+        if (!IDF_OK_AT(a.status, sB + (uint32_t)(a.n_b * a.b_bytes) - smem_u32(smem_raw) - 1u, a.smem_bytes) || !IDF_OK_AT(a.status, a.n_a - 1, PAIR_MAX_A) ||
+            !IDF_OK_AT(a.status, a.n_b - 1, PAIR_MAX_B) || !IDF_OK_AT(a.status, a.R - 1, PAIR_MAX_R)) s_abort = 1;
     }
     if (warp == 2) {
         // ("full" barriers are those of the pair's first CTA: its producer's arrival and the bytes of both; "empty" ones are each CTA's own)
@@ -361,7 +362,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(512u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"((uint32_t)PAIR_TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -399,6 +400,8 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const uint32_t fresh = kb != 0 ? 0u : (i == v.i_lo ? all : (i < v.nr ? 1u : 0u));           // the accumulator's first row
                         const uint32_t done = kb != a.n_kb - 1 ? 0u : (i == v.i_hi ? all : (i - a.Kh + 1 >= v.j_lo ? oldest : 0u));    // ... its last one
                         const bool end = !more && kb == a.n_kb - 1 && i == v.i_hi;
+                        if (!IDF_OK_AT(a.status, n - 1, PAIR_MAX_R) || !IDF_OK_AT(a.status, (j_hi - n + 1) * a.N, PAIR_TMEM) || !IDF_OK_AT(a.status, (j_hi + 1) * a.N - 1, PAIR_TMEM) ||
+                            !IDF_OK_AT(a.status, v.row0 + i - a.base_ty, a.n_in) || !IDF_OK_AT(a.status, stage, a.n_a)) { *abort_flag = 1; ok = false; break; }
                         if (!mbar_wait(a_empty + 8u * stage, ph, abort_flag)) { ok = false; break; }
                         if (rank == 0) {
                             s_sched[stage] = make_uint4((uint32_t)n | (uint32_t)j_hi << 8 | (end ? 1u << 16 : 0u), first | release << 16, fresh | done << 16,
@@ -428,6 +431,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         // the tap rows that input row i is the first to use, in the order the MMAs want them
                         for (int j = min(w.nr - 1, i); j >= max(w.j_lo, i - a.Kh + 1); --j) {
                             if (i != w.i_lo && j != w.j_lo) continue;
+                            if (!IDF_OK_AT(a.status, i - j, a.Kh) || !IDF_OK_AT(a.status, n0 + a.N / 2 - 1, a.Cout) || !IDF_OK_AT(a.status, stage, a.n_b)) { *abort_flag = 1; ok = false; break; }
                             if (!mbar_wait(b_empty + 8u * stage, ph, abort_flag)) { ok = false; break; }
                             if (rank == 0) mbar_expect_tx(b_full + 8u * stage, 2u * (uint32_t)a.Kw * half);
                             // (slot of a tap in the parameters: see tc_weight_slot, stride 1)
@@ -570,6 +574,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             p.valid = bs < a.BS && bx < a.BX && p.s < a.S && p.x < a.Wout;
             p.ring = ((long long)p.s * a.Wout + p.x) * a.Cout + p.n0;
             p.out = (long long)p.s * a.out_stream_stride + (long long)(POOL ? p.x >> 1 : p.x) * a.Cout + p.n0;
+            if (!IDF_OK_AT(a.status, w.nr * a.N - 1, PAIR_TMEM) || !IDF_OK_AT(a.status, w.nr - 1, a.R)) { *abort_flag = 1; break; }
             if (!POOL) {
                 for (int j = w.j_lo; j < w.nr; ++j) {
                     const bool has = w.has_taps(a, j);
@@ -610,7 +615,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)PAIR_TMEM) : "memory");
     }
 }
 

@@ -12,6 +12,7 @@
 namespace idf {
 
 constexpr int PAIR_MAX_A = 8, PAIR_MAX_B = 24, PAIR_MAX_R = 8;     // stages of input rows and of tap rows, rows of a work item
+constexpr int PAIR_TMEM = 512;                                     // columns of tensor memory
 constexpr int PAIR_MMA_WARPS = 2;                                  // issuing warps: each issues for every other accumulator
 constexpr int PAIR_CLUSTERS = 74;                                  // two SMs each
 constexpr double PAIR_ROW_CLK = 800, PAIR_ITEM_CLK = 600;          // cycles from one input row to the next with little to do in it, and between items
@@ -53,7 +54,7 @@ inline PairTiles pair_tiles(int S, int Wout, int Cout, int Kh, int Kw, int swb, 
     double best_t = 0;
     for (int N = 256; N >= 32; N /= 2) {
         if (Cout % N) continue;
-        for (int R = g.row_step; R <= PAIR_MAX_R && R * N <= 512; R += g.row_step) {
+        for (int R = g.row_step; R <= PAIR_MAX_R && R * N <= PAIR_TMEM; R += g.row_step) {
             PairTiles t = g;
             t.N = N; t.R = R;
             t.b_tile = ((size_t)(N / 2) * swb + 1023) / 1024 * 1024;

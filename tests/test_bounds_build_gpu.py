@@ -12,6 +12,7 @@ import torch
 from paper_1804_10727_b200 import idf
 from paper_1804_10727_b200.workloads import Layer, conv, POOL
 from helpers import SMALL_NETS, assert_close, assert_equal, rand_net, small_dims, with_path, with_shifts
+from test_cta_pairs_gpu import CASES as PAIR_CASES
 
 pytestmark = pytest.mark.gpu
 
@@ -73,6 +74,20 @@ def test_tensor_core_and_sparse_kernels_through_the_range_checked_build(orc, nam
         net = idf.Net(mode, layers, W, C0, S, ws, bs, row_block=rb)
         got = idf.infer(net, x, chunks=chunks, last=last)
         _check(mode, got, want, f"{name}/chunks={chunks}/rb={rb}")
+        net.close()
+
+
+@pytest.mark.parametrize("name,mode,layers,H,W,S", PAIR_CASES, ids=[c[0] for c in PAIR_CASES])
+def test_cta_pairs_through_the_range_checked_build(orc, debug_flags, name, mode, layers, H, W, S):
+    layers = with_shifts(layers, 11) if mode == "i8" else layers
+    x, ws, bs = rand_net(mode, layers, H, W, layers[0].cin, S=S, seed=len(name))
+    want = orc.forward(mode, layers, x, ws, bs)
+    debug_flags(idf.DEBUG_FORCE_CTA_PAIRS)
+    for chunks, rb, last in ((None, 0, True), ([1] * H, 0, False), ([3, 2, 5, 1], 3, True), ([H // 2 + 1], 64, False)):
+        net = idf.Net(mode, layers, W, layers[0].cin, S, ws, bs, row_block=rb)
+        got = idf.infer(net, x, chunks=chunks, last=last)
+        assert net.pair_launches()[0] == net.status()[0] > 0
+        (assert_equal if mode == "i8" else assert_close)(got, want, f"{name}/chunks={chunks}/rb={rb}")
         net.close()
 
 
