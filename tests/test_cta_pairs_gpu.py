@@ -9,6 +9,7 @@ import torch
 from paper_1804_10727_b200 import idf
 from paper_1804_10727_b200.workloads import Layer, conv, POOL
 from helpers import assert_close, assert_equal, rand_net, with_shifts
+from test_full_size_gpu import _bf16_down_up
 
 pytestmark = pytest.mark.gpu
 
@@ -116,3 +117,32 @@ def test_pool_rows_taken_and_parked_in_one_launch(debug_flags, push):
         assert torch.equal(out, outs[0]), f"{push} rows a push, run {rep}: {int((out != outs[0]).sum())} of {out.numel()} differ"
     assert int(outs[0].ne(0).sum()) > outs[0].numel() // 4
     net.close()
+
+
+def test_hidden_rows_match_oracle(orc, debug_flags):
+    """Rows between layers, emitted and pooled by pairs, against the oracle: int8 nets exactly; a bf16 layer's rounded rows, passed on by a 1x1
+    identity layer, are the rounding of some value within the strict tolerance of the oracle's unrounded one."""
+    debug_flags(idf.DEBUG_FORCE_CTA_PAIRS)
+    layers = with_shifts((conv(128, 128, 3, pad=1), POOL, conv(128, 256, 3, pad=1), conv(256, 64, 3, pad=1), POOL), 11)
+    x, ws, bs = rand_net("i8", layers, 24, 40, 128, S=6, seed=3)
+    want = orc.forward("i8", layers, x, ws, bs)
+    net = idf.Net("i8", layers, 40, 128, 6, ws, bs)
+    for chunks in (None, [1] * 24, [7, 2, 9]):
+        assert_equal(idf.infer(net, x, chunks=chunks, last=True), want, f"i8/{chunks and len(chunks)}")
+        assert all(net.pair_launches()[i] > 0 for i in (0, 2, 3))
+    net.close()
+    for layer, pool in ((conv(64, 128, 3, pad=1), False), (conv(128, 128, 3, pad=1, relu=0), True), (conv(128, 64, 5), True)):
+        layers = (layer,) + ((POOL,) if pool else ()) + (conv(layer.cout, layer.cout, 1, relu=0),)
+        x, ws, bs = rand_net("bf16", layers, 17, 34, layer.cin, S=5, seed=layer.cin + layer.cout)
+        ws[-1], bs[-1] = np.eye(layer.cout, dtype=np.float32).reshape(layer.cout, 1, 1, layer.cout), None
+        want = orc.conv_layer("bf16", layer, x, ws[0], bs[0])
+        want = orc.pool_layer("bf16", want) if pool else want
+        tol = 1e-4 + 1e-3 * np.abs(want)
+        lo, hi = _bf16_down_up(want - tol)[0], _bf16_down_up(want + tol)[1]
+        net = idf.Net("bf16", layers, 34, layer.cin, 5, ws, bs)
+        for chunks in (None, [1] * 17, [7, 2, 3]):
+            got = idf.infer(net, x, chunks=chunks, last=True).astype(np.float64)
+            assert net.pair_launches()[0] > 0 and got.shape == want.shape
+            bad = (got < lo) | (got > hi)
+            assert not bad.any(), (layer, pool, chunks, int(bad.sum()), bad.size)
+        net.close()

@@ -28,12 +28,17 @@ CASES = [
     ("time_1d", conv(32, 32, 9, one_d=True, relu=0), 120, 1, 20),            # shifted views of whole rows: no zero weights
     ("time_1d_stride2_pad", conv(64, 32, 9, stride=2, pad=4, one_d=True, relu=0), 120, 1, 20),
     ("window_1d_pad", conv(2, 48, 5, pad=2, one_d=True, relu=0), 50, 1, 3),
+    ("pairs_128ch", conv(64, 128, 3, pad=1, relu=0), 11, 22, 7),             # several streams to a tile, halos between them
+    ("pairs_two_k_blocks_5x5", conv(128, 64, 5, pad=4, relu=0), 10, 37, 3),
+    ("pairs_two_tiles_a_row", conv(64, 64, 3, relu=0), 9, 133, 2),
 ]
 
 
 @pytest.mark.parametrize("name,layer,H,W,S", CASES, ids=[c[0] for c in CASES])
-def test_nonfinite_input_stays_in_its_receptive_field(orc, name, layer, H, W, S):
+def test_nonfinite_input_stays_in_its_receptive_field(orc, debug_flags, name, layer, H, W, S):
     layers = (layer,)
+    pairs = name.startswith("pairs")
+    debug_flags(idf.DEBUG_FORCE_CTA_PAIRS if pairs else 0)
     for k, value in enumerate((np.inf, -np.inf, np.nan)):
         x, ws, bs = rand_net("bf16", layers, H, W, layer.cin, S=S, seed=k)
         r = np.random.default_rng(k)
@@ -48,7 +53,7 @@ def test_nonfinite_input_stays_in_its_receptive_field(orc, name, layer, H, W, S)
         for chunks in (None, [1] * H, [4, 2, H]):
             net = idf.Net("bf16", layers, W, layer.cin, S, ws, bs)
             whole = idf.infer(net, x, chunks=chunks, last=True)
-            assert net.status()[0] > 0
+            assert net.status()[0] > 0 and (not pairs or net.pair_launches()[0] > 0)
             got = whole[pick]
             assert np.isfinite(np.delete(whole, pick, 0)).all()
             what = f"{name}/{value}/{chunks and len(chunks)}"

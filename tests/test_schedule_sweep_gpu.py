@@ -3,7 +3,7 @@
 The result must not depend on how segments are grouped into pushes (the paper's output is defined by
 the whole input, Eq. 1).  Each kernel that exchanges rows with state in global memory - the CUDA-core
 conv (ring), the sparse conv (ring), the stand-alone max-pool (one state row), the tensor-core conv
-with and without row chunks (ring), its folded max-pool (pool state row) and the averaging sink (sums) -
+with and without row chunks (ring), its folded max-pool (pool state row), both on CTA pairs, and the averaging sink (sums) -
 is driven through every combination of
     first row of the launch even/odd  x  last row even/odd  x  1, 2 or many rows per launch
     x  rows begun by an earlier launch or not  x  rows left open for a later launch or not,
@@ -68,11 +68,33 @@ SWEEP_NETS = [
     ("avg_sink_i8", "i8", (conv(2, 8, 3), AVG), 20, 9, 3, 2),
 ]
 
+# nets whose wide layers the CTA-pair kernel takes: by the library's rule on blocks of eight rows and more, and every launch where it is forced
+PAIR_NETS = [
+    ("pairs_conv_pool_i8", "i8", (conv(128, 128, 3, pad=1), POOL, conv(128, 128, 3)), 26, 24, 3, 128),
+    ("pairs_valid_pool_k2_i8", "i8", (conv(128, 128, 2), POOL, conv(128, 64, 3, pad=1), POOL), 27, 21, 3, 128),
+    ("pairs_two_k_blocks_k5_i8", "i8", (conv(256, 128, 5, pad=2), POOL), 25, 18, 3, 256),
+    ("pairs_one_stream_odd_width_i8", "i8", (conv(128, 128, 3), POOL, conv(128, 128, 1)), 24, 133, 1, 128),
+    ("pairs_conv_pool_bf16", "bf16", (conv(64, 128, 3, pad=1), POOL), 23, 31, 3, 64),
+]
+
+
+def _shift(C0):
+    return 7 if C0 < 64 else 11                # (few outputs at the limits of int8)
+
+
+@pytest.mark.parametrize("name,mode,layers,H,W,S,C0", PAIR_NETS, ids=[c[0] for c in PAIR_NETS])
+@pytest.mark.parametrize("forced", [False, True], ids=["by_rule", "forced"])
+def test_every_grouping_of_rows_on_cta_pairs(orc, debug_flags, forced, name, mode, layers, H, W, S, C0):
+    debug_flags(idf.DEBUG_FORCE_CTA_PAIRS if forced else 0)
+    test_every_grouping_of_rows_gives_the_oracle_result(orc, name, mode, layers, H, W, S, C0)
+    if mode == "i8":
+        test_integer_results_are_bit_identical_run_after_run(name, mode, layers, H, W, S, C0)
+
 
 @pytest.mark.parametrize("name,mode,layers,H,W,S,C0", SWEEP_NETS, ids=[c[0] for c in SWEEP_NETS])
 def test_every_grouping_of_rows_gives_the_oracle_result(orc, name, mode, layers, H, W, S, C0):
     if mode == "i8":
-        layers = with_shifts(layers, 7)
+        layers = with_shifts(layers, _shift(C0))
     x, ws, bs = rand_net(mode, layers, H, W, C0, S=S, seed=41 + len(name))
     want = orc.forward(mode, layers, x, ws, bs)
     seg = idf.segments_from_maps(x, mode).cuda()
@@ -80,11 +102,13 @@ def test_every_grouping_of_rows_gives_the_oracle_result(orc, name, mode, layers,
         net = idf.Net(mode, layers, W, C0, S, ws, bs, row_block=rb)
         out = net.alloc_out(H)
         net.open()
+        pairs = 0
         for sizes in SIZE_PATTERNS:
             for last in (False, True):
                 out.zero_()
                 rows = _pushes(net, seg, out, _groups(H, sizes), last)
                 net.status()
+                pairs += sum(net.pair_launches())
                 got = out[:, :rows].cpu().numpy()
                 what = f"{name}/rb={rb}/sizes={sizes}/last={last}"
                 if mode == "i8" and layers[-1].kind != "avg":
@@ -93,13 +117,14 @@ def test_every_grouping_of_rows_gives_the_oracle_result(orc, name, mode, layers,
                     assert np.array_equal(got, want.astype(np.float32)), what
                 else:
                     assert_close(got, want, what)
+        assert not name.startswith("pairs") or rb or pairs > 0
         net.close()
 
 
 @pytest.mark.parametrize("name,mode,layers,H,W,S,C0", [c for c in SWEEP_NETS if c[1] == "i8"],
                          ids=[c[0] for c in SWEEP_NETS if c[1] == "i8"])
 def test_integer_results_are_bit_identical_run_after_run(name, mode, layers, H, W, S, C0):
-    layers = with_shifts(layers, 7)
+    layers = with_shifts(layers, _shift(C0))
     x, ws, bs = rand_net(mode, layers, H, W, C0, S=S, seed=41 + len(name))
     seg = idf.segments_from_maps(x, mode).cuda()
     net = idf.Net(mode, layers, W, C0, S, ws, bs, row_block=3)
