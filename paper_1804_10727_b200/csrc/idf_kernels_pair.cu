@@ -421,7 +421,9 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (lane == 0) {
             const uint32_t full0 = map_to_rank(b_full, 0);
             const uint32_t half = (uint32_t)(a.N / 2) * a.swb;
-            int stage = 0;
+            // Ahead of the dependency wait only stages that nobody has used are filled: a wait for a used one is bounded, and it would last as
+            // long as the kernel in front of this one does.
+            int stage = 0, unused = a.n_b;
             uint32_t ph = 1;
             bool ok = true;
             for (bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1); more && ok; more = w.next(a)) {
@@ -432,6 +434,7 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         for (int j = min(w.nr - 1, i); j >= max(w.j_lo, i - a.Kh + 1); --j) {
                             if (i != w.i_lo && j != w.j_lo) continue;
                             if (!IDF_OK_AT(a.status, i - j, a.Kh) || !IDF_OK_AT(a.status, n0 + a.N / 2 - 1, a.Cout) || !IDF_OK_AT(a.status, stage, a.n_b)) { *abort_flag = 1; ok = false; break; }
+                            if (unused-- == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
                             if (!mbar_wait(b_empty + 8u * stage, ph, abort_flag)) { ok = false; break; }
                             if (rank == 0) mbar_expect_tx(b_full + 8u * stage, 2u * (uint32_t)a.Kw * half);
                             // (slot of a tap in the parameters: see tc_weight_slot, stride 1)
@@ -440,8 +443,8 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             if (++stage == a.n_b) { stage = 0; ph ^= 1u; }
                         }
             }
-            if (ok) pair_drain(stage, ph, a.n_b, [&](int s, uint32_t parity) { return mbar_wait(b_empty + 8u * s, parity, abort_flag); });
             asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (ok) pair_drain(stage, ph, a.n_b, [&](int s, uint32_t parity) { return mbar_wait(b_empty + 8u * s, parity, abort_flag); });
         }
         __syncwarp();
     } else if (warp < PAIR_W_WARP) {

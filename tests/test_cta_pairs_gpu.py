@@ -146,3 +146,14 @@ def test_hidden_rows_match_oracle(orc, debug_flags):
             bad = (got < lo) | (got > hi)
             assert not bad.any(), (layer, pool, chunks, int(bad.sum()), bad.size)
         net.close()
+
+
+def test_slow_kernel_in_front(orc):
+    """A layer whose events are scattered one by one takes long over an input without zeros; the launch that depends on it starts early and must
+    not give up meanwhile."""
+    layers = with_shifts((Layer("conv", 128, 256, 4, 4, 1, 0, 1, 0, idf.PATH_SPARSE), conv(256, 128, 3, pad=1)), 11)
+    x, ws, bs = rand_net("i8", layers, 20, 68, 128, S=1, seed=9, zero_frac=0.0)
+    net = idf.Net("i8", layers, 68, 128, 1, ws, bs, row_block=16)
+    assert_equal(idf.infer(net, x, last=True), orc.forward("i8", layers, x, ws, bs), "slow first layer")
+    assert net.pair_launches()[1] > 0
+    net.close()
