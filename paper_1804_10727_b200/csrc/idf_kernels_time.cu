@@ -115,6 +115,9 @@ conv_time_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int it = first; it < a.n_items && ok; it += step) {
                 for (int kb = 0; kb < a.n_kb && ok; ++kb)
                     for (int ky = 0; ky < a.Kh; ++ky, ++t) {
+                        // (ahead of the dependency wait only stages that nobody has used are filled: the wait for a used one is bounded, and it
+                        // would last as long as the kernel in front of this one does)
+                        if (t == a.n_w) asm volatile("griddepcontrol.wait;" ::: "memory");
                         if (!mbar_wait(bar_we + 8u * stage, ph, abort_flag)) { ok = false; break; }
                         mbar_expect_tx(bar_w + 8u * stage, (uint32_t)a.N * a.swb);
                         // (slot of tap ky in the parameters: see tc_weight_slot)

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_1804_10727_b200 import idf
-from paper_1804_10727_b200.workloads import conv
+from paper_1804_10727_b200.workloads import Layer, conv
 from helpers import assert_close, assert_equal, rand_net, with_shifts
 
 pytestmark = pytest.mark.gpu
@@ -52,3 +52,14 @@ def test_time_tiles_match_oracle(orc, debug_flags, name, mode, layer, H, S):
         net = idf.Net(mode, layers, 1, layer.cin, S, ws, bs)
         assert_equal(idf.infer(net, x, chunks=[40, 3], last=True), want, name + "/row ring")
         net.close()
+
+
+def test_slow_kernel_in_front(orc):
+    """A layer whose events are scattered one by one takes long over an input without zeros (0.7 s here); the launch that depends on it starts
+    early and must not give up meanwhile, though its weight tiles do not all fit."""
+    layers = with_shifts((Layer("conv", 512, 512, 9, 1, 1, 0, 1, 0, idf.PATH_SPARSE), conv(512, 256, 9, one_d=True)), 12)
+    x, ws, bs = rand_net("i8", layers, 190, 1, 512, S=1, seed=9, zero_frac=0.0)
+    net = idf.Net("i8", layers, 1, 512, 1, ws, bs, row_block=256)
+    assert_equal(idf.infer(net, x, last=True), orc.forward("i8", layers, x, ws, bs), "slow first layer")
+    assert net.status()[1] > 0
+    net.close()
