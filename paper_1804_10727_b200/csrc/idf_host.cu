@@ -159,18 +159,24 @@ void as_planned(const LayerPlan& P, ConvArgs* t)
 }
 
 // Whether a launch is one for the CTA-pair kernel; `ring`: the row-ring kernel's plan for it.
-// Measured on 650 random layers against that kernel (mean time ring / pairs): 2D layers of a multiple of 128 output channels, all rows in one
-// launch 1.5 (the worst 0.91), 8 to 12 rows at a time 1.25, 6 or 7 with four K blocks and more 1.05 to 1.7 (256 -> 256, 5 streams of 39 x 32
-// in sevens: 109 -> 95 us).  A launch of fewer rows mostly waits for the rows it exchanges with the ring, 0.8 to 0.9 - unless the row-ring
-// kernel takes it in two turns of the SMs (256 -> 256, 64 x 56, one row: 1.10; 30 such layers 1.2, 0.96 to 2.4).  Of a multiple of 64
-// channels, two K blocks and more 1.5; with one K block 1.3, but 0.54 where the launch is large (int8 64 -> 64, 2048 streams: MMAs of 64
-// columns wait for operands); of other channel counts 1.2 with some at 0.5.
+// Measured on random layers against that kernel (mean time ring / pairs; 4700 layers of 64 to 512 channels, 6 to 112 rows a launch): 2D layers of a
+// multiple of 128 output channels 1.1 to 1.2 at 8 to 12 rows with one K block, 1.2 with two, 1.3 to 2.3 with four and more, growing to 1.3 to 3
+// at 72 rows and more; six or seven rows only with four K blocks and more (1.1 to 2.2).
+// Where the row-ring kernel takes the launch in one turn of the SMs that it fills by two thirds (its light build: two CTAs to an SM), the pairs
+// catch up later: one K block 0.92 to 0.97 below 12 rows (down to 0.7), 0.94 to 1.01 below 16, 1.04 to 1.08 below 24; two K blocks 0.97 to 0.99
+// below 12, 1.11 below 16 (64 -> 128, 69 streams of 113-wide rows, ten at a time: 21 us a launch on the ring, 28 on pairs).
+// A launch of fewer rows mostly waits for the rows it exchanges with the ring, 0.8 to 0.9 - unless the row-ring kernel takes it in two turns of the
+// SMs (256 -> 256, 64 x 56, one row: 1.10; 30 such layers 1.2, 0.96 to 2.4).  Of a multiple of 64 channels, two K blocks and more 1.5; with one
+// K block 1.3, but 0.54 where the launch is large (int8 64 -> 64, 2048 streams: MMAs of 64 columns wait for operands); of other channel
+// counts 1.2 with some at 0.5.
 bool by_pairs(const LayerPlan& P, const TcPlan& ring, const ConvArgs& a)
 {
     if (!P.pair.ok || a.r1 <= a.r0 || (debug_flags() & IDF_DEBUG_NO_CTA_PAIRS)) return false;
     if (debug_flags() & IDF_DEBUG_FORCE_CTA_PAIRS) return true;
-    const long long rows = a.r1 - a.r0;
-    if (rows < 8 && !(rows >= 6 && P.pair.n_kb >= 4)) return a.Cout % 128 == 0 && !ring.light && (long long)ring.n_mt * ring.n_nt > 148;
+    const long long rows = a.r1 - a.r0, ctas = (long long)ring.n_mt * ring.n_nt, turn = ring.light ? 2 * 148 : 148;
+    const bool full_turn = ctas <= turn && 3 * ctas > 2 * turn;
+    const int least = P.pair.n_kb >= 4 ? 6 : !full_turn || P.pair.n_kb == 3 ? 8 : P.pair.n_kb == 2 ? 12 : 16;
+    if (rows < least) return a.Cout % 128 == 0 && !ring.light && ctas > 148;
     return a.Cout % 128 == 0 || (a.Cout % 64 == 0 && P.pair.n_kb >= 2);
 }
 

@@ -71,6 +71,18 @@ def test_rows_one_by_one(orc, S):
     net.close()
 
 
+@pytest.mark.parametrize("cin,S,chunks", [(64, 296, (15, 16)), (64, 192, (7, 8)), (128, 140, (11, 12))])    # 148, 96 and 140 tiles: full turns and not
+def test_rows_in_one_turn(orc, cin, S, chunks):
+    """The rule where the row-ring kernel takes a launch in one turn of the SMs, on both sides of its line."""
+    layers = (conv(cin, 128, 3, pad=1),)
+    x, ws, bs = rand_net("bf16", layers, sum(chunks), 30, cin, S=S, seed=S)
+    pick = np.r_[0:3, S - 1]
+    net = idf.Net("bf16", layers, 30, cin, S, ws, bs)
+    assert_close(idf.infer(net, x, chunks=chunks, last=True)[pick], orc.forward("bf16", layers, x[pick], ws, bs), f"{cin}/{S}")
+    assert net.pair_launches() == [1] and net.status() == [2]
+    net.close()
+
+
 def test_hidden_rows(orc, debug_flags):
     """bf16 rows between layers, emitted and pooled by pairs: against the row-ring kernels, off by one rounding (2^-8 of the value; the
     sums of the next layer average that out, so twice it over the largest output bounds them)."""
@@ -104,7 +116,7 @@ def test_pool_rows_taken_and_parked_in_one_launch(debug_flags, push):
     net.open()
     outs = []
     for rep in range(11):
-        debug_flags(idf.DEBUG_NO_CTA_PAIRS if rep == 0 else 0)
+        debug_flags(idf.DEBUG_NO_CTA_PAIRS if rep == 0 else idf.DEBUG_FORCE_CTA_PAIRS if push < 16 else 0)
         out = net.alloc_out(H)
         net.reset()
         for r in range(0, H - push, push):
