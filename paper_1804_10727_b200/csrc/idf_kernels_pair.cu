@@ -421,9 +421,9 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (lane == 0) {
             const uint32_t full0 = map_to_rank(b_full, 0);
             const uint32_t half = (uint32_t)(a.N / 2) * a.swb;
-            // Ahead of the dependency wait only stages that nobody has used are filled: a wait for a used one is bounded, and it would last as
+            // A stage that is not free at once is waited for behind the dependency wait: the wait is bounded, and before that it would last as
             // long as the kernel in front of this one does.
-            int stage = 0, unused = a.n_b;
+            int stage = 0;
             uint32_t ph = 1;
             bool ok = true;
             for (bool more = w.start(a, blockIdx.x >> 1, gridDim.x >> 1); more && ok; more = w.next(a)) {
@@ -434,8 +434,10 @@ conv_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         for (int j = min(w.nr - 1, i); j >= max(w.j_lo, i - a.Kh + 1); --j) {
                             if (i != w.i_lo && j != w.j_lo) continue;
                             if (!IDF_OK_AT(a.status, i - j, a.Kh) || !IDF_OK_AT(a.status, n0 + a.N / 2 - 1, a.Cout) || !IDF_OK_AT(a.status, stage, a.n_b)) { *abort_flag = 1; ok = false; break; }
-                            if (unused-- == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-                            if (!mbar_wait(b_empty + 8u * stage, ph, abort_flag)) { ok = false; break; }
+                            if (!mbar_test(b_empty + 8u * stage, ph)) {
+                                asm volatile("griddepcontrol.wait;" ::: "memory");
+                                if (!mbar_wait(b_empty + 8u * stage, ph, abort_flag)) { ok = false; break; }
+                            }
                             if (rank == 0) mbar_expect_tx(b_full + 8u * stage, 2u * (uint32_t)a.Kw * half);
                             // (slot of a tap in the parameters: see tc_weight_slot, stride 1)
                             for (int kx = 0; kx < a.Kw; ++kx)
