@@ -166,7 +166,7 @@ void as_planned(const LayerPlan& P, ConvArgs* t)
 // catch up later: one K block 0.92 to 0.97 below 12 rows (down to 0.7), 0.94 to 1.01 below 16, 1.04 to 1.08 below 24; two K blocks 0.97 to 0.99
 // below 12, 1.11 below 16 (64 -> 128, 69 streams of 113-wide rows, ten at a time: 21 us a launch on the ring, 28 on pairs).
 // A launch of fewer rows mostly waits for the rows it exchanges with the ring, 0.8 to 0.9 - unless the row-ring kernel takes it in two turns of the
-// SMs (256 -> 256, 64 x 56, one row: 1.10; 30 such layers 1.2, 0.96 to 2.4).  Of a multiple of 64 channels, two K blocks and more 1.5; with one
+// SMs and more (400 such layers of one to seven rows: 1.02 to 1.2 in two turns, the worst 0.90, 1.3 to 2.9 from 600 CTAs on).  Of a multiple of 64 channels, two K blocks and more 1.5; with one
 // K block 1.3, but 0.54 where the launch is large (int8 64 -> 64, 2048 streams: MMAs of 64 columns wait for operands); of other channel
 // counts 1.2 with some at 0.5.
 bool by_pairs(const LayerPlan& P, const TcPlan& ring, const ConvArgs& a)

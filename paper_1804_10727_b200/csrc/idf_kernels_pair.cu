@@ -121,31 +121,12 @@ __device__ __forceinline__ void pair_mma(uint32_t tmem_d, uint32_t alo, uint32_t
                      ::"r"(tmem_d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(fresh) : "memory");
 }
 
-// W sums of one position -> the words of W emitted values; returns their number
+// W sums of one position -> the words of W emitted values
 template <int DT, int W>
 __device__ __forceinline__ void pack_out(const uint32_t* v, const uint32_t* bias, int bf16, int relu, int shift, uint32_t* pk)
 {
-    if (DT == 2) { pack_i8<W>(v, (const int*)bias, relu, shift, pk); return; }
-    float f[W];
-#pragma unroll
-    for (int j = 0; j < W; ++j) f[j] = __uint_as_float(v[j]);
-    if (bias) {
-#pragma unroll
-        for (int j4 = 0; j4 < W / 4; ++j4) {
-            const float4 b4 = ((const float4*)bias)[j4];
-            f[4 * j4] += b4.x; f[4 * j4 + 1] += b4.y; f[4 * j4 + 2] += b4.z; f[4 * j4 + 3] += b4.w;
-        }
-    }
-    if (bf16) {
-#pragma unroll
-        for (int j = 0; j < W / 2; ++j) {
-            if (relu) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
-            else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < W; ++j) pk[j] = __float_as_uint(relu ? fmaxf(f[j], 0.f) : f[j]);
-    }
+    if (DT == 2) pack_i8<W>(v, (const int*)bias, relu, shift, pk);
+    else pack_f<W>(v, (const float*)bias, bf16, relu, pk);
 }
 
 template <int W>
@@ -160,7 +141,7 @@ __device__ __forceinline__ void ring_add(uint32_t* v, const uint32_t* r)
 #pragma unroll
     for (int j = 0; j < W; ++j) v[j] = DT == 1 ? __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(r[j])) : v[j] + r[j];
 }
-// n (4, 8 or 16) words to an address of that alignment, at most 32 bytes at a time
+// NW words: 4 to an address of 16-byte alignment, 8, 16 or 32 to one of 32 bytes (wide) or 16, 32 bytes at a time
 template <int NW>
 __device__ __forceinline__ void store_words(unsigned char* p, const uint32_t* v, int wide)
 {
@@ -179,8 +160,7 @@ __device__ __forceinline__ long long ring_row(const PairArgs& a, int row)
 {
     return (long long)((a.ring_slot0 + row) % a.ring_rows) * a.S * a.Wout * a.Cout;
 }
-// 16 columns from column c on of a row that exchanges state with the ring: what an earlier block left (fetched before) is added; true: the
-// row is complete and its sums are to be emitted, else they are parked.
+// 16 columns from column c on of what an earlier block left of a row; false: nothing
 __device__ __forceinline__ bool ring_fetch(const PairArgs& a, const PairSpot& p, int row, int c, uint32_t* r)
 {
     const long long at = ring_row(a, row) + p.ring + c;
@@ -188,6 +168,7 @@ __device__ __forceinline__ bool ring_fetch(const PairArgs& a, const PairSpot& p,
     if (have) ring_load<16>((const uint32_t*)a.ring_in + at, r);
     return have;
 }
+// ... is added; true: the row is complete and its sums are to be emitted, else they are parked
 template <int DT>
 __device__ __forceinline__ bool ring_exchange(const PairArgs& a, const PairSpot& p, int row, int c, uint32_t* v, bool have, const uint32_t* r)
 {
@@ -632,6 +613,7 @@ bool pair_make_plan(int dtype, int Win, int Cin, int Cout, int Kh, int Kw, int s
     if (dtype != 1 && dtype != 2) return false;
     const int es = dtype == 1 ? 2 : 1, row = Cin * es;
     if (Win == 1 || stride != 1 || Kh * Kw == 1 || Kh * Kw > 256) return false;
+    // (fewer than 64 channels to a slice: only where the launches are forced here, which the library's rule never does)
     if (!(row == 64 || (row >= 128 && row % 128 == 0)) || Cout % 32 != 0) return false;
     p->swb = row >= 128 ? 128 : row;
     p->KB = p->swb / es;

@@ -308,39 +308,41 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t* v, int wid
     else { st_global_v4(p, v); st_global_v4((unsigned char*)p + 16, v + 4); }
 }
 
-// f(c + b) of 16 fp32 sums as bf16 or fp32, straight to global memory (wide: dst is 32-byte aligned)
-template <int OUT>
-__device__ __forceinline__ void emit16f(const uint32_t* v, const float* bias_c, int relu, unsigned char* dst, int wide)
+// f(c + b) of W fp32 sums: W / 2 words of bf16 pairs, or W of fp32
+template <int W>
+__device__ __forceinline__ void pack_f(const uint32_t* v, const float* bias_c, int bf16, int relu, uint32_t* pk)
 {
-    float f[16];
+    float f[W];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+    for (int j = 0; j < W; ++j) f[j] = __uint_as_float(v[j]);
     if (bias_c) {
 #pragma unroll
-        for (int j4 = 0; j4 < 4; ++j4) {
+        for (int j4 = 0; j4 < W / 4; ++j4) {
             const float4 b4 = ((const float4*)bias_c)[j4];
             f[4 * j4] += b4.x; f[4 * j4 + 1] += b4.y; f[4 * j4 + 2] += b4.z; f[4 * j4 + 3] += b4.w;
         }
     }
-    if (OUT == E_BF16) {
-        uint32_t pk[8];
+    if (bf16) {
         if (relu) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
+            for (int j = 0; j < W / 2; ++j) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
         } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
+            for (int j = 0; j < W / 2; ++j) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pk[j]) : "f"(f[2 * j + 1]), "f"(f[2 * j]));
         }
-        st_global_32(dst, pk, wide);
     } else {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t w[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) w[j] = __float_as_uint(relu ? fmaxf(f[8 * h + j], 0.f) : f[8 * h + j]);
-            st_global_32(dst + 32 * h, w, wide);
-        }
+        for (int j = 0; j < W; ++j) pk[j] = __float_as_uint(relu ? fmaxf(f[j], 0.f) : f[j]);
     }
+}
+// ... of 16, straight to global memory (wide: dst is 32-byte aligned)
+template <int OUT>
+__device__ __forceinline__ void emit16f(const uint32_t* v, const float* bias_c, int relu, unsigned char* dst, int wide)
+{
+    uint32_t pk[16];
+    pack_f<16>(v, bias_c, OUT == E_BF16, relu, pk);
+    st_global_32(dst, pk, wide);
+    if (OUT != E_BF16) st_global_32(dst + 32, pk + 8, wide);
 }
 // element-wise maximum of two 32-bit words holding OP = 0: two bf16, 1: one fp32, 2: four int8
 template <int OP>
